@@ -401,6 +401,7 @@ ptca_status ptca_init(const ptca_lattice* lattice, const ptca_params* params, pt
     }
     cudaError_t ce = ptca::configure_cluster_kernels((size_t)optin);
     if (ce == cudaSuccess && c->large) ce = ptca::configure_large_kernels((size_t)optin);
+    if (ce == cudaSuccess) ce = ptca::configure_resolvent_kernels((size_t)optin);
     if (ce != cudaSuccess) {
         delete c;
         return cuda_fail(ce, "ptca_init (configuring kernel shared memory)");
@@ -634,9 +635,24 @@ static StageArgs base_args(ptca_ctx* ctx) {
 cudaError_t ptca_screen_stage(ptca_ctx* ctx, ptca::StageArgs& a, cudaStream_t st);
 cudaError_t ptca_screen_part(ptca_ctx* ctx, ptca::StageArgs& a, int part, int row_base, int half, cudaStream_t st);
 
+// Whether the context's sweeps take their free energies from determinants
+// (resolvent.cuh): the default reduction of a PTCA_MIXED context (rows up to the
+// shared-memory orders, shared above) with windows of up to 16 sites per
+// layer and T not below 1/4096 of the spectrum's half width.  The reductions
+// that a launch configuration names explicitly keep their own kernels.
+static bool on_determinants(const ptca_ctx* ctx) {
+    if (ctx->prec != 1 || ctx->panel > 1 || ctx->reduction != (ctx->large ? 2 : 0)) return false;
+    return ptca::resolvent_supported(to_model(ctx->p));
+}
+
+// Stages of at most this many visits run the latency-bound form: a group of
+// threads per node instead of one warp.
+static bool few_visits(const ptca_ctx* ctx) { return ctx->max_stage <= 128; }
+
 // A stage launch and a re-solve launch in the context's configuration
 // (shared-memory kernels, or the large-cluster kernels).
 static cudaError_t launch_stage_ctx(const ptca_ctx* ctx, const StageArgs& a, cudaStream_t st) {
+    if (on_determinants(ctx)) return ptca::launch_stage_resolvent(a, few_visits(ctx), ctx->sms, st);
     if (ctx->large && ctx->reduction == 2) return ptca::launch_stage_large_shared(a, ctx->large_grid, st);
     if (ctx->large && ctx->prec == 1 && ctx->nw == 8 && ctx->cl_size > 0)
         return ptca::launch_stage_cluster(ctx->cl_size, a, ctx->cl_grid, st);
@@ -647,6 +663,7 @@ static cudaError_t launch_stage_ctx(const ptca_ctx* ctx, const StageArgs& a, cud
     return ptca::launch_stage(ctx->prec, ctx->nw, a, st);
 }
 static cudaError_t launch_resolve_ctx(const ptca_ctx* ctx, const StageArgs& a, cudaStream_t st) {
+    if (on_determinants(ctx)) return ptca::launch_resolve_resolvent(a, ctx->sms, st);
     if (ctx->large) return ptca::launch_resolve_large(a, ctx->resolve_grid, st);
     return ptca::launch_resolve(a, ctx->resolve_grid, st);
 }
@@ -677,6 +694,8 @@ static cudaError_t check_stage(ptca_ctx* ctx, const StageArgs& a, int s, cudaStr
             e = ptca::launch_check(1, a, c0, cnt, e32, ld, F32, 0, st);
             if (e == cudaSuccess) e = ptca::launch_check(0, a, c0, cnt, e64, ld, F64, ctx->resolve_grid, st);
         }
+        // the free energies that the sweep decides on
+        if (e == cudaSuccess && on_determinants(ctx)) e = ptca::launch_check_resolvent(a, few_visits(ctx), c0, cnt, F32, st);
         if (e == cudaSuccess)
             e = ptca::launch_check_compare(a.m, a.sites + c0, cnt, e32, e64, ld, F32, F64, ctx->d_chk_out + ptca::kCheckCols * s, st);
     }
@@ -685,13 +704,18 @@ static cudaError_t check_stage(ptca_ctx* ctx, const StageArgs& a, int s, cudaStr
 
 // One launch per stage (Sec. III.a stage = one kernel); with the surrogate
 // enabled each stage is screened first and only passing sites are solved.
-static cudaError_t sweep_stages(ptca_ctx* ctx, int32_t n_sweeps, cudaStream_t st, const Collect* col = nullptr) {
+// captured: the launches go into a graph that is replayed for later sweeps, so
+// the sweep index comes from the device counter; they are not timed one by one.
+static cudaError_t sweep_stages(ptca_ctx* ctx, int32_t n_sweeps, cudaStream_t st, const Collect* col = nullptr,
+                                bool captured = false) {
     StageArgs a = base_args(ctx);
+    if (captured) a.sweep_dev = ctx->d_sweep_ctr;
     int64_t g = 0;
     int prev_s = -1;
     cudaError_t e = cudaSuccess;
+    auto launched = [&](int kind, int64_t items, auto f) { return captured ? f() : timed_launch(ctx, kind, items, st, f); };
     for (int sw = 0; sw < n_sweeps && e == cudaSuccess; ++sw) {
-        a.sweep = (uint64_t)(ctx->sweeps + sw);
+        a.sweep = (uint64_t)(captured ? sw : ctx->sweeps + sw);
         if (col) {
             a.sg_feat = col->feat + (size_t)sw * ctx->N * ptca::SG_IN;
             a.sg_center = col->center + (size_t)sw * ctx->N;
@@ -711,10 +735,9 @@ static cudaError_t sweep_stages(ptca_ctx* ctx, int32_t n_sweeps, cudaStream_t st
             if (ctx->checker) e = check_stage(ctx, a, s, st);
             if (e == cudaSuccess && ctx->sg.enabled && !col) e = ptca_screen_stage(ctx, a, st);
             if (e == cudaSuccess)
-                e = timed_launch(ctx, 0, 2 * (int64_t)a.count, st,
-                                 [&] { return launch_stage_ctx(ctx, a, st); });
-            if (e == cudaSuccess && a.margin > 0.0) {
-                e = timed_launch(ctx, 1, 0, st, [&] { return launch_resolve_ctx(ctx, a, st); });
+                e = launched(0, 2 * (int64_t)a.count, [&] { return launch_stage_ctx(ctx, a, st); });
+            if (e == cudaSuccess && (a.margin > 0.0 || on_determinants(ctx))) {
+                e = launched(1, 0, [&] { return launch_resolve_ctx(ctx, a, st); });
                 if (e == cudaSuccess) e = cudaMemsetAsync(ctx->d_flag_count, 0, sizeof(unsigned int), st);
             }
             prev_s = s;
@@ -723,7 +746,9 @@ static cudaError_t sweep_stages(ptca_ctx* ctx, int32_t n_sweeps, cudaStream_t st
     if (e == cudaSuccess && g > 0)
         e = ptca::launch_copy_sites(ctx->d_S[g & 1], ctx->d_S[(g + 1) & 1], ctx->d_sites + ctx->h_start[prev_s],
                                     ctx->h_start[prev_s + 1] - ctx->h_start[prev_s], st);
-    if (e == cudaSuccess) e = ptca::launch_set_u64(ctx->d_sweep_ctr, (unsigned long long)(ctx->sweeps + n_sweeps), st);
+    if (e == cudaSuccess)
+        e = captured ? ptca::launch_add_u64(ctx->d_sweep_ctr, (unsigned long long)n_sweeps, st)
+                     : ptca::launch_set_u64(ctx->d_sweep_ctr, (unsigned long long)(ctx->sweeps + n_sweeps), st);
     return e;
 }
 
@@ -946,7 +971,10 @@ cudaError_t ptca_internal_settle(ptca_ctx* ctx, cudaStream_t st, bool have_strea
 }
 
 // Everything one persistent sweep launch needs, as stream work (capturable).
+// On determinants a stage takes tens of microseconds, spread over the whole GPU by
+// thread-block clusters: there the stages stay separate launches.
 static cudaError_t enqueue_persistent(ptca_ctx* ctx, int32_t n_sweeps, cudaStream_t st) {
+    if (on_determinants(ctx)) return sweep_stages(ctx, n_sweeps, st, nullptr, true);
     ptca::PersistArgs p;
     std::memset(&p, 0, sizeof p);
     p.st = base_args(ctx);
@@ -971,7 +999,15 @@ static cudaError_t enqueue_persistent(ptca_ctx* ctx, int32_t n_sweeps, cudaStrea
 }
 
 static cudaError_t sweep_graph(ptca_ctx* ctx, int32_t n_sweeps, cudaStream_t st) {
-    if (ctx->graph && ctx->graph_sweeps == n_sweeps) return cudaGraphLaunch(ctx->graph, st);
+    // A graph of per-stage launches holds one sweep, whatever the call's count.
+    const bool per_sweep = on_determinants(ctx);
+    const int32_t held = per_sweep ? 1 : n_sweeps;
+    auto replay = [&]() {
+        cudaError_t r = cudaSuccess;
+        for (int32_t k = 0; k < n_sweeps && r == cudaSuccess; k += held) r = cudaGraphLaunch(ctx->graph, st);
+        return r;
+    };
+    if (ctx->graph && ctx->graph_sweeps == held) return replay();
     drop_graph(ctx);
     cudaStream_t cap = nullptr;
     cudaError_t e = cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking);
@@ -979,7 +1015,7 @@ static cudaError_t sweep_graph(ptca_ctx* ctx, int32_t n_sweeps, cudaStream_t st)
     cudaGraph_t g = nullptr;
     e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
     if (e == cudaSuccess) {
-        cudaError_t e2 = enqueue_persistent(ctx, n_sweeps, cap);
+        cudaError_t e2 = enqueue_persistent(ctx, held, cap);
         e = cudaStreamEndCapture(cap, &g);
         if (e2 != cudaSuccess) e = e2;
     }
@@ -992,8 +1028,8 @@ static cudaError_t sweep_graph(ptca_ctx* ctx, int32_t n_sweeps, cudaStream_t st)
         ctx->graph_failed = true;  // fall back to direct persistent launches
         return enqueue_persistent(ctx, n_sweeps, st);
     }
-    ctx->graph_sweeps = n_sweeps;
-    return cudaGraphLaunch(ctx->graph, st);
+    ctx->graph_sweeps = held;
+    return replay();
 }
 
 // Stream work of n_sweeps sweeps in the context's launch configuration
@@ -1452,7 +1488,7 @@ ptca_status ptca_stage_run(ptca_ctx* ctx, int64_t sweep_index, const int32_t* si
     a.rec_base = 0;
     PTCA_CUDA(cudaMemsetAsync(ctx->d_counters, 0, 4 * sizeof(unsigned long long), st));
     cudaError_t e = launch_stage_ctx(ctx, a, st);
-    if (e == cudaSuccess && a.margin > 0.0) {
+    if (e == cudaSuccess && (a.margin > 0.0 || on_determinants(ctx))) {
         e = launch_resolve_ctx(ctx, a, st);
         if (e == cudaSuccess) e = cudaMemsetAsync(a.flag_count, 0, sizeof(unsigned int), st);
     }

@@ -342,6 +342,7 @@ struct StageArgs {
     int32_t rec_base;
     int32_t nA;
     uint64_t sweep;
+    const unsigned long long* sweep_dev;  // added to sweep when set (launches captured in a graph)
     double* Fbuf;
     double* fillbuf;
     int32_t* ticket;
@@ -394,7 +395,8 @@ struct StageVar {
 
 __device__ __forceinline__ StageVar stage_var(const StageArgs& a) {
     StageVar v;
-    v.S_in = a.S_in; v.S_out = a.S_out; v.sites = a.sites; v.perm = a.perm; v.rec_base = a.rec_base; v.sweep = a.sweep;
+    v.S_in = a.S_in; v.S_out = a.S_out; v.sites = a.sites; v.perm = a.perm; v.rec_base = a.rec_base;
+    v.sweep = a.sweep + (a.sweep_dev ? *a.sweep_dev : 0);
     return v;
 }
 

@@ -196,6 +196,13 @@ cudaError_t launch_set_u64(unsigned long long* p, unsigned long long v, cudaStre
     return cudaGetLastError();
 }
 
+__global__ void k_add_u64(unsigned long long* p, unsigned long long v) { *p += v; }
+
+cudaError_t launch_add_u64(unsigned long long* p, unsigned long long v, cudaStream_t st) {
+    k_add_u64<<<1, 1, 0, st>>>(p, v);
+    return cudaGetLastError();
+}
+
 // Initial spins: uniform on the sphere from the counter generator.
 // Initial classical variables: unit vectors uniform on the sphere; for the
 // Holstein model distortions x uniform in [-1, 1] in component 0.

@@ -88,6 +88,7 @@ cudaError_t launch_check_compare(const Model& m, const int32_t* sites, int count
 cudaError_t launch_barrier_selftest(int blocks, unsigned int* bar, int32_t* err, unsigned long long timeout_ns,
                                     cudaStream_t st);
 cudaError_t launch_set_u64(unsigned long long* p, unsigned long long v, cudaStream_t st);
+cudaError_t launch_add_u64(unsigned long long* p, unsigned long long v, cudaStream_t st);
 // Large traveling clusters (orders above cluster_max_order, up to
 // large_max_order): one 16-warp CTA per matrix, the matrix in a global slot
 // per CTA (a.gL, gL_stride elements of float2/double2; the re-solve uses
@@ -121,5 +122,18 @@ int cluster_stage_grid(int C, int nA);
 cudaError_t launch_stage_cluster(int C, const StageArgs& a, int grid, cudaStream_t st);
 cudaError_t launch_observables(const double* S, int Lx, int Ly, const double* rec_Facc, const double* rec_fill,
                                const uint8_t* rec_acc, const int32_t* rec_n, int N, double* out, cudaStream_t st);
+
+
+// Stage kernels on determinants (kernels_resolvent.cu, PTCA_MIXED): whether
+// the problem's windows and temperature fit them, and a stage launch.
+bool resolvent_supported(const Model& m);
+cudaError_t configure_resolvent_kernels(size_t smem_limit);
+// few: stages too small to fill the GPU (the same for every launch of a context,
+// since the two forms round differently).
+cudaError_t launch_stage_resolvent(const StageArgs& a, bool few, int sms, cudaStream_t st);
+// Their free energies of visits c0 .. c0 + count - 1 for the checker (F[2k],
+// F[2k + 1] of visit c0 + k), and the double-float re-solve.
+cudaError_t launch_check_resolvent(const StageArgs& a, bool few, int c0, int count, double* F, cudaStream_t st);
+cudaError_t launch_resolve_resolvent(const StageArgs& a, int sms, cudaStream_t st);
 
 }  // namespace ptca

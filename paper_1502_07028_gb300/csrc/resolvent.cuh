@@ -1,0 +1,1095 @@
+// resolvent.cuh -- free energies of a visit from determinants of its cluster
+// matrix, without an eigenvalue.
+//
+// F = -T sum_k ln(1 + e^(-x_k)), x = (eps - mu)/T, is a short sum of
+// ln|det(mu - H + i T y_j)| over nodes y_j plus Tr H and Tr H^2
+// (fermi_nodes.cuh); the phases of the same determinants give the filling.
+// The window's hopping couples only neighbouring layers of sites, by a
+// multiple of the identity.  So the matrix is eliminated layer by layer with
+// blocks of order B = 2 (sites per layer), the update site last:
+//   A = (mu - H)/(T y) + i,   D_0 = A_00,
+//   X_k = D_k^-1,  D_{k+1} = A_{k+1,k+1} - t'^2 X_k        (t' = t/(T y)),
+// and, on a ring of layers, with the border blocks C_k, E_k that couple layer
+// k to the last one: C_{k+1} = -t' X_k C_k, E_{k+1} = -t' E_k X_k,
+// S -= E_k X_k C_k.  Every Schur complement of A keeps an imaginary part
+// of at least 1, so its 2x2 (one site's) pivots are never small, no pivoting is
+// needed, and the phases of their determinants add up without a branch cut.
+// H_new differs from H_old in the update site's 2x2 block alone: both visits'
+// determinants share every pivot but the last, dF comes from the last one, and
+// the rounding of the elimination cancels in it.
+//
+// Work per node: about (4 (L - 2) + 2) B^3 complex multiply-adds on a ring of L
+// layers, (L - 1) B^3 on an open one, against (4/3) n^3 for a Householder
+// reduction of each of the two matrices (n = B L): 0.10 M against 5.6 M at
+// n = 128, times 13 nodes at |x| <= 512.
+//
+// One node is eliminated by LPN lanes of a warp, which holds 32 / LPN nodes: the
+// larger the tile per lane, the fewer shuffles and loads per multiply-add.
+// Lane (r, c) of a GR x GC grid holds the rows of sites r + GR i and the columns of
+// sites c + GC j (both spins) in registers.  The pivot block, row and column
+// travel by shuffles (Gauss-Jordan in place, one site's two rows at a time);
+// the products read their operands from shared memory, where a matrix row is
+// padded by two elements so that the row groups hit different banks.
+#pragma once
+
+#include <cooperative_groups.h>
+
+#include "fermi_nodes.cuh"
+#include "kernels.cuh"
+
+namespace ptca {
+
+__device__ __forceinline__ dfl2 cfms(dfl2 a, dfl2 b, dfl2 acc) {
+    return mk(dot2_acc(acc.x, -a.x, b.x, a.y, b.y), dot2_acc(acc.y, -a.x, b.y, -a.y, b.x));
+}
+__device__ __forceinline__ float2 shfl_c(float2 v, int src) {
+    v.x = __shfl_sync(FULL_MASK, v.x, src);
+    v.y = __shfl_sync(FULL_MASK, v.y, src);
+    return v;
+}
+__device__ __forceinline__ dfl2 shfl_c(dfl2 v, int src) {
+    v.x.hi = __shfl_sync(FULL_MASK, v.x.hi, src);
+    v.x.lo = __shfl_sync(FULL_MASK, v.x.lo, src);
+    v.y.hi = __shfl_sync(FULL_MASK, v.y.hi, src);
+    v.y.lo = __shfl_sync(FULL_MASK, v.y.lo, src);
+    return v;
+}
+// Two consecutive elements of a matrix row (the first at an even index).
+__device__ __forceinline__ void ld2(const float2* p, float2& a, float2& b) {
+    const float4 v = *reinterpret_cast<const float4*>(p);
+    a = make_float2(v.x, v.y);
+    b = make_float2(v.z, v.w);
+}
+__device__ __forceinline__ void ld2(const dfl2* p, dfl2& a, dfl2& b) { a = p[0]; b = p[1]; }
+__device__ __forceinline__ void st2(float2* p, float2 a, float2 b) {
+    *reinterpret_cast<float4*>(p) = make_float4(a.x, a.y, b.x, b.y);
+}
+__device__ __forceinline__ void st2(dfl2* p, dfl2 a, dfl2 b) { p[0] = a; p[1] = b; }
+
+// Scalar helpers of the two arithmetics.
+__device__ __forceinline__ float rs_rcp(float x) { return __fdividef(1.f, x); }
+__device__ __forceinline__ dfl rs_rcp(dfl x) { return dfl(1.f, 0.f) / x; }
+__device__ __forceinline__ float rs_log1p(float q) { return log1pf(q); }
+__device__ __forceinline__ double rs_log1p(dfl q) { return log1p(double(q)); }
+__device__ __forceinline__ float rs_phase(float y, float x) { return atan2f(y, x); }
+__device__ __forceinline__ double rs_phase(dfl y, dfl x) { return atan2(double(y), double(x)); }
+
+__device__ __forceinline__ float2 cmulp(float2 a, float2 b) {
+    return make_float2(__fmaf_rn(-a.y, b.y, a.x * b.x), __fmaf_rn(a.y, b.x, a.x * b.y));
+}
+// g with 1 + g = -det(P + i): the determinant of a pivot block (stored without
+// its i) against i^2.
+template <typename V> __device__ __forceinline__ V rs_det_g(V p00, V p01, V p10, V p11) {
+    V m;
+    m.x = p00.x * p11.x; m.y = p00.x * p11.y;
+    m.x = m.x - p00.y * p11.y;
+    m.y = m.y + p00.y * p11.x;
+    m = cfms(p01, p10, m);
+    m = mk(p00.y + p11.y - m.x, -(p00.x + p11.x + m.y));
+    return m;
+}
+
+// Running sum of a lane's logarithms or phases: a float pair in FP32 (the
+// pivots' own rounding is all that is left), FP64 in double-float.
+template <typename T> struct RsSum;
+template <> struct RsSum<float> {
+    dfl v = dfl(0.f, 0.f);
+    __device__ __forceinline__ void add(float x) {
+        const dfl s = two_sum(v.hi, x);
+        v = dfl(s.hi, v.lo + s.lo);
+    }
+    __device__ __forceinline__ void merge(int o) { v = v + shfl_xor_dfl(v, o); }
+    __device__ __forceinline__ double value() const { return double(v); }
+};
+template <> struct RsSum<dfl> {
+    double v = 0.0;
+    __device__ __forceinline__ void add(double x) { v += x; }
+    __device__ __forceinline__ void merge(int o) { v += __shfl_xor_sync(FULL_MASK, v, o); }
+    __device__ __forceinline__ double value() const { return v; }
+};
+
+// On-site terms of a window site: mu - H = [[d + z, x - iy], [x + iy, d - z]].
+template <typename T> struct RsSite { T d, x, y, z; };
+template <typename T> struct RsOut { double lnd, th; T P[8]; };  // P: the last pivot block, without its i
+
+// Window of a visit in layer order.
+struct RsVisit {
+    int c, site, n, L, ns, u, us;   // stage index, lattice site, order, layers, sites per layer, update layer and site
+    int per, cls;                   // cluster periodic; node class (-1: |x| beyond the last class)
+};
+// Sums over the window, FP64.
+struct RsTerms { double x1, x2, cl, sn[3], lnu; };
+
+template <int GR_, int GC_, int SR_, int SC_, int MAXT_, int MINB_> struct RsTile {
+    static constexpr int GR = GR_, GC = GC_, SR = SR_, SC = SC_;
+    static constexpr int MAXT = MAXT_, MINB = MINB_;       // launch bounds of the stage kernels
+    static constexpr int NS = GR * SR, B = 2 * NS, RS = B + 2;
+    static constexpr int LPN = GR * GC, NPW = 32 / LPN;
+    // Elements of a node's buffers: padded so that the nodes of a warp start in
+    // different banks.
+    static constexpr int NODE = 3 * B * RS + (NPW == 1 ? 0 : LPN >= 16 ? 8 : LPN > 1 ? 2 * LPN : 2);
+    static_assert(GR * SR == GC * SC && GR % GC == 0 && 32 % LPN == 0, "square blocks");
+};
+using RsT1 = RsTile<1, 1, 1, 1, 256, 2>;    // chains: a node per lane
+using RsT4 = RsTile<2, 2, 2, 2, 256, 2>;    // up to 4 sites per layer: 4x4 per lane, eight nodes per warp
+using RsT8 = RsTile<4, 4, 2, 2, 224, 2>;    // two nodes per warp
+using RsT12 = RsTile<4, 4, 3, 3, 224, 1>;   // 6x6 per lane
+using RsT16 = RsTile<8, 4, 2, 4, 256, 1>;   // 4x8 per lane, one node per warp
+
+template <class Tl> struct RsNode {
+    using V = float2;
+    static constexpr int GR = Tl::GR, GC = Tl::GC, SR = Tl::SR, SC = Tl::SC, NS = Tl::NS, RS = Tl::RS;
+    using Tile = V[2 * SR][2 * SC];
+
+    // Tile row a: spin a / SR of site r + GR (a % SR); column likewise.  In
+    // memory rows are grouped by spin and columns by site (the two spins of a
+    // site in one 16-byte load), so that a row of the left operand and the
+    // matching row of the right one are col = 2 site + spin apart.
+    static __device__ __forceinline__ int row(int r, int a) { return (a / SR) * NS + r + GR * (a % SR); }
+    static __device__ __forceinline__ int csite(int c, int s) { return c + GC * s; }
+    static __device__ __forceinline__ V shfl(V v, int src) { return Tl::LPN == 1 ? v : shfl_c(v, src); }
+
+    static __device__ __forceinline__ void store(V* M, const Tile& a, int r, int c) {
+#pragma unroll
+        for (int i = 0; i < 2 * SR; ++i) {
+            V* p = M + row(r, i) * RS;
+#pragma unroll
+            for (int j = 0; j < SC; ++j) st2(p + 2 * csite(c, j), a[i][j], a[i][SC + j]);
+        }
+    }
+
+    static __device__ __forceinline__ void load(Tile& a, const V* M, int r, int c) {
+#pragma unroll
+        for (int i = 0; i < 2 * SR; ++i)
+#pragma unroll
+            for (int j = 0; j < SC; ++j) ld2(M + row(r, i) * RS + 2 * csite(c, j), a[i][j], a[i][SC + j]);
+    }
+
+    // o = P Q
+    static __device__ __forceinline__ void mul(Tile& o, const V* P, const V* Q, int ns, int r, int c) {
+#pragma unroll
+        for (int i = 0; i < 2 * SR; ++i)
+#pragma unroll
+            for (int j = 0; j < 2 * SC; ++j) o[i][j] = make_float2(0.f, 0.f);
+#pragma unroll 2
+        for (int k = 0; k < ns; ++k) {   // site k: its two columns of P, its two rows of Q
+            V p[2 * SR][2];
+#pragma unroll
+            for (int i = 0; i < 2 * SR; ++i) ld2(P + row(r, i) * RS + 2 * k, p[i][0], p[i][1]);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const V* q = Q + (h * NS + k) * RS;
+                V b[2 * SC];
+#pragma unroll
+                for (int j = 0; j < SC; ++j) ld2(q + 2 * csite(c, j), b[j], b[SC + j]);
+#pragma unroll
+                for (int i = 0; i < 2 * SR; ++i)
+#pragma unroll
+                    for (int j = 0; j < 2 * SC; ++j) o[i][j] = cfma(p[i][h], b[j], o[i][j]);
+            }
+        }
+    }
+    // M = f o, between the warp's last read of the operands and the next
+    static __device__ __forceinline__ void put(V* M, Tile& o, float f, int r, int c) {
+#pragma unroll
+        for (int i = 0; i < 2 * SR; ++i)
+#pragma unroll
+            for (int j = 0; j < 2 * SC; ++j) o[i][j] = make_float2(f * o[i][j].x, f * o[i][j].y);
+        __syncwarp();
+        store(M, o, r, c);
+        __syncwarp();
+    }
+
+    // The block of layer l without its i on the diagonal, minus tt X (X in a).
+    static __device__ __forceinline__ void layer(Tile& a, const RsSite<float>* site, const float* hop, float s, float tt,
+                                                 int ns, int r, int c, bool chain) {
+#pragma unroll
+        for (int i = 0; i < SR; ++i) {
+            const int sr = r + GR * i;
+            const float f = sr < ns ? tt : 0.f;
+#pragma unroll
+            for (int j = 0; j < SC; ++j) {
+                const int sc = csite(c, j);
+                const float h = hop[sr * NS + sc] * s;
+                V uu = make_float2(h, 0.f), dd = uu, ud = make_float2(0.f, 0.f), du = ud;
+                if (sr == sc && sr < ns) {
+                    const RsSite<float> o = site[sr];
+                    const float x = o.x * s, y = o.y * s;
+                    uu.x = (o.d + o.z) * s;
+                    dd.x = (o.d - o.z) * s;
+                    ud = make_float2(x, -y);
+                    du = make_float2(x, y);
+                }
+                if (chain) {
+                    const V x00 = a[i][j], x01 = a[i][SC + j], x10 = a[SR + i][j], x11 = a[SR + i][SC + j];
+                    uu = make_float2(uu.x - f * x00.x, -(f * x00.y));
+                    dd = make_float2(dd.x - f * x11.x, -(f * x11.y));
+                    ud = make_float2(ud.x - f * x01.x, ud.y - f * x01.y);
+                    du = make_float2(du.x - f * x10.x, du.y - f * x10.y);
+                }
+                a[i][j] = uu;
+                a[SR + i][SC + j] = dd;
+                a[i][SC + j] = ud;
+                a[SR + i][j] = du;
+            }
+        }
+    }
+
+    // Gauss-Jordan inversion in place of the block a + i, one site at a time;
+    // site `skip` and the padding from ns on are left out.  The sums of
+    // ln|det|^2 and of the phases of the 2x2 pivots (against i^2) go to lnd, th.
+    // The pivots of one round lie in tile row 0 and columns 0 .. GR/GC - 1;
+    // the tile is turned by a round's worth afterwards (SR rounds are a full
+    // turn), so that the body exists once: unrolled over the rounds it
+    // overflowed the instruction cache (1.45 no-instruction stalls per issue).
+    static __device__ __forceinline__ void invert(Tile& a, RsSum<float>& lnd, RsSum<float>& th, int skip, int ns, int r, int c,
+                                                  int nl, int base) {
+        constexpr int QR = GR / GC;
+        static_assert(NS <= Tl::LPN || NS == 1, "a lane per pivot");
+        const V zero = make_float2(0.f, 0.f);
+        V g = zero;
+#pragma unroll 1
+        for (int p0 = 0; p0 < ns; p0 += GR) {
+#pragma unroll
+            for (int s = 0; s < QR; ++s) {
+#pragma unroll 1
+                for (int cp = 0; cp < GC; ++cp) {
+                    const int rp = s * GC + cp, p = p0 + rp;
+                    if (p == skip || p >= ns) continue;
+                    const int src = base + rp * GC + cp;
+                    const V p00 = shfl(a[0][s], src), p01 = shfl(a[0][SC + s], src);
+                    const V p10 = shfl(a[SR][s], src), p11 = shfl(a[SR][SC + s], src);
+                    const V gp = rs_det_g(p00, p01, p10, p11);
+                    if (nl == p) g = gp;
+                    // inverse of P + i: -(adj) conj(1 + g)/|1 + g|^2
+                    const float gr = 1.f + gp.x, rq = rs_rcp(gr * gr + gp.y * gp.y);
+                    const V w = make_float2(-(gr * rq), gp.y * rq), wn = make_float2(-w.x, -w.y);   // 1/det
+                    const V i00 = cmulp(make_float2(p11.x, p11.y + 1.f), w), i11 = cmulp(make_float2(p00.x, p00.y + 1.f), w);
+                    const V i01 = cmulp(p01, wn), i10 = cmulp(p10, wn);
+                    const bool pr = r == rp, pc = c == cp;
+                    V q0[2 * SR], q1[2 * SR];
+                    const int csrc = base + r * GC + cp, rsrc = base + rp * GC + c;
+#pragma unroll
+                    for (int k = 0; k < 2 * SR; ++k) {
+                        const V c0 = shfl(a[k][s], csrc), c1 = shfl(a[k][SC + s], csrc);
+                        q0[k] = cfma(c1, i10, cmulp(c0, i00));
+                        q1[k] = cfma(c1, i11, cmulp(c0, i01));
+                    }
+                    if (pr) {
+                        q0[0] = make_float2(-i00.x, -i00.y);
+                        q1[0] = make_float2(-i01.x, -i01.y);
+                        q0[SR] = make_float2(-i10.x, -i10.y);
+                        q1[SR] = make_float2(-i11.x, -i11.y);
+                    }
+#pragma unroll
+                    for (int j = 0; j < 2 * SC; ++j) {
+                        const V r0 = shfl(a[0][j], rsrc), r1 = shfl(a[SR][j], rsrc);
+                        if (pr) { a[0][j] = zero; a[SR][j] = zero; }
+#pragma unroll
+                        for (int k = 0; k < 2 * SR; ++k) a[k][j] = cfms(q1[k], r1, cfms(q0[k], r0, a[k][j]));
+                    }
+                    if (pc) {
+#pragma unroll
+                        for (int k = 0; k < 2 * SR; ++k) {
+                            a[k][s] = make_float2(-q0[k].x, -q0[k].y);
+                            a[k][SC + s] = make_float2(-q1[k].x, -q1[k].y);
+                        }
+                    }
+                }
+            }
+            turn(a);
+        }
+        // padding shorter than a full turn
+#pragma unroll 1
+        for (int p0 = (ns + GR - 1) / GR; p0 < SR; ++p0) turn(a);
+        if (nl < NS) {
+            lnd.add(log1pf((g.x + g.x) + (g.x * g.x + g.y * g.y)));
+            th.add(atan2f(g.y, 1.f + g.x));
+        }
+    }
+    static __device__ __forceinline__ void turn(Tile& a) {
+        if constexpr (SR > 1) {
+            Tile b;
+#pragma unroll
+            for (int i = 0; i < 2 * SR; ++i)
+#pragma unroll
+                for (int j = 0; j < 2 * SC; ++j)
+                    b[i][j] = a[(i / SR) * SR + (i % SR + 1) % SR][(j / SC) * SC + (j % SC + GR / GC) % SC];
+#pragma unroll
+            for (int i = 0; i < 2 * SR; ++i)
+#pragma unroll
+                for (int j = 0; j < 2 * SC; ++j) a[i][j] = b[i][j];
+        }
+    }
+
+    // One node of one visit: the sums over all pivots but the update site's,
+    // and that site's last pivot block.  s: 1 / (T y), tp: t / (T y).
+    static __device__ __forceinline__ void run(const RsVisit& v, const RsSite<float>* site, const float* hop, float s, float tp,
+                                               V* buf, int lane, RsOut<float>* out) {
+        const int base = lane & ~(Tl::LPN - 1), nl = lane - base;
+        const int r = nl / GC, c = nl % GC;
+        const int L = v.L, ns = v.ns;
+        V *X = buf, *C = buf + Tl::B * RS, *E = C + Tl::B * RS;
+        const bool ring = v.per && L >= 3;
+        const float tt = tp * tp, tau2 = (v.per && L == 2) ? 4.f * tt : tt;
+        Tile a, S;
+        RsSum<float> lnd, th;
+        layer(S, site + v.u * ns, hop, s, tt, ns, r, c, false);
+#pragma unroll 1
+        for (int o = 0; o < L; ++o) {
+            const bool last = o == L - 1;
+            if (last) {
+#pragma unroll
+                for (int i = 0; i < 2 * SR; ++i)
+#pragma unroll
+                    for (int j = 0; j < 2 * SC; ++j) a[i][j] = S[i][j];
+            } else {
+                // elimination order: round the ring from the update layer, or
+                // from both ends of an open window towards it
+                int l;
+                if (v.per) { l = v.u + 1 + o; if (l >= L) l -= L; }
+                else l = o < v.u ? o : L - 1 - (o - v.u);
+                layer(a, site + l * ns, hop, s, tt, ns, r, c, o > 0 && (v.per || o != v.u));
+            }
+            invert(a, lnd, th, last ? v.us : -1, ns, r, c, nl, base);
+            if (last) break;
+            if (ring && o > 0) {
+                // Stored: W_k = E_k X_k and Y_k = X_k C_k; the next border
+                // blocks are -t' times these, and at the last eliminated layer the
+                // direct bond t' is added (-t' (Y - 1)).  X leaves the registers
+                // meanwhile (they hold S and one product).
+                if (o == L - 2)
+                    for (int k = nl; k < 2 * ns; k += Tl::LPN) {
+                        const int d = ((k & 1) * NS + (k >> 1)) * RS + k;
+                        C[d].x -= 1.f;
+                        E[d].x -= 1.f;
+                    }
+                store(X, a, r, c);
+                __syncwarp();
+                Tile w;
+#pragma unroll 1
+                for (int q = 0; q < (o < L - 2 ? 3 : 2); ++q) {   // E X -> E, S += t' E C, X C -> C
+                    mul(w, q == 2 ? X : E, q == 0 ? X : C, ns, r, c);
+                    if (q == 1) {
+#pragma unroll
+                        for (int i = 0; i < 2 * SR; ++i)
+#pragma unroll
+                            for (int j = 0; j < 2 * SC; ++j)
+                                S[i][j] = make_float2(S[i][j].x + tp * w[i][j].x, S[i][j].y + tp * w[i][j].y);
+                    } else {
+                        put(q == 0 ? E : C, w, -tp, r, c);
+                    }
+                }
+                load(a, X, r, c);
+                __syncwarp();
+                continue;
+            }
+            if (!ring && !(o == L - 2 || (!v.per && o == v.u - 1))) continue;
+            // S -= (coupling)^2 X, on real sites; the ring's first layer also
+            // starts the border blocks with t' X.
+            const float cc = ring ? tt : tau2;
+#pragma unroll
+            for (int i = 0; i < 2 * SR; ++i) {
+                const float f = (r + GR * (i % SR)) < ns ? cc : 0.f;
+#pragma unroll
+                for (int j = 0; j < 2 * SC; ++j) S[i][j] = make_float2(S[i][j].x - f * a[i][j].x, S[i][j].y - f * a[i][j].y);
+            }
+            if (ring) {
+                Tile w;
+#pragma unroll
+                for (int i = 0; i < 2 * SR; ++i) {
+                    const float f = (r + GR * (i % SR)) < ns ? tp : 0.f;
+#pragma unroll
+                    for (int j = 0; j < 2 * SC; ++j) w[i][j] = make_float2(f * a[i][j].x, f * a[i][j].y);
+                }
+                store(C, w, r, c);
+                store(E, w, r, c);
+                __syncwarp();
+            }
+        }
+        // last pivot block: the lane holding rows and columns of the update site
+#pragma unroll
+        for (int i = 0; i < SR; ++i)
+#pragma unroll
+            for (int j = 0; j < SC; ++j)
+                if (r + GR * i == v.us && csite(c, j) == v.us) {
+                    out->P[0] = a[i][j].x; out->P[1] = a[i][j].y;
+                    out->P[2] = a[i][SC + j].x; out->P[3] = a[i][SC + j].y;
+                    out->P[4] = a[SR + i][j].x; out->P[5] = a[SR + i][j].y;
+                    out->P[6] = a[SR + i][SC + j].x; out->P[7] = a[SR + i][SC + j].y;
+                }
+#pragma unroll
+        for (int o = Tl::LPN / 2; o > 0; o >>= 1) {
+            lnd.merge(o);
+            th.merge(o);
+        }
+        if (nl == 0) {
+            out->lnd = 0.5 * lnd.value();
+            out->th = th.value();
+        }
+        __syncwarp();
+    }
+};
+
+// ---------------------------------------------------------------------------
+// The same elimination by a group of GR x GC threads per node, for stages with
+// too few visits to fill the GPU and for the re-solve: there the time of one
+// node counts, not the throughput.  Thread (r, c) holds rows r + GR i and columns
+// c + GC j (a row is 2 site + spin); one row is pivoted at a time, its
+// row and column broadcast through double-buffered shared memory (one barrier of
+// the group per pivot), and nothing is padded.  Against one warp per node
+// with a 2x4 tile per lane: 45 us instead of 400 us per node in double-float
+// at n = 128.
+// ---------------------------------------------------------------------------
+template <int GR_, int GC_, int R_, int C_, int DFG_, int SPG_> struct RsGroupShape {
+    static constexpr int SPG = SPG_;                              // ... and at most of the FP32 stage kernel
+    static constexpr int DFG = DFG_;                              // groups per CTA of the re-solve
+    static constexpr int GR = GR_, GC = GC_, R = R_, C = C_, TPN = GR * GC;
+    static constexpr int B = GR * R > GC * C ? GR * R : GC * C;   // largest block order
+    static constexpr int RS = B + 1;                              // elements per matrix row
+};
+using RsG8 = RsGroupShape<8, 4, 1, 2, 4, 8>;       // one warp, up to 4 sites per layer
+using RsG16 = RsGroupShape<16, 8, 1, 2, 3, 4>;     // four warps, up to 8 sites
+using RsG24 = RsGroupShape<16, 8, 2, 3, 3, 4>;     // ... 12 sites
+using RsG32 = RsGroupShape<16, 16, 2, 2, 2, 2>;    // eight warps, up to 16 sites
+
+template <typename T, class Gp> struct RsGroup {
+    using V = cplx_t<T>;
+    static constexpr int GR = Gp::GR, GC = Gp::GC, R = Gp::R, C = Gp::C, RS = Gp::RS;
+    using Tile = V[R][C];
+    // Shared memory of a group: three matrices, two broadcast buffers of a pivot
+    // row and column, the pivots of a layer.
+    struct Smem { V X[Gp::B * RS], C[Gp::B * RS], E[Gp::B * RS], row[2][Gp::B], col[2][Gp::B], piv[Gp::B]; };
+
+    static __device__ __forceinline__ void sync(int id) {
+        if constexpr (Gp::TPN == 32) __syncwarp();
+        else asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(Gp::TPN) : "memory");
+    }
+    static __device__ __forceinline__ void store(V* M, const Tile& a, T f, int b, int r, int c) {
+#pragma unroll
+        for (int i = 0; i < R; ++i)
+#pragma unroll
+            for (int j = 0; j < C; ++j) {
+                const int x = r + GR * i, y = c + GC * j;
+                if (x < b && y < b) M[x * RS + y] = mk(f * a[i][j].x, f * a[i][j].y);
+            }
+    }
+    static __device__ __forceinline__ void mul(Tile& o, const V* P, const V* Q, int b, int r, int c) {
+#pragma unroll
+        for (int i = 0; i < R; ++i)
+#pragma unroll
+            for (int j = 0; j < C; ++j) o[i][j] = mk(T(0.f), T(0.f));
+        // rows and columns past the block read the last one and are not used
+#pragma unroll 2
+        for (int k = 0; k < b; ++k) {
+            V p[R];
+#pragma unroll
+            for (int i = 0; i < R; ++i) p[i] = P[(r + GR * i < b ? r + GR * i : b - 1) * RS + k];
+#pragma unroll
+            for (int j = 0; j < C; ++j) {
+                const V q = Q[k * RS + (c + GC * j < b ? c + GC * j : b - 1)];
+#pragma unroll
+                for (int i = 0; i < R; ++i) o[i][j] = cfma(p[i], q, o[i][j]);
+            }
+        }
+    }
+    // The block of a layer without its i, minus tt X (X in a).
+    static __device__ __forceinline__ void layer(Tile& a, const RsSite<T>* site, const T* hop, int hs, T s, T tt, int b,
+                                                 int r, int c, bool chain) {
+#pragma unroll
+        for (int i = 0; i < R; ++i)
+#pragma unroll
+            for (int j = 0; j < C; ++j) {
+                const int x = r + GR * i, y = c + GC * j, sx = x >> 1, sy = y >> 1;
+                V e = mk(T(0.f), T(0.f));
+                if (x < b && y < b) {
+                    if (sx == sy) {
+                        const RsSite<T> o = site[sx];
+                        if (x == y) e.x = ((x & 1) ? o.d - o.z : o.d + o.z) * s;
+                        else { e.x = o.x * s; e.y = (x & 1) ? o.y * s : -(o.y * s); }
+                    } else if (((x ^ y) & 1) == 0) {
+                        e.x = hop[sx * hs + sy] * s;
+                    }
+                    if (chain) { e.x = e.x - tt * a[i][j].x; e.y = e.y - tt * a[i][j].y; }
+                }
+                a[i][j] = e;
+            }
+    }
+    // Gauss-Jordan inversion in place of a + i; rows 2 skip and 2 skip + 1 are
+    // left out.  The pivots go to sm.piv (without their i).
+    static __device__ __forceinline__ void invert(Tile& a, Smem& sm, int skip, int b, int r, int c, int id) {
+#pragma unroll 1
+        for (int p = 0; p < b; ++p) {
+            if ((p >> 1) == skip) continue;
+            V* row = sm.row[p & 1];
+            V* col = sm.col[p & 1];
+#pragma unroll
+            for (int i = 0; i < R; ++i)
+#pragma unroll
+                for (int j = 0; j < C; ++j) {
+                    if (r + GR * i == p && c + GC * j < b) row[c + GC * j] = a[i][j];
+                    if (c + GC * j == p && r + GR * i < b) col[r + GR * i] = a[i][j];
+                }
+            sync(id);
+            const V pv = row[p];
+            if (r == 0 && c == 0) sm.piv[p] = pv;
+            const T im = pv.y + T(1.f), rq = rs_rcp(pv.x * pv.x + im * im);
+            const V w = mk(pv.x * rq, -(im * rq));     // 1/(pivot + i)
+            const V zero = mk(T(0.f), T(0.f));
+            V rv[C];
+#pragma unroll
+            for (int j = 0; j < C; ++j) rv[j] = c + GC * j < b ? row[c + GC * j] : zero;
+#pragma unroll
+            for (int i = 0; i < R; ++i) {
+                const bool pr = r + GR * i == p;
+                const V q = pr ? mk(-w.x, -w.y) : cfma(r + GR * i < b ? col[r + GR * i] : zero, w, zero);
+#pragma unroll
+                for (int j = 0; j < C; ++j) {
+                    const V x = cfms(q, rv[j], pr ? zero : a[i][j]);
+                    a[i][j] = c + GC * j == p ? mk(-q.x, -q.y) : x;
+                }
+            }
+        }
+    }
+
+    static __device__ __forceinline__ void run(const RsVisit& v, const RsSite<T>* site, const T* hop, int hs, T s, T tp,
+                                               Smem& sm, int t, int id, RsOut<T>* out) {
+        const int r = t / GC, c = t % GC, L = v.L, ns = v.ns, b = 2 * ns;
+        const bool ring = v.per && L >= 3;
+        const T tt = tp * tp, tau2 = (v.per && L == 2) ? T(4.f) * tt : tt, one = T(1.f);
+        Tile a, S;
+        RsSum<T> lnd, th;
+        layer(S, site + v.u * ns, hop, hs, s, tt, b, r, c, false);
+#pragma unroll 1
+        for (int o = 0; o < L; ++o) {
+            const bool last = o == L - 1;
+            if (last) {
+#pragma unroll
+                for (int i = 0; i < R; ++i)
+#pragma unroll
+                    for (int j = 0; j < C; ++j) a[i][j] = S[i][j];
+            } else {
+                int l;
+                if (v.per) { l = v.u + 1 + o; if (l >= L) l -= L; }
+                else l = o < v.u ? o : L - 1 - (o - v.u);
+                layer(a, site + l * ns, hop, hs, s, tt, b, r, c, o > 0 && (v.per || o != v.u));
+            }
+            invert(a, sm, last ? v.us : -1, b, r, c, id);
+            sync(id);
+            for (int p = t; p < b; p += Gp::TPN)
+                if (!(last && (p >> 1) == v.us)) {
+                    const V pv = sm.piv[p];
+                    lnd.add(rs_log1p((pv.y + pv.y) + (pv.x * pv.x + pv.y * pv.y)));
+                    th.add(rs_phase(-pv.x, one + pv.y));
+                }
+            if (last) break;
+            if (ring && o > 0) {
+                if (o == L - 2 && t < b) {
+                    sm.C[t * RS + t].x = sm.C[t * RS + t].x - one;
+                    sm.E[t * RS + t].x = sm.E[t * RS + t].x - one;
+                }
+                store(sm.X, a, one, b, r, c);
+                sync(id);
+                Tile w;
+                mul(w, sm.E, sm.X, b, r, c);
+                sync(id);
+                store(sm.E, w, -tp, b, r, c);
+                sync(id);
+                mul(w, sm.E, sm.C, b, r, c);
+#pragma unroll
+                for (int i = 0; i < R; ++i)
+#pragma unroll
+                    for (int j = 0; j < C; ++j) S[i][j] = mk(S[i][j].x + tp * w[i][j].x, S[i][j].y + tp * w[i][j].y);
+                if (o < L - 2) {
+                    mul(w, sm.X, sm.C, b, r, c);
+                    sync(id);
+                    store(sm.C, w, -tp, b, r, c);
+                }
+                sync(id);
+                continue;
+            }
+            if (!ring && !(o == L - 2 || (!v.per && o == v.u - 1))) continue;
+            const T cc = ring ? tt : tau2;
+#pragma unroll
+            for (int i = 0; i < R; ++i)
+#pragma unroll
+                for (int j = 0; j < C; ++j) S[i][j] = mk(S[i][j].x - cc * a[i][j].x, S[i][j].y - cc * a[i][j].y);
+            if (ring) {
+                store(sm.C, a, tp, b, r, c);
+                store(sm.E, a, tp, b, r, c);
+                sync(id);
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < R; ++i)
+#pragma unroll
+            for (int j = 0; j < C; ++j) {
+                const int x = r + GR * i, y = c + GC * j;
+                if ((x >> 1) == v.us && (y >> 1) == v.us) {
+                    const int k = 4 * (x & 1) + 2 * (y & 1);
+                    out->P[k] = a[i][j].x;
+                    out->P[k + 1] = a[i][j].y;
+                }
+            }
+        // rows 0 .. b - 1 were summed by the group's first threads
+        if (t < 32) {
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) { lnd.merge(o); th.merge(o); }
+            if (t == 0) {
+                out->lnd = 0.5 * lnd.value();
+                out->th = th.value();
+            }
+        }
+        sync(id);
+    }
+};
+
+// ---------------------------------------------------------------------------
+// A CTA's share of a stage: up to VB visits.  Shared memory (byte offsets):
+// the visits' headers, FP64 terms, node results, window sites, in-layer
+// hopping, and one set of block buffers per concurrently eliminated node.
+// ---------------------------------------------------------------------------
+struct RsLayout { size_t terms, out, site, hop, buf, total; };
+
+// kOut: nodes kept per visit.  One hopping table when all windows have one shape.
+template <class Tl>
+__host__ __device__ inline RsLayout rs_layout(int vb, int max_sites, int nw, bool uniform) {
+    RsLayout L;
+    size_t o = align16((size_t)vb * sizeof(RsVisit));
+    L.terms = o; o = align16(o + (size_t)vb * sizeof(RsTerms));
+    L.out = o;   o = align16(o + (size_t)vb * kFermiOut * sizeof(RsOut<float>));
+    L.site = o;  o = align16(o + (size_t)vb * max_sites * sizeof(RsSite<float>));
+    L.hop = o;   o = align16(o + (size_t)(uniform ? 1 : vb) * Tl::NS * Tl::NS * sizeof(float));
+    L.buf = o;   o = align16(o + (size_t)nw * Tl::NPW * Tl::NODE * sizeof(float2));
+    L.total = o;
+    return L;
+}
+
+__constant__ FermiNodes c_fermi[kFermiClasses] = {PTCA_FERMI_NODES};
+__constant__ FermiNodes c_fermi_df[kFermiClasses] = {PTCA_FERMI_NODES_DF};
+
+// The nodes of an arithmetic: their approximation error is below its rounding.
+template <typename T> struct RsFermi {
+    static __device__ __forceinline__ const FermiNodes& tab(int cls) { return sizeof(T) == 4 ? c_fermi[cls] : c_fermi_df[cls]; }
+};
+
+// Window of a visit in layer order (layers along its longest axis, so that a
+// layer has the fewest sites), gathered by GL lanes of a warp: the on-site
+// terms, the in-layer hopping (when hop is given), Tr x and Tr x^2 over the
+// window, the classical energy, and the node class from Gershgorin's bound on
+// |mu - H|.
+template <typename T, int GL>
+__device__ __forceinline__ void rs_gather(const Model& m, const double* S, int c, int site, RsVisit& h, RsTerms& w,
+                                          RsSite<T>* sites, T* hop, int hs, int gl) {
+    const Window win = make_window(m, site);
+    const int ext[3] = {win.ex, win.ey, win.ez}, up[3] = {win.uwx, win.uwy, win.uwz};
+    int ax = 0;
+    if (ext[1] > ext[0]) ax = 1;
+    if (ext[2] > (ax ? ext[1] : ext[0])) ax = 2;
+    const int L = ax == 0 ? ext[0] : ax == 1 ? ext[1] : ext[2];
+    const int e0 = ax == 0 ? ext[1] : ext[0], e1 = ax == 2 ? ext[1] : ext[2];  // the other axes, in order
+    const int u0 = ax == 0 ? up[1] : up[0], u1 = ax == 2 ? up[1] : up[2];
+    const int ns = e0 * e1, nsite = ns * L, per = m.cluster_periodic;
+    const double mus = m.mu - m.e0;
+    double x1 = 0.0, x2 = 0.0, cl = 0.0;
+    float bound = 0.f;
+    for (int k = gl; k < nsite; k += GL) {
+        const int l = k / ns, q = k % ns, q0 = q % e0, q1 = q / e0;
+        const int wx = ax == 0 ? l : q0, wy = ax == 1 ? l : (ax == 0 ? q0 : q1), wz = ax == 2 ? l : q1;
+        const double* v = S + 3 * (int64_t)window_site(m, win, wx, wy, wz);
+        const double v0 = v[0], v1 = v[1], v2 = v[2], m2 = v0 * v0 + v1 * v1 + v2 * v2;
+        const double d = mus - m.lam * v0;
+        sites[k].d = T(d); sites[k].x = T(m.JH * v0); sites[k].y = T(m.JH * v1); sites[k].z = T(m.JH * v2);
+        x1 -= 2.0 * d;
+        x2 += 2.0 * (d * d + m.JH * m.JH * m2);
+        if (m.cls_on) cl += m.ca * m2 + m.cb * v0 + m.cc;
+        bound = fmaxf(bound, fabsf((float)d) + fabsf((float)m.JH) * sqrtf((float)m2));
+    }
+    // in-layer bonds (an axis of extent 2 of a periodic cluster has two)
+    if (hop) for (int k = gl; k < hs * hs; k += GL) {
+        const int a = k / hs, b = k % hs;
+        double bonds = 0.0;
+        if (a < ns && b < ns) {
+            const int d0 = abs(a % e0 - b % e0), d1 = abs(a / e0 - b / e0);
+            if (d1 == 0 && d0 > 0) bonds = (d0 == 1) + (per && d0 == e0 - 1);
+            if (d0 == 0 && d1 > 0) bonds = (d1 == 1) + (per && d1 == e1 - 1);
+        }
+        hop[k] = T(m.t * bonds);
+    }
+#pragma unroll
+    for (int o = GL / 2; o > 0; o >>= 1) {
+        x1 += __shfl_xor_sync(FULL_MASK, x1, o);
+        x2 += __shfl_xor_sync(FULL_MASK, x2, o);
+        if (m.cls_on) cl += __shfl_xor_sync(FULL_MASK, cl, o);
+        bound = fmaxf(bound, __shfl_xor_sync(FULL_MASK, bound, o));
+    }
+    if (gl == 0) {
+        double pairs = 0.0, deg = 0.0;
+        for (int k = 0; k < 3; ++k) {
+            const int e = k == 0 ? L : k == 1 ? e0 : e1;
+            if (e < 2) continue;
+            const double lines = (double)(nsite / e);
+            pairs += lines * (per ? (e == 2 ? 4.0 : (double)e) : (double)(e - 1));
+            deg += e == 2 && !per ? 1.0 : 2.0;
+        }
+        x2 += 4.0 * m.t * m.t * pairs;
+        const double X = ((double)bound * (1.0 + 1e-6) + deg * fabs(m.t)) / m.T;
+        int cls = 0;
+        while (cls < kFermiClasses && !(X <= c_fermi[cls].X)) ++cls;
+        h.c = c; h.site = site; h.n = 2 * nsite; h.L = L; h.ns = ns; h.per = per;
+        h.u = ax == 0 ? up[0] : ax == 1 ? up[1] : up[2];
+        h.us = u1 * e0 + u0;
+        h.cls = cls < kFermiClasses ? cls : -1;
+        w.x1 = x1 / m.T;
+        w.x2 = x2 / (m.T * m.T);
+        w.cl = cl;
+    }
+}
+
+// What a visit's free energies are for: the stage's decision, with decisions
+// near the threshold left to the re-solve; the re-solve's decision; or the
+// precision checker, which takes the two free energies alone (Fbuf[2c],
+// Fbuf[2c + 1]).
+enum RsMode { RS_STAGE, RS_RESOLVE, RS_CHECK };
+
+// Metropolis on dF and the visit's records (one thread).  fine: the free
+// energies are valid (the window lies within the node classes).
+template <RsMode kMode>
+__device__ __forceinline__ void rs_commit(const StageArgs& a, const StageVar& v, const RsVisit& h, const RsTerms& w,
+                                          bool fine, double Fo, double dF, double fo, double fn) {
+    const Model& m = a.m;
+    const double Fn = Fo + dF;
+    const double* so = v.S_in + 3 * (int64_t)h.site;
+    const int c = h.c, site = h.site;
+    if constexpr (kMode == RS_CHECK) {
+        if (fine) { a.Fbuf[2 * c] = Fo; a.Fbuf[2 * c + 1] = Fn; }
+        return;
+    }
+    if (fine && !isfinite(dF)) atomicExch(a.err, 1);
+    const double dFe = stage2_dF(a, c, dF);
+    if constexpr (kMode == RS_STAGE) {
+        // near the threshold, or a window beyond the last node class
+        if (!fine || (a.margin > 0.0 && fabs(w.lnu + dFe / m.T) < a.margin)) {
+            a.flag_list[atomicAdd(a.flag_count, 1u)] = c;
+            atomicAdd(&a.counters[2], 1ull);
+            return;
+        }
+    }
+    const bool acc = w.lnu < -dFe / m.T;
+    if (a.sg_feat) collect_sample(a, v.S_in, make_window(m, site), v.rec_base + c, w.sn, dF);
+    double* dst = v.S_out + 3 * (int64_t)site;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) dst[k] = acc ? w.sn[k] : so[k];
+    const int r = v.rec_base + c;
+    a.rec_site[r] = site;
+    a.rec_Fold[r] = Fo;
+    a.rec_Fnew[r] = Fn;
+    a.rec_lnu[r] = w.lnu;
+    a.rec_acc[r] = acc ? 1 : 0;
+    a.rec_Facc[r] = acc ? Fn : Fo;
+    a.rec_fill[r] = acc ? fn : fo;
+    a.rec_n[r] = h.n;
+    if (acc) atomicAdd(&a.counters[0], 1ull);
+    atomicAdd(&a.counters[1], 2ull);
+}
+
+// Free energies, filling and decision of a visit from its nodes' results (DL
+// lanes of a warp, one per node; `on` is false for lanes beyond the last visit).
+template <typename T, RsMode kMode, int DL>
+__device__ __forceinline__ void rs_decide(const StageArgs& a, const StageVar& v, const RsVisit& h, const RsTerms& w,
+                                          const RsOut<T>* out, int lane, bool on) {
+    const Model& m = a.m;
+    const double* so = v.S_in + 3 * (int64_t)h.site;
+    const double invT = 1.0 / m.T;
+    const double dx = w.sn[0] - so[0], dy = w.sn[1] - so[1], dz = w.sn[2] - so[2];
+    const double oo = so[0] * so[0] + so[1] * so[1] + so[2] * so[2];
+    const double nn = w.sn[0] * w.sn[0] + w.sn[1] * w.sn[1] + w.sn[2] * w.sn[2];
+    double Lo = 0.0, Th = 0.0, dL = 0.0, dT = 0.0, ce = 0.0, cc = 0.0;
+    const bool fine = on && h.cls >= 0;
+    if (fine) {
+        const FermiNodes& f = RsFermi<T>::tab(h.cls);
+        ce = f.e;
+        cc = f.c;
+        if (lane < f.M) {
+            const RsOut<T>& r = out[lane];
+            const double s = 1.0 / (m.T * f.y[lane]);
+            const T dd = T(-m.lam * dx * s), jx = T(m.JH * dx * s), jy = T(m.JH * dy * s), jz = T(m.JH * dz * s);
+            const auto p00 = mk(r.P[0], r.P[1]), p01 = mk(r.P[2], r.P[3]), p10 = mk(r.P[4], r.P[5]), p11 = mk(r.P[6], r.P[7]);
+            const auto g = rs_det_g(p00, p01, p10, p11);
+            const auto gn = rs_det_g(mk(p00.x + dd + jz, p00.y), mk(p01.x + jx, p01.y - jy), mk(p10.x + jx, p10.y + jy),
+                                     mk(p11.x + dd - jz, p11.y));
+            const T q = (g.x + g.x) + (g.x * g.x + g.y * g.y), qn = (gn.x + gn.x) + (gn.x * gn.x + gn.y * gn.y);
+            // det_new / det_old = 1 + z, with det_new - det_old formed from the
+            // change of the block (no cancellation between the two determinants)
+            const auto zero = mk(T(0.f), T(0.f));
+            const T ax = dd + jz, bx = dd - jz;
+            auto num = cfma(p11, mk(ax, T(0.f)), cfma(p00, mk(bx, T(0.f)), zero));
+            num = cfms(p01, mk(jx, jy), num);
+            num = cfms(p10, mk(jx, -jy), num);
+            // (P + i): the i of the two diagonal entries; minus det of the change
+            num = mk(num.x + ax * bx - (jx * jx + jy * jy), num.y + ax + bx);
+            const T gr = T(1.f) + g.x, rq = rs_rcp(gr * gr + g.y * g.y);
+            // z = num / det_old, det_old = -(1 + g)
+            const auto z = cfms(num, mk(gr * rq, -(g.y * rq)), zero);
+            const T zq = (z.x + z.x) + (z.x * z.x + z.y * z.y);
+            const double dl = zq < T(1.f) && T(-0.5f) < zq ? 0.5 * (double)rs_log1p(zq)
+                                                           : 0.5 * ((double)rs_log1p(qn) - (double)rs_log1p(q));
+            const double t0 = (double)rs_phase(g.y, T(1.f) + g.x), t1 = (double)rs_phase(gn.y, T(1.f) + gn.x);
+            Lo = f.a[lane] * (r.lnd + 0.5 * (double)rs_log1p(q));
+            Th = f.b[lane] * (r.th + t0);
+            dL = f.a[lane] * dl;
+            dT = f.b[lane] * (t1 - t0);
+        }
+    }
+#pragma unroll
+    for (int o = DL / 2; o > 0; o >>= 1) {
+        Lo += __shfl_xor_sync(FULL_MASK, Lo, o);
+        Th += __shfl_xor_sync(FULL_MASK, Th, o);
+        dL += __shfl_xor_sync(FULL_MASK, dL, o);
+        dT += __shfl_xor_sync(FULL_MASK, dT, o);
+    }
+    if (lane != 0 || !on) return;
+    const double dx1 = 2.0 * m.lam * dx * invT;
+    // d(d^2 + J^2 |v|^2) of the site's two rows, d = mu - e0 - lam v_x
+    const double mus = m.mu - m.e0, d0 = mus - m.lam * so[0], d1 = mus - m.lam * w.sn[0];
+    const double dx2 = 2.0 * (d1 * d1 - d0 * d0 + m.JH * m.JH * (nn - oo)) * invT * invT;
+    const double Fo = -m.T * (h.n * (0.69314718055994530942 + cc) + 0.5 * ce * w.x2 + Lo - 0.5 * w.x1) + w.cl;
+    double dF = -m.T * (0.5 * ce * dx2 + dL - 0.5 * dx1);
+    if (m.cls_on) dF += m.ca * (nn - oo) + m.cb * dx;
+    const double fo = 0.5 * h.n - Th;
+    rs_commit<kMode>(a, v, h, w, fine, Fo, dF, fo, fo - dT);
+}
+
+// A window beyond the last node class (fields thousands of T long): both
+// matrices reduced and solved in FP64 by the CTA, the matrix in its global
+// re-solve slot.  Reached only by configurations that a caller sets far from
+// any the chain visits, so plain: one thread per row, no blocking.
+inline size_t rs_exact_bytes(int n) { return (size_t)n * 48 + ((size_t)n * 12 > 512 ? (size_t)n * 12 : 512); }
+__device__ __noinline__ void rs_exact(const StageArgs& a, const StageVar& v, const RsVisit& h, RsTerms& w,
+                                      unsigned char* smem) {
+    const int n = h.n, tid = threadIdx.x, nt = blockDim.x;
+    double2* vk = reinterpret_cast<double2*>(smem);
+    double2* p = vk + n;
+    double* d = reinterpret_cast<double*>(p + n);
+    double* e2 = d + n;
+    double* sp = e2 + n;                // window spins (12 n bytes); later the block sums
+    double2* A = a.gA + (int64_t)blockIdx.x * a.gA_stride;
+    const Model& m = a.m;
+    const Window win = make_window(m, h.site);
+    double F[2], fill[2];
+    for (int var = 0; var < 2; ++var) {
+        __syncthreads();
+        build_cluster<double>(m, win, v.S_in, var ? w.sn : nullptr, sp, A);
+        __syncthreads();
+        const double cl = window_classical(m, sp, n / 2);
+        __syncthreads();
+        for (int k = 0; k < n; ++k) {
+            const int q = n - 1 - k;     // order of the trailing block
+            double s = 0.0;
+            for (int i = tid; i < q; i += nt) {
+                vk[i] = A[tri(k + 1 + i) + k];
+                s += cabs2(vk[i]);
+            }
+            __syncthreads();
+            const double s2 = block_sum<double>(s, sp);
+            if (tid == 0) {
+                d[k] = A[tri(k) + k].x;
+                if (q > 0) e2[k] = s2;
+            }
+            if (q < 2 || !(s2 > 0.0)) { __syncthreads(); continue; }
+            double2 first;
+            double tau;
+            reflector_head<double>(s2, vk[0], first, tau);
+            __syncthreads();
+            if (tid == 0) vk[0] = first;
+            __syncthreads();
+            s = 0.0;
+            for (int i = tid; i < q; i += nt) {
+                double2 r = make_double2(0.0, 0.0);
+                for (int j = 0; j < q; ++j) {
+                    if (j <= i) r = cfma(A[tri(k + 1 + i) + k + 1 + j], vk[j], r);
+                    else r = cfma_conj_a(A[tri(k + 1 + j) + k + 1 + i], vk[j], r);
+                }
+                r.x *= tau; r.y *= tau;
+                p[i] = r;
+                s += vk[i].x * r.x + vk[i].y * r.y;
+            }
+            const double K = 0.5 * tau * block_sum<double>(s, sp + 32);
+            for (int i = tid; i < q; i += nt) p[i] = make_double2(p[i].x - K * vk[i].x, p[i].y - K * vk[i].y);
+            __syncthreads();
+            for (int i = tid; i < q; i += nt)
+                for (int j = 0; j <= i; ++j) {
+                    double2& x = A[tri(k + 1 + i) + k + 1 + j];
+                    x = cfms_conj_b(p[i], vk[j], cfms_conj_b(vk[i], p[j], x));
+                }
+            __syncthreads();
+        }
+        __syncthreads();
+        double lo = 1e300, hi = -1e300, em = 0.0;
+        for (int i = 0; i < n; ++i) {
+            const double el = i > 0 ? sqrt(e2[i - 1]) : 0.0, er = i < n - 1 ? sqrt(e2[i]) : 0.0;
+            lo = fmin(lo, d[i] - el - er);
+            hi = fmax(hi, d[i] + el + er);
+            if (i < n - 1) em = fmax(em, e2[i]);
+        }
+        const double nrm = fmax(fabs(lo), fabs(hi)), pad = 1e-12 * (hi - lo + nrm) + 1e-300;
+        double sf = 0.0, sn = 0.0;
+        for (int k = tid; k < n; k += nt) {
+            const double lam = eig_f64(n, d, e2, k, lo - pad, hi + pad, DBL_MIN * fmax(1.0, em), nrm);
+            const double x = -(lam - (m.mu - m.e0)) / m.T;
+            sf += softplus(x);
+            sn += 1.0 / (1.0 + exp(-x));
+        }
+        __syncthreads();
+        F[var] = -m.T * block_sum<double>(sf, sp) + cl;
+        fill[var] = block_sum<double>(sn, sp + 32);
+        __syncthreads();
+    }
+    if (tid == 0) rs_commit<RS_RESOLVE>(a, v, h, w, true, F[0], F[1] - F[0], fill[0], fill[1]);
+    __syncthreads();
+}
+
+// Visits [first, first + nv) of the work list (nv <= vb <= 32), by the CTA.
+// uniform: all windows have one shape (periodic lattices), so that a warp may
+// hold nodes of several visits.
+template <class Tl, RsMode kMode>
+__device__ __forceinline__ void rs_visits(const StageArgs& a, const StageVar& v, const int32_t* list, int first, int nv,
+                                          int vb, int max_sites, bool uniform, unsigned char* smem, int* s_task) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const RsLayout lay = rs_layout<Tl>(vb, max_sites, nw, uniform);
+    RsVisit* hd = reinterpret_cast<RsVisit*>(smem);
+    RsTerms* tm = reinterpret_cast<RsTerms*>(smem + lay.terms);
+    RsOut<float>* out = reinterpret_cast<RsOut<float>*>(smem + lay.out);
+    RsSite<float>* sites = reinterpret_cast<RsSite<float>*>(smem + lay.site);
+    float* hop = reinterpret_cast<float*>(smem + lay.hop);
+    float2* buf = reinterpret_cast<float2*>(smem + lay.buf) + (size_t)(warp * Tl::NPW + lane / Tl::LPN) * Tl::NODE;
+    // Small windows: several visits per warp, so that its FP64 instructions
+    // serve them together.
+    constexpr int GL = Tl::NS == 1 ? 8 : Tl::NS <= 4 ? 16 : 32;
+    for (int k0 = warp * (32 / GL); k0 < nv; k0 += nw * (32 / GL)) {
+        const int k = k0 + lane / GL < nv ? k0 + lane / GL : nv - 1;   // lanes past the end repeat the last visit
+        const int c = list ? list[first + k] : first + k;
+        float* hk = uniform ? (k == 0 ? hop : nullptr) : hop + k * Tl::NS * Tl::NS;
+        rs_gather<float, GL>(a.m, v.S_in, c, v.sites[c], hd[k], tm[k], sites + k * max_sites, hk, Tl::NS, lane % GL);
+    }
+    if (threadIdx.x == 0) *s_task = 0;
+    __syncthreads();
+    if (warp == nw - 1 && lane < nv) {
+        // proposals and uniforms of the CTA's visits, one lane each, beside
+        // the other warps' eliminations
+        const int site = hd[lane].site;
+        double u0, u1;
+        propose(a.m, v.sweep, (uint32_t)site, v.S_in + 3 * (int64_t)site, tm[lane].sn);
+        uniform2(a.m.seed, v.sweep, (uint32_t)site, RNG_ACCEPT, u0, u1);
+        tm[lane].lnu = log(u0);
+    }
+    __syncwarp();
+    // Tasks: NPW nodes per warp, of one visit unless the windows are uniform.
+    for (;;) {
+        int task = 0;
+        if (lane == 0) task = atomicAdd(s_task, 1);
+        task = __shfl_sync(FULL_MASK, task, 0);
+        int k = 0, j = uniform ? task * Tl::NPW + lane / Tl::LPN : task;
+        for (; k < nv; ++k) {
+            const int cls = hd[k].cls, M = cls < 0 ? 0 : c_fermi[cls].M;
+            const int nt = uniform ? M : (M + Tl::NPW - 1) / Tl::NPW;
+            if (j < nt) break;
+            j -= nt;
+        }
+        bool idle = k >= nv;
+        if (__all_sync(FULL_MASK, idle)) break;
+        if (uniform) {
+            // lanes past the last node repeat the warp's first one, unrecorded
+            const int k0 = __shfl_sync(FULL_MASK, k, 0), j0 = __shfl_sync(FULL_MASK, j, 0);
+            if (idle) { k = k0; j = j0; }
+        } else {
+            const int M = c_fermi[hd[k].cls].M;
+            j = j * Tl::NPW + lane / Tl::LPN;
+            idle = j >= M;
+            if (idle) j = M - 1;
+        }
+        const double s = 1.0 / (a.m.T * c_fermi[hd[k].cls].y[j]);
+        RsOut<float> spare;
+        RsNode<Tl>::run(hd[k], sites + k * max_sites, hop + (uniform ? 0 : k * Tl::NS * Tl::NS), (float)s, (float)(a.m.t * s), buf,
+                        lane, idle ? &spare : out + k * kFermiOut + j);
+    }
+    __syncthreads();
+    constexpr int DL = Tl::NS <= 4 ? 16 : 32;
+    const bool half = DL == 16 && uniform;   // 16 lanes per visit hold the nodes of the classes up to |x| = 1024
+    if (half) {
+        bool wide = false;
+        for (int k = 0; k < nv; ++k) wide |= hd[k].cls >= 0 && c_fermi[hd[k].cls].M > 16;
+        if (!wide) {
+            for (int k0 = 2 * warp; k0 < nv; k0 += 2 * nw) {
+                const int k = k0 + lane / 16;
+                const bool on = k < nv;
+                rs_decide<float, kMode, 16>(a, v, hd[on ? k : nv - 1], tm[on ? k : nv - 1], out + (on ? k : nv - 1) * kFermiOut,
+                                            lane & 15, on);
+            }
+            return;
+        }
+    }
+    for (int k = warp; k < nv; k += nw) rs_decide<float, kMode, 32>(a, v, hd[k], tm[k], out + k * kFermiOut, lane, true);
+}
+
+// One visit by a thread-block cluster of node groups: node j goes to
+// group j mod (groups of the cluster), results to the first CTA.
+template <typename T, class Gp> struct RsGroupLayout { size_t terms, out, site, hop, buf, total; };
+template <typename T, class Gp> __host__ __device__ inline RsGroupLayout<T, Gp> rs_group_layout(int max_sites, int max_layer, int groups) {
+    RsGroupLayout<T, Gp> L;
+    size_t o = align16(sizeof(RsVisit));
+    L.terms = o; o = align16(o + sizeof(RsTerms));
+    L.out = o;   o = align16(o + kFermiMaxNodes * sizeof(RsOut<T>));
+    L.site = o;  o = align16(o + (size_t)max_sites * sizeof(RsSite<T>));
+    L.hop = o;   o = align16(o + (size_t)max_layer * max_layer * sizeof(T));
+    L.buf = o;   o = align16(o + (size_t)groups * sizeof(typename RsGroup<T, Gp>::Smem));
+    L.total = o;
+    return L;
+}
+
+template <typename T, class Gp, RsMode kMode>
+__device__ __forceinline__ void rs_visit_groups(const StageArgs& a, const StageVar& v, int c, int max_sites, int max_layer,
+                                                unsigned char* smem) {
+    namespace cg = cooperative_groups;
+    const cg::cluster_group cl = cg::this_cluster();
+    const int size = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, groups = blockDim.x / Gp::TPN;
+    const int g = threadIdx.x / Gp::TPN, t = threadIdx.x % Gp::TPN;
+    const auto lay = rs_group_layout<T, Gp>(max_sites, max_layer, groups);
+    RsVisit& h = *reinterpret_cast<RsVisit*>(smem);
+    RsTerms& tm = *reinterpret_cast<RsTerms*>(smem + lay.terms);
+    RsOut<T>* out = reinterpret_cast<RsOut<T>*>(smem + lay.out);
+    RsSite<T>* sites = reinterpret_cast<RsSite<T>*>(smem + lay.site);
+    T* hop = reinterpret_cast<T*>(smem + lay.hop);
+    auto& sm = reinterpret_cast<typename RsGroup<T, Gp>::Smem*>(smem + lay.buf)[g];
+    if (warp == 0) rs_gather<T, 32>(a.m, v.S_in, c, v.sites[c], h, tm, sites, hop, max_layer, lane);
+    __syncthreads();
+    // Nodes of this group, then (one thread of the first CTA's last group, which
+    // has the fewest) the proposal.
+    RsOut<T>* const out0 = size > 1 ? cl.map_shared_rank(out, 0) : out;
+    if (h.cls >= 0) {
+        const FermiNodes& f = RsFermi<T>::tab(h.cls);
+        for (int j = (size - 1 - rank) + size * g; j < f.M; j += size * groups) {
+            const double s = 1.0 / (a.m.T * f.y[j]);
+            RsGroup<T, Gp>::run(h, sites, hop, max_layer, T(s), T(a.m.t * s), sm, t, 1 + g, out0 + j);
+        }
+    }
+    if (rank == 0 && threadIdx.x == blockDim.x - 1) {
+        double u0, u1;
+        propose(a.m, v.sweep, (uint32_t)h.site, v.S_in + 3 * (int64_t)h.site, tm.sn);
+        uniform2(a.m.seed, v.sweep, (uint32_t)h.site, RNG_ACCEPT, u0, u1);
+        tm.lnu = log(u0);
+    }
+    if (size > 1) cl.sync();
+    else __syncthreads();
+    if (rank != 0) return;
+    if constexpr (kMode == RS_RESOLVE) {
+        if (h.cls < 0) {
+            rs_exact(a, v, h, tm, smem + lay.out);
+            return;
+        }
+    }
+    if (warp == 0) rs_decide<T, kMode, 32>(a, v, h, tm, out, lane, true);
+}
+
+}  // namespace ptca
