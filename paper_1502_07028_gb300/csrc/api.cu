@@ -647,7 +647,7 @@ static bool on_determinants(const ptca_ctx* ctx) {
 
 // Stages of at most this many visits run the latency-bound form: a group of
 // threads per node instead of one warp.
-static bool few_visits(const ptca_ctx* ctx) { return ctx->max_stage <= 128; }
+static bool few_visits(const ptca_ctx* ctx) { return ctx->max_stage <= 64; }
 
 // A stage launch and a re-solve launch in the context's configuration
 // (shared-memory kernels, or the large-cluster kernels).
@@ -695,7 +695,7 @@ static cudaError_t check_stage(ptca_ctx* ctx, const StageArgs& a, int s, cudaStr
             if (e == cudaSuccess) e = ptca::launch_check(0, a, c0, cnt, e64, ld, F64, ctx->resolve_grid, st);
         }
         // the free energies that the sweep decides on
-        if (e == cudaSuccess && on_determinants(ctx)) e = ptca::launch_check_resolvent(a, few_visits(ctx), c0, cnt, F32, st);
+        if (e == cudaSuccess && on_determinants(ctx)) e = ptca::launch_check_resolvent(a, few_visits(ctx), c0, cnt, F32, ctx->sms, st);
         if (e == cudaSuccess)
             e = ptca::launch_check_compare(a.m, a.sites + c0, cnt, e32, e64, ld, F32, F64, ctx->d_chk_out + ptca::kCheckCols * s, st);
     }

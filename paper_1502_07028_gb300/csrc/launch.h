@@ -124,16 +124,20 @@ cudaError_t launch_observables(const double* S, int Lx, int Ly, const double* re
                                const uint8_t* rec_acc, const int32_t* rec_n, int N, double* out, cudaStream_t st);
 
 
-// Stage kernels on determinants (kernels_resolvent.cu, PTCA_MIXED): whether
-// the problem's windows and temperature fit them, and a stage launch.
+// Stage kernels on determinants (kernels_resolvent*.cu, PTCA_MIXED): whether
+// the problem's windows and temperature fit them, and a stage launch.  few:
+// stages too small to fill the GPU (the same for every launch of a context, since
+// the two forms round differently).
 bool resolvent_supported(const Model& m);
 cudaError_t configure_resolvent_kernels(size_t smem_limit);
-// few: stages too small to fill the GPU (the same for every launch of a context,
-// since the two forms round differently).
+cudaError_t configure_resolvent_groups(size_t smem_limit);
 cudaError_t launch_stage_resolvent(const StageArgs& a, bool few, int sms, cudaStream_t st);
 // Their free energies of visits c0 .. c0 + count - 1 for the checker (F[2k],
 // F[2k + 1] of visit c0 + k), and the double-float re-solve.
-cudaError_t launch_check_resolvent(const StageArgs& a, bool few, int c0, int count, double* F, cudaStream_t st);
+cudaError_t launch_check_resolvent(const StageArgs& a, bool few, int c0, int count, double* F, int sms,
+                                   cudaStream_t st);
 cudaError_t launch_resolve_resolvent(const StageArgs& a, int sms, cudaStream_t st);
+enum RsMode : int;
+cudaError_t launch_groups(RsMode mode, const StageArgs& a, int c0, cudaStream_t st);
 
 }  // namespace ptca

@@ -23,6 +23,13 @@
 // reduction of each of the two matrices (n = B L): 0.10 M against 5.6 M at
 // n = 128, times 13 nodes at |x| <= 512.
 //
+// Short rings pay three products per layer for little.  Where every bond joins
+// sites of opposite parity the parity that the update site does not have can
+// go first: its 2x2 pivots are independent, and what is left is a dense matrix of
+// half the order, done as two blocks with two inversions and two products
+// (RsPairs).  It is taken on rings of four layers (4x4 and 4x4x4 clusters):
+// 4 b^3 multiply-adds instead of 9 b^3.
+//
 // One node is eliminated by LPN lanes of a warp, which holds 32 / LPN nodes: the
 // larger the tile per lane, the fewer shuffles and loads per multiply-add.
 // Lane (r, c) of a GR x GC grid holds the rows of sites r + GR i and the columns of
@@ -68,7 +75,13 @@ __device__ __forceinline__ void st2(dfl2* p, dfl2 a, dfl2 b) { p[0] = a; p[1] = 
 
 // Scalar helpers of the two arithmetics.
 __device__ __forceinline__ float rs_rcp(float x) { return __fdividef(1.f, x); }
-__device__ __forceinline__ dfl rs_rcp(dfl x) { return dfl(1.f, 0.f) / x; }
+// Newton correction r (1 + e + e^2) of the FP32 reciprocal, e = 1 - x r from one
+// fused multiply-add each for the two parts of x: relative error a few 2^-48.
+__device__ __forceinline__ dfl rs_rcp(dfl x) {
+    const float r = __fdividef(1.f, x.hi);
+    const float e = __fmaf_rn(-x.lo, r, __fmaf_rn(-x.hi, r, 1.f));
+    return fast_two_sum(r, r * __fmaf_rn(e, e, e));
+}
 __device__ __forceinline__ float rs_log1p(float q) { return log1pf(q); }
 __device__ __forceinline__ double rs_log1p(dfl q) { return log1p(double(q)); }
 __device__ __forceinline__ float rs_phase(float y, float x) { return atan2f(y, x); }
@@ -117,6 +130,16 @@ struct RsVisit {
     int c, site, n, L, ns, u, us;   // stage index, lattice site, order, layers, sites per layer, update layer and site
     int per, cls;                   // cluster periodic; node class (-1: |x| beyond the last class)
 };
+// A window split by parity: kept sites (of the update site's parity) in two
+// blocks, block 1 ending with the update site; eliminated sites; for each kept
+// site the set of its eliminated neighbours.
+struct RsPairs {
+    int na, nb, ne;                 // sites of block 0, of block 1, eliminated
+    int kept[32], gone[32];         // window sites (layer order); kept: block 0, then block 1
+    uint32_t near[32];
+};
+constexpr int kPairSites = 64;      // largest window
+
 // Sums over the window, FP64.
 struct RsTerms { double x1, x2, cl, sn[3], lnu; };
 
@@ -127,7 +150,8 @@ template <int GR_, int GC_, int SR_, int SC_, int MAXT_, int MINB_> struct RsTil
     static constexpr int LPN = GR * GC, NPW = 32 / LPN;
     // Elements of a node's buffers: padded so that the nodes of a warp start in
     // different banks.
-    static constexpr int NODE = 3 * B * RS + (NPW == 1 ? 0 : LPN >= 16 ? 8 : LPN > 1 ? 2 * LPN : 2);
+    static constexpr int PAD = NPW == 1 ? 0 : LPN >= 16 ? 8 : LPN > 1 ? 2 * LPN : 2;
+    static constexpr int node(bool pairs) { return (pairs ? 2 * B * RS + 8 * NS : 3 * B * RS) + PAD; }
     static_assert(GR * SR == GC * SC && GR % GC == 0 && 32 % LPN == 0, "square blocks");
 };
 using RsT1 = RsTile<1, 1, 1, 1, 256, 2>;    // chains: a node per lane
@@ -322,6 +346,148 @@ template <class Tl> struct RsNode {
         }
     }
 
+    // o = P^t Q with P^t the block transpose of P (2x2 blocks stay as they are)
+    static __device__ __forceinline__ void mul_t(Tile& o, const V* P, const V* Q, int ns, int r, int c) {
+#pragma unroll
+        for (int i = 0; i < 2 * SR; ++i)
+#pragma unroll
+            for (int j = 0; j < 2 * SC; ++j) o[i][j] = make_float2(0.f, 0.f);
+#pragma unroll 2
+        for (int k = 0; k < ns; ++k) {
+            V p[2 * SR][2];
+#pragma unroll
+            for (int i = 0; i < 2 * SR; ++i) ld2(P + ((i / SR) * NS + k) * RS + 2 * (r + GR * (i % SR)), p[i][0], p[i][1]);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                const V* q = Q + (h * NS + k) * RS;
+                V b[2 * SC];
+#pragma unroll
+                for (int j = 0; j < SC; ++j) ld2(q + 2 * csite(c, j), b[j], b[SC + j]);
+#pragma unroll
+                for (int i = 0; i < 2 * SR; ++i)
+#pragma unroll
+                    for (int j = 0; j < 2 * SC; ++j) o[i][j] = cfma(p[i][h], b[j], o[i][j]);
+            }
+        }
+    }
+
+    // Block (row0, col0) of the kept sites' matrix after the eliminated parity:
+    // on-site terms (without i) minus t'^2 times the pivot inverses of common
+    // neighbours (inv: 4 elements per eliminated site).
+    static __device__ __forceinline__ void pair_block(Tile& a, const RsPairs& pt, int row0, int nr, int col0, int nc,
+                                                      const RsSite<float>* site, const V* inv, float s, float tt, int r, int c) {
+#pragma unroll 1
+        for (int i = 0; i < SR; ++i)
+#pragma unroll 1
+            for (int j = 0; j < SC; ++j) {
+                const int x = r + GR * i, y = csite(c, j);
+                V uu = make_float2(0.f, 0.f), ud = uu, du = uu, dd = uu;
+                if (x < nr && y < nc) {
+                    uint32_t both = pt.near[row0 + x] & pt.near[col0 + y];
+                    while (both) {
+                        const int e = __ffs(both) - 1;
+                        both &= both - 1;
+                        V p, q;
+                        ld2(inv + 4 * e, p, q);
+                        uu = csub(uu, p);
+                        ud = csub(ud, q);
+                        ld2(inv + 4 * e + 2, p, q);
+                        du = csub(du, p);
+                        dd = csub(dd, q);
+                    }
+                    uu = make_float2(tt * uu.x, tt * uu.y);
+                    ud = make_float2(tt * ud.x, tt * ud.y);
+                    du = make_float2(tt * du.x, tt * du.y);
+                    dd = make_float2(tt * dd.x, tt * dd.y);
+                    if (row0 + x == col0 + y) {
+                        const RsSite<float> o = site[pt.kept[row0 + x]];
+                        uu.x += (o.d + o.z) * s;
+                        dd.x += (o.d - o.z) * s;
+                        ud = make_float2(ud.x + o.x * s, ud.y - o.y * s);
+                        du = make_float2(du.x + o.x * s, du.y + o.y * s);
+                    }
+                }
+#pragma unroll
+                for (int k = 0; k < SR; ++k)
+#pragma unroll
+                    for (int l = 0; l < SC; ++l)
+                        if (k == i && l == j) {
+                            a[k][l] = uu;
+                            a[k][SC + l] = ud;
+                            a[SR + k][l] = du;
+                            a[SR + k][SC + l] = dd;
+                        }
+            }
+    }
+
+    static __device__ __forceinline__ void finish(const Tile& a, int us, RsSum<float>& lnd, RsSum<float>& th, int r, int c,
+                                                  int nl, RsOut<float>* out) {
+        // last pivot block: the lane holding rows and columns of the update site
+#pragma unroll
+        for (int i = 0; i < SR; ++i)
+#pragma unroll
+            for (int j = 0; j < SC; ++j)
+                if (r + GR * i == us && csite(c, j) == us) {
+                    out->P[0] = a[i][j].x; out->P[1] = a[i][j].y;
+                    out->P[2] = a[i][SC + j].x; out->P[3] = a[i][SC + j].y;
+                    out->P[4] = a[SR + i][j].x; out->P[5] = a[SR + i][j].y;
+                    out->P[6] = a[SR + i][SC + j].x; out->P[7] = a[SR + i][SC + j].y;
+                }
+#pragma unroll
+        for (int o = Tl::LPN / 2; o > 0; o >>= 1) {
+            lnd.merge(o);
+            th.merge(o);
+        }
+        if (nl == 0) {
+            out->lnd = 0.5 * lnd.value();
+            out->th = th.value();
+        }
+        __syncwarp();
+    }
+
+    // run() for a window split by parity.
+    static __device__ __forceinline__ void run_pairs(const RsPairs& pt, const RsSite<float>* site, float s, float tp, V* buf,
+                                                     int lane, RsOut<float>* out) {
+        const int base = lane & ~(Tl::LPN - 1), nl = lane - base;
+        const int r = nl / GC, c = nl % GC;
+        const float tt = tp * tp;
+        V *X = buf, *C = buf + Tl::B * RS, *inv = C + Tl::B * RS;
+        RsSum<float> lnd, th;
+        for (int e = nl; e < pt.ne; e += Tl::LPN) {
+            const RsSite<float> o = site[pt.gone[e]];
+            const V p00 = make_float2((o.d + o.z) * s, 0.f), p11 = make_float2((o.d - o.z) * s, 0.f);
+            const V p01 = make_float2(o.x * s, -(o.y * s)), p10 = make_float2(o.x * s, o.y * s);
+            const V g = rs_det_g(p00, p01, p10, p11);
+            const float gr = 1.f + g.x, rq = rs_rcp(gr * gr + g.y * g.y);
+            const V w = make_float2(-(gr * rq), g.y * rq), wn = make_float2(-w.x, -w.y);
+            st2(inv + 4 * e, cmulp(make_float2(p11.x, 1.f), w), cmulp(p01, wn));
+            st2(inv + 4 * e + 2, cmulp(p10, wn), cmulp(make_float2(p00.x, 1.f), w));
+            lnd.add(log1pf((g.x + g.x) + (g.x * g.x + g.y * g.y)));
+            th.add(atan2f(g.y, 1.f + g.x));
+        }
+        __syncwarp();
+        Tile a, S;
+        pair_block(a, pt, 0, pt.na, 0, pt.na, site, inv, s, tt, r, c);
+#pragma unroll 1
+        for (int o = 0;; ++o) {
+            invert(a, lnd, th, o == 0 ? -1 : pt.nb - 1, o == 0 ? pt.na : pt.nb, r, c, nl, base);
+            if (o) break;
+            store(X, a, r, c);
+            pair_block(a, pt, 0, pt.na, pt.na, pt.nb, site, inv, s, tt, r, c);
+            store(C, a, r, c);
+            pair_block(S, pt, pt.na, pt.nb, pt.na, pt.nb, site, inv, s, tt, r, c);
+            __syncwarp();
+            mul(a, X, C, pt.na, r, c);
+            put(X, a, 1.f, r, c);
+            mul_t(a, C, X, pt.na, r, c);
+#pragma unroll
+            for (int i = 0; i < 2 * SR; ++i)
+#pragma unroll
+                for (int j = 0; j < 2 * SC; ++j) a[i][j] = csub(S[i][j], a[i][j]);
+        }
+        finish(a, pt.nb - 1, lnd, th, r, c, nl, out);
+    }
+
     // One node of one visit: the sums over all pivots but the update site's,
     // and that site's last pivot block.  s: 1 / (T y), tp: t / (T y).
     static __device__ __forceinline__ void run(const RsVisit& v, const RsSite<float>* site, const float* hop, float s, float tp,
@@ -407,27 +573,7 @@ template <class Tl> struct RsNode {
                 __syncwarp();
             }
         }
-        // last pivot block: the lane holding rows and columns of the update site
-#pragma unroll
-        for (int i = 0; i < SR; ++i)
-#pragma unroll
-            for (int j = 0; j < SC; ++j)
-                if (r + GR * i == v.us && csite(c, j) == v.us) {
-                    out->P[0] = a[i][j].x; out->P[1] = a[i][j].y;
-                    out->P[2] = a[i][SC + j].x; out->P[3] = a[i][SC + j].y;
-                    out->P[4] = a[SR + i][j].x; out->P[5] = a[SR + i][j].y;
-                    out->P[6] = a[SR + i][SC + j].x; out->P[7] = a[SR + i][SC + j].y;
-                }
-#pragma unroll
-        for (int o = Tl::LPN / 2; o > 0; o >>= 1) {
-            lnd.merge(o);
-            th.merge(o);
-        }
-        if (nl == 0) {
-            out->lnd = 0.5 * lnd.value();
-            out->th = th.value();
-        }
-        __syncwarp();
+        finish(a, v.us, lnd, th, r, c, nl, out);
     }
 };
 
@@ -458,8 +604,9 @@ template <typename T, class Gp> struct RsGroup {
     static constexpr int GR = Gp::GR, GC = Gp::GC, R = Gp::R, C = Gp::C, RS = Gp::RS;
     using Tile = V[R][C];
     // Shared memory of a group: three matrices, two broadcast buffers of a pivot
-    // row and column, the pivots of a layer.
-    struct Smem { V X[Gp::B * RS], C[Gp::B * RS], E[Gp::B * RS], row[2][Gp::B], col[2][Gp::B], piv[Gp::B]; };
+    // row and column; the node's pivots follow (bytes() with n of them).
+    struct Smem { V X[Gp::B * RS], C[Gp::B * RS], E[Gp::B * RS], row[2][Gp::B], col[2][Gp::B]; };
+    static __host__ __device__ constexpr size_t bytes(int n) { return sizeof(Smem) + (size_t)n * sizeof(V); }
 
     static __device__ __forceinline__ void sync(int id) {
         if constexpr (Gp::TPN == 32) __syncwarp();
@@ -474,7 +621,7 @@ template <typename T, class Gp> struct RsGroup {
                 if (x < b && y < b) M[x * RS + y] = mk(f * a[i][j].x, f * a[i][j].y);
             }
     }
-    static __device__ __forceinline__ void mul(Tile& o, const V* P, const V* Q, int b, int r, int c) {
+    static __device__ __forceinline__ void mul(Tile& o, const V* P, const V* Q, int b, int bc, int r, int c) {
 #pragma unroll
         for (int i = 0; i < R; ++i)
 #pragma unroll
@@ -487,7 +634,7 @@ template <typename T, class Gp> struct RsGroup {
             for (int i = 0; i < R; ++i) p[i] = P[(r + GR * i < b ? r + GR * i : b - 1) * RS + k];
 #pragma unroll
             for (int j = 0; j < C; ++j) {
-                const V q = Q[k * RS + (c + GC * j < b ? c + GC * j : b - 1)];
+                const V q = Q[k * RS + (c + GC * j < bc ? c + GC * j : bc - 1)];
 #pragma unroll
                 for (int i = 0; i < R; ++i) o[i][j] = cfma(p[i], q, o[i][j]);
             }
@@ -516,8 +663,8 @@ template <typename T, class Gp> struct RsGroup {
             }
     }
     // Gauss-Jordan inversion in place of a + i; rows 2 skip and 2 skip + 1 are
-    // left out.  The pivots go to sm.piv (without their i).
-    static __device__ __forceinline__ void invert(Tile& a, Smem& sm, int skip, int b, int r, int c, int id) {
+    // left out.  The pivots go to piv (without their i).
+    static __device__ __forceinline__ void invert(Tile& a, Smem& sm, V* piv, int skip, int b, int r, int c, int id) {
 #pragma unroll 1
         for (int p = 0; p < b; ++p) {
             if ((p >> 1) == skip) continue;
@@ -532,7 +679,7 @@ template <typename T, class Gp> struct RsGroup {
                 }
             sync(id);
             const V pv = row[p];
-            if (r == 0 && c == 0) sm.piv[p] = pv;
+            if (r == 0 && c == 0) piv[p] = pv;
             const T im = pv.y + T(1.f), rq = rs_rcp(pv.x * pv.x + im * im);
             const V w = mk(pv.x * rq, -(im * rq));     // 1/(pivot + i)
             const V zero = mk(T(0.f), T(0.f));
@@ -554,6 +701,7 @@ template <typename T, class Gp> struct RsGroup {
 
     static __device__ __forceinline__ void run(const RsVisit& v, const RsSite<T>* site, const T* hop, int hs, T s, T tp,
                                                Smem& sm, int t, int id, RsOut<T>* out) {
+        V* const piv = reinterpret_cast<V*>(&sm + 1);
         const int r = t / GC, c = t % GC, L = v.L, ns = v.ns, b = 2 * ns;
         const bool ring = v.per && L >= 3;
         const T tt = tp * tp, tau2 = (v.per && L == 2) ? T(4.f) * tt : tt, one = T(1.f);
@@ -574,15 +722,9 @@ template <typename T, class Gp> struct RsGroup {
                 else l = o < v.u ? o : L - 1 - (o - v.u);
                 layer(a, site + l * ns, hop, hs, s, tt, b, r, c, o > 0 && (v.per || o != v.u));
             }
-            invert(a, sm, last ? v.us : -1, b, r, c, id);
-            sync(id);
-            for (int p = t; p < b; p += Gp::TPN)
-                if (!(last && (p >> 1) == v.us)) {
-                    const V pv = sm.piv[p];
-                    lnd.add(rs_log1p((pv.y + pv.y) + (pv.x * pv.x + pv.y * pv.y)));
-                    th.add(rs_phase(-pv.x, one + pv.y));
-                }
+            invert(a, sm, piv + o * b, last ? v.us : -1, b, r, c, id);
             if (last) break;
+            sync(id);
             if (ring && o > 0) {
                 if (o == L - 2 && t < b) {
                     sm.C[t * RS + t].x = sm.C[t * RS + t].x - one;
@@ -591,17 +733,17 @@ template <typename T, class Gp> struct RsGroup {
                 store(sm.X, a, one, b, r, c);
                 sync(id);
                 Tile w;
-                mul(w, sm.E, sm.X, b, r, c);
+                mul(w, sm.E, sm.X, b, b, r, c);
                 sync(id);
                 store(sm.E, w, -tp, b, r, c);
                 sync(id);
-                mul(w, sm.E, sm.C, b, r, c);
+                mul(w, sm.E, sm.C, b, b, r, c);
 #pragma unroll
                 for (int i = 0; i < R; ++i)
 #pragma unroll
                     for (int j = 0; j < C; ++j) S[i][j] = mk(S[i][j].x + tp * w[i][j].x, S[i][j].y + tp * w[i][j].y);
                 if (o < L - 2) {
-                    mul(w, sm.X, sm.C, b, r, c);
+                    mul(w, sm.X, sm.C, b, b, r, c);
                     sync(id);
                     store(sm.C, w, -tp, b, r, c);
                 }
@@ -620,25 +762,155 @@ template <typename T, class Gp> struct RsGroup {
                 sync(id);
             }
         }
+        finish(a, sm, piv, b * L, b * (L - 1) + 2 * v.us, v.us, lnd, th, r, c, t, id, out);
+    }
+
+    // o = P^t Q with P^t the block transpose of P (2x2 blocks stay as they are)
+    static __device__ __forceinline__ void mul_t(Tile& o, const V* P, const V* Q, int b, int nrow, int r, int c) {
+#pragma unroll
+        for (int i = 0; i < R; ++i)
+#pragma unroll
+            for (int j = 0; j < C; ++j) o[i][j] = mk(T(0.f), T(0.f));
+#pragma unroll 2
+        for (int k = 0; k < b; ++k) {
+            V p[R];
+#pragma unroll
+            for (int i = 0; i < R; ++i) {
+                const int x = r + GR * i < nrow ? r + GR * i : nrow - 1;
+                p[i] = P[((k & ~1) + (x & 1)) * RS + (x & ~1) + (k & 1)];
+            }
+#pragma unroll
+            for (int j = 0; j < C; ++j) {
+                const V q = Q[k * RS + (c + GC * j < nrow ? c + GC * j : nrow - 1)];
+#pragma unroll
+                for (int i = 0; i < R; ++i) o[i][j] = cfma(p[i], q, o[i][j]);
+            }
+        }
+    }
+    // Block of the kept sites' matrix after the eliminated parity (RsNode::pair_block).
+    static __device__ __forceinline__ void pair_block(Tile& a, const RsPairs& pt, int row0, int nr, int col0, int nc,
+                                                      const RsSite<T>* site, const V* inv, T s, T tt, int r, int c) {
+#pragma unroll
+        for (int i = 0; i < R; ++i)
+#pragma unroll
+            for (int j = 0; j < C; ++j) {
+                const int x = r + GR * i, y = c + GC * j, sx = x >> 1, sy = y >> 1;
+                V e = mk(T(0.f), T(0.f));
+                if (sx < nr && sy < nc) {
+                    uint32_t both = pt.near[row0 + sx] & pt.near[col0 + sy];
+                    const int q = 2 * (x & 1) + (y & 1);
+                    while (both) {
+                        const int k = __ffs(both) - 1;
+                        both &= both - 1;
+                        e = csub(e, inv[4 * k + q]);
+                    }
+                    e = mk(tt * e.x, tt * e.y);
+                    if (row0 + sx == col0 + sy) {
+                        const RsSite<T> o = site[pt.kept[row0 + sx]];
+                        if (x == y) e.x = e.x + ((x & 1) ? o.d - o.z : o.d + o.z) * s;
+                        else { e.x = e.x + o.x * s; e.y = e.y + ((x & 1) ? o.y * s : -(o.y * s)); }
+                    }
+                }
+                a[i][j] = e;
+            }
+    }
+    // run() for a window split by parity.
+    static __device__ __forceinline__ void run_pairs(const RsPairs& pt, const RsSite<T>* site, T s, T tp, Smem& sm, int t,
+                                                     int id, RsOut<T>* out) {
+        V* const piv = reinterpret_cast<V*>(&sm + 1);
+        const int r = t / GC, c = t % GC;
+        const T tt = tp * tp, one = T(1.f);
+        V* const inv = sm.E;
+        RsSum<T> lnd, th;
+        for (int e = t; e < pt.ne; e += Gp::TPN) {
+            const RsSite<T> o = site[pt.gone[e]];
+            const V zero = mk(T(0.f), T(0.f));
+            const V p00 = mk((o.d + o.z) * s, T(0.f)), p11 = mk((o.d - o.z) * s, T(0.f));
+            const V p01 = mk(o.x * s, -(o.y * s)), p10 = mk(o.x * s, o.y * s);
+            const V g = rs_det_g(p00, p01, p10, p11);
+            const T gr = one + g.x, rq = rs_rcp(gr * gr + g.y * g.y);
+            const V w = mk(-(gr * rq), g.y * rq);
+            inv[4 * e] = cfma(mk(p11.x, one), w, zero);
+            inv[4 * e + 1] = cfms(p01, w, zero);
+            inv[4 * e + 2] = cfms(p10, w, zero);
+            inv[4 * e + 3] = cfma(mk(p00.x, one), w, zero);
+            lnd.add(rs_log1p((g.x + g.x) + (g.x * g.x + g.y * g.y)));
+            th.add(rs_phase(g.y, one + g.x));
+        }
+        sync(id);
+        Tile a, S;
+        const int ba = 2 * pt.na, bb = 2 * pt.nb;
+        pair_block(a, pt, 0, pt.na, 0, pt.na, site, inv, s, tt, r, c);
+#pragma unroll 1
+        for (int o = 0;; ++o) {
+            invert(a, sm, piv + (o ? ba : 0), o ? pt.nb - 1 : -1, o ? bb : ba, r, c, id);
+            if (o) break;
+            store(sm.X, a, one, ba, r, c);
+            pair_block(a, pt, 0, pt.na, pt.na, pt.nb, site, inv, s, tt, r, c);
+#pragma unroll
+            for (int i = 0; i < R; ++i)
+#pragma unroll
+                for (int j = 0; j < C; ++j)
+                    if (r + GR * i < ba && c + GC * j < bb) sm.C[(r + GR * i) * RS + c + GC * j] = a[i][j];
+            pair_block(S, pt, pt.na, pt.nb, pt.na, pt.nb, site, inv, s, tt, r, c);
+            sync(id);
+            mul(a, sm.X, sm.C, ba, bb, r, c);
+            sync(id);
+#pragma unroll
+            for (int i = 0; i < R; ++i)
+#pragma unroll
+                for (int j = 0; j < C; ++j)
+                    if (r + GR * i < ba && c + GC * j < bb) sm.X[(r + GR * i) * RS + c + GC * j] = a[i][j];
+            sync(id);
+            mul_t(a, sm.C, sm.X, ba, bb, r, c);
+#pragma unroll
+            for (int i = 0; i < R; ++i)
+#pragma unroll
+                for (int j = 0; j < C; ++j) a[i][j] = csub(S[i][j], a[i][j]);
+            sync(id);
+        }
+        finish(a, sm, piv, ba + bb, ba + bb - 2, pt.nb - 1, lnd, th, r, c, t, id, out);
+    }
+
+    // Results of a node: the last pivot block, and the sums over the np pivots
+    // but the update site's two, on top of what lnd and th hold already.
+    static __device__ __forceinline__ void finish(const Tile& a, Smem& sm, const V* piv, int np, int skip, int us, RsSum<T>& lnd,
+                                                  RsSum<T>& th, int r, int c, int t, int id, RsOut<T>* out) {
+        const T one = T(1.f);
 #pragma unroll
         for (int i = 0; i < R; ++i)
 #pragma unroll
             for (int j = 0; j < C; ++j) {
                 const int x = r + GR * i, y = c + GC * j;
-                if ((x >> 1) == v.us && (y >> 1) == v.us) {
+                if ((x >> 1) == us && (y >> 1) == us) {
                     const int k = 4 * (x & 1) + 2 * (y & 1);
                     out->P[k] = a[i][j].x;
                     out->P[k + 1] = a[i][j].y;
                 }
             }
-        // rows 0 .. b - 1 were summed by the group's first threads
-        if (t < 32) {
+        sync(id);
+        // Logarithm and phase of two pivots at a time (their product against i^2
+        // has a phase within (-pi, pi)), all at the end: FP64 logarithms of a few
+        // lanes after each layer took longer than the eliminations of a chain.
+        for (int p = 2 * t; p < np; p += 2 * Gp::TPN) {
+            if (p == skip) continue;
+            const V u = piv[p], w = piv[p + 1];
+            // (1 - i u)(1 - i w) = 1 + g
+            const V g = mk(u.y + w.y - (u.x * w.x - u.y * w.y), -(u.x + w.x) - (u.x * w.y + u.y * w.x));
+            lnd.add(rs_log1p((g.x + g.x) + (g.x * g.x + g.y * g.y)));
+            th.add(rs_phase(g.y, one + g.x));
+        }
 #pragma unroll
-            for (int o = 16; o > 0; o >>= 1) { lnd.merge(o); th.merge(o); }
-            if (t == 0) {
-                out->lnd = 0.5 * lnd.value();
-                out->th = th.value();
-            }
+        for (int o = 16; o > 0; o >>= 1) { lnd.merge(o); th.merge(o); }
+        double2* part = reinterpret_cast<double2*>(sm.row[0]);   // per-warp partial sums
+        if (Gp::TPN > 32) sync(id);
+        if ((t & 31) == 0) part[t >> 5] = make_double2(lnd.value(), th.value());
+        sync(id);
+        if (t == 0) {
+            double l = part[0].x, h = part[0].y;
+            for (int k = 1; k < Gp::TPN / 32; ++k) { l += part[k].x; h += part[k].y; }
+            out->lnd = 0.5 * l;
+            out->th = h;
         }
         sync(id);
     }
@@ -653,20 +925,20 @@ struct RsLayout { size_t terms, out, site, hop, buf, total; };
 
 // kOut: nodes kept per visit.  One hopping table when all windows have one shape.
 template <class Tl>
-__host__ __device__ inline RsLayout rs_layout(int vb, int max_sites, int nw, bool uniform) {
+__host__ __device__ inline RsLayout rs_layout(int vb, int max_sites, int nw, bool uniform, bool pairs) {
     RsLayout L;
-    size_t o = align16((size_t)vb * sizeof(RsVisit));
+    size_t o = align16((size_t)vb * sizeof(RsVisit)) + (pairs ? align16(sizeof(RsPairs)) : 0);
     L.terms = o; o = align16(o + (size_t)vb * sizeof(RsTerms));
     L.out = o;   o = align16(o + (size_t)vb * kFermiOut * sizeof(RsOut<float>));
     L.site = o;  o = align16(o + (size_t)vb * max_sites * sizeof(RsSite<float>));
     L.hop = o;   o = align16(o + (size_t)(uniform ? 1 : vb) * Tl::NS * Tl::NS * sizeof(float));
-    L.buf = o;   o = align16(o + (size_t)nw * Tl::NPW * Tl::NODE * sizeof(float2));
+    L.buf = o;   o = align16(o + (size_t)nw * Tl::NPW * Tl::node(pairs) * sizeof(float2));
     L.total = o;
     return L;
 }
 
-__constant__ FermiNodes c_fermi[kFermiClasses] = {PTCA_FERMI_NODES};
-__constant__ FermiNodes c_fermi_df[kFermiClasses] = {PTCA_FERMI_NODES_DF};
+static __constant__ FermiNodes c_fermi[kFermiClasses] = {PTCA_FERMI_NODES};
+static __constant__ FermiNodes c_fermi_df[kFermiClasses] = {PTCA_FERMI_NODES_DF};
 
 // The nodes of an arithmetic: their approximation error is below its rounding.
 template <typename T> struct RsFermi {
@@ -746,28 +1018,72 @@ __device__ __forceinline__ void rs_gather(const Model& m, const double* S, int c
     }
 }
 
+// The parity split of a periodic lattice's windows (all alike), by one warp.
+// Window sites in layer order, as rs_gather places them.
+__device__ __forceinline__ void rs_pairs(const Model& m, int site, RsPairs& t, int lane) {
+    const Window win = make_window(m, site);
+    const int ext[3] = {win.ex, win.ey, win.ez}, up[3] = {win.uwx, win.uwy, win.uwz};
+    int ax = 0;
+    if (ext[1] > ext[0]) ax = 1;
+    if (ext[2] > (ax ? ext[1] : ext[0])) ax = 2;
+    const int e0 = ax == 0 ? ext[1] : ext[0], e1 = ax == 2 ? ext[1] : ext[2], e2 = ext[ax];
+    const int u0 = ax == 0 ? up[1] : up[0], u1 = ax == 2 ? up[1] : up[2], u2 = up[ax];
+    const int ns = e0 * e1, n = ns * e2, per = m.cluster_periodic;
+    const int u = u2 * ns + u1 * e0 + u0;
+    auto parity = [&](int k) { return (k % e0 + k / e0 % e1 + k / ns) & 1; };
+    auto bond = [&](int a, int b) {
+        const int d0 = abs(a % e0 - b % e0), d1 = abs(a / e0 % e1 - b / e0 % e1), d2 = abs(a / ns - b / ns);
+        const int h0 = d0 == 1 || (per && d0 == e0 - 1 && d0 > 0), h1 = d1 == 1 || (per && d1 == e1 - 1 && d1 > 0),
+                  h2 = d2 == 1 || (per && d2 == e2 - 1 && d2 > 0);
+        return (h0 && !d1 && !d2) || (h1 && !d0 && !d2) || (h2 && !d0 && !d1);
+    };
+    const int pu = parity(u);
+    // kept and eliminated sites in order, the update site last
+    int nk = 0, ne = 0;
+    for (int k0 = 0; k0 < n; k0 += 32) {
+        const int k = k0 + lane;
+        const bool in = k < n, keep = in && k != u && parity(k) == pu, drop = in && parity(k) != pu;
+        const unsigned bk = __ballot_sync(FULL_MASK, keep), bd = __ballot_sync(FULL_MASK, drop), below = (1u << lane) - 1u;
+        if (keep) t.kept[nk + __popc(bk & below)] = k;
+        if (drop) t.gone[ne + __popc(bd & below)] = k;
+        nk += __popc(bk);
+        ne += __popc(bd);
+    }
+    if (lane == 0) {
+        t.kept[nk] = u;
+        t.na = (nk + 1) / 2;
+        t.nb = nk + 1 - t.na;
+        t.ne = ne;
+    }
+    __syncwarp();
+    if (lane <= nk) {
+        uint32_t near = 0;
+        for (int e = 0; e < ne; ++e) near |= (uint32_t)bond(t.kept[lane], t.gone[e]) << e;
+        t.near[lane] = near;
+    }
+}
+
 // What a visit's free energies are for: the stage's decision, with decisions
 // near the threshold left to the re-solve; the re-solve's decision; or the
 // precision checker, which takes the two free energies alone (Fbuf[2c],
 // Fbuf[2c + 1]).
-enum RsMode { RS_STAGE, RS_RESOLVE, RS_CHECK };
+enum RsMode : int { RS_STAGE, RS_RESOLVE, RS_CHECK };
 
 // Metropolis on dF and the visit's records (one thread).  fine: the free
 // energies are valid (the window lies within the node classes).
-template <RsMode kMode>
-__device__ __forceinline__ void rs_commit(const StageArgs& a, const StageVar& v, const RsVisit& h, const RsTerms& w,
-                                          bool fine, double Fo, double dF, double fo, double fn) {
+__device__ __forceinline__ void rs_commit(RsMode mode, const StageArgs& a, const StageVar& v, const RsVisit& h,
+                                          const RsTerms& w, bool fine, double Fo, double dF, double fo, double fn) {
     const Model& m = a.m;
     const double Fn = Fo + dF;
     const double* so = v.S_in + 3 * (int64_t)h.site;
     const int c = h.c, site = h.site;
-    if constexpr (kMode == RS_CHECK) {
+    if (mode == RS_CHECK) {
         if (fine) { a.Fbuf[2 * c] = Fo; a.Fbuf[2 * c + 1] = Fn; }
         return;
     }
     if (fine && !isfinite(dF)) atomicExch(a.err, 1);
     const double dFe = stage2_dF(a, c, dF);
-    if constexpr (kMode == RS_STAGE) {
+    if (mode == RS_STAGE) {
         // near the threshold, or a window beyond the last node class
         if (!fine || (a.margin > 0.0 && fabs(w.lnu + dFe / m.T) < a.margin)) {
             a.flag_list[atomicAdd(a.flag_count, 1u)] = c;
@@ -795,8 +1111,8 @@ __device__ __forceinline__ void rs_commit(const StageArgs& a, const StageVar& v,
 
 // Free energies, filling and decision of a visit from its nodes' results (DL
 // lanes of a warp, one per node; `on` is false for lanes beyond the last visit).
-template <typename T, RsMode kMode, int DL>
-__device__ __forceinline__ void rs_decide(const StageArgs& a, const StageVar& v, const RsVisit& h, const RsTerms& w,
+template <typename T, int DL>
+__device__ __forceinline__ void rs_decide(RsMode mode, const StageArgs& a, const StageVar& v, const RsVisit& h, const RsTerms& w,
                                           const RsOut<T>* out, int lane, bool on) {
     const Model& m = a.m;
     const double* so = v.S_in + 3 * (int64_t)h.site;
@@ -857,7 +1173,7 @@ __device__ __forceinline__ void rs_decide(const StageArgs& a, const StageVar& v,
     double dF = -m.T * (0.5 * ce * dx2 + dL - 0.5 * dx1);
     if (m.cls_on) dF += m.ca * (nn - oo) + m.cb * dx;
     const double fo = 0.5 * h.n - Th;
-    rs_commit<kMode>(a, v, h, w, fine, Fo, dF, fo, fo - dT);
+    rs_commit(mode, a, v, h, w, fine, Fo, dF, fo, fo - dT);
 }
 
 // A window beyond the last node class (fields thousands of T long): both
@@ -865,7 +1181,7 @@ __device__ __forceinline__ void rs_decide(const StageArgs& a, const StageVar& v,
 // re-solve slot.  Reached only by configurations that a caller sets far from
 // any the chain visits, so plain: one thread per row, no blocking.
 inline size_t rs_exact_bytes(int n) { return (size_t)n * 48 + ((size_t)n * 12 > 512 ? (size_t)n * 12 : 512); }
-__device__ __noinline__ void rs_exact(const StageArgs& a, const StageVar& v, const RsVisit& h, RsTerms& w,
+static __device__ __noinline__ void rs_exact(const StageArgs& a, const StageVar& v, const RsVisit& h, RsTerms& w, int slot,
                                       unsigned char* smem) {
     const int n = h.n, tid = threadIdx.x, nt = blockDim.x;
     double2* vk = reinterpret_cast<double2*>(smem);
@@ -873,7 +1189,7 @@ __device__ __noinline__ void rs_exact(const StageArgs& a, const StageVar& v, con
     double* d = reinterpret_cast<double*>(p + n);
     double* e2 = d + n;
     double* sp = e2 + n;                // window spins (12 n bytes); later the block sums
-    double2* A = a.gA + (int64_t)blockIdx.x * a.gA_stride;
+    double2* A = a.gA + (int64_t)slot * a.gA_stride;
     const Model& m = a.m;
     const Window win = make_window(m, h.site);
     double F[2], fill[2];
@@ -945,24 +1261,25 @@ __device__ __noinline__ void rs_exact(const StageArgs& a, const StageVar& v, con
         fill[var] = block_sum<double>(sn, sp + 32);
         __syncthreads();
     }
-    if (tid == 0) rs_commit<RS_RESOLVE>(a, v, h, w, true, F[0], F[1] - F[0], fill[0], fill[1]);
+    if (tid == 0) rs_commit(RS_RESOLVE, a, v, h, w, true, F[0], F[1] - F[0], fill[0], fill[1]);
     __syncthreads();
 }
 
 // Visits [first, first + nv) of the work list (nv <= vb <= 32), by the CTA.
 // uniform: all windows have one shape (periodic lattices), so that a warp may
-// hold nodes of several visits.
-template <class Tl, RsMode kMode>
-__device__ __forceinline__ void rs_visits(const StageArgs& a, const StageVar& v, const int32_t* list, int first, int nv,
+// hold nodes of several visits.  kPairs: windows split by parity (uniform).
+template <class Tl, bool kPairs>
+__device__ __forceinline__ void rs_visits(RsMode mode, const StageArgs& a, const StageVar& v, const int32_t* list, int first, int nv,
                                           int vb, int max_sites, bool uniform, unsigned char* smem, int* s_task) {
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    const RsLayout lay = rs_layout<Tl>(vb, max_sites, nw, uniform);
+    const RsLayout lay = rs_layout<Tl>(vb, max_sites, nw, uniform, kPairs);
     RsVisit* hd = reinterpret_cast<RsVisit*>(smem);
+    RsPairs& pt = *reinterpret_cast<RsPairs*>(smem + align16((size_t)vb * sizeof(RsVisit)));
     RsTerms* tm = reinterpret_cast<RsTerms*>(smem + lay.terms);
     RsOut<float>* out = reinterpret_cast<RsOut<float>*>(smem + lay.out);
     RsSite<float>* sites = reinterpret_cast<RsSite<float>*>(smem + lay.site);
     float* hop = reinterpret_cast<float*>(smem + lay.hop);
-    float2* buf = reinterpret_cast<float2*>(smem + lay.buf) + (size_t)(warp * Tl::NPW + lane / Tl::LPN) * Tl::NODE;
+    float2* buf = reinterpret_cast<float2*>(smem + lay.buf) + (size_t)(warp * Tl::NPW + lane / Tl::LPN) * Tl::node(kPairs);
     // Small windows: several visits per warp, so that its FP64 instructions
     // serve them together.
     constexpr int GL = Tl::NS == 1 ? 8 : Tl::NS <= 4 ? 16 : 32;
@@ -972,6 +1289,7 @@ __device__ __forceinline__ void rs_visits(const StageArgs& a, const StageVar& v,
         float* hk = uniform ? (k == 0 ? hop : nullptr) : hop + k * Tl::NS * Tl::NS;
         rs_gather<float, GL>(a.m, v.S_in, c, v.sites[c], hd[k], tm[k], sites + k * max_sites, hk, Tl::NS, lane % GL);
     }
+    if (kPairs && warp == nw - 1) rs_pairs(a.m, v.sites[list ? list[first] : first], pt, lane);
     if (threadIdx.x == 0) *s_task = 0;
     __syncthreads();
     if (warp == nw - 1 && lane < nv) {
@@ -1010,8 +1328,10 @@ __device__ __forceinline__ void rs_visits(const StageArgs& a, const StageVar& v,
         }
         const double s = 1.0 / (a.m.T * c_fermi[hd[k].cls].y[j]);
         RsOut<float> spare;
-        RsNode<Tl>::run(hd[k], sites + k * max_sites, hop + (uniform ? 0 : k * Tl::NS * Tl::NS), (float)s, (float)(a.m.t * s), buf,
-                        lane, idle ? &spare : out + k * kFermiOut + j);
+        RsOut<float>* const to = idle ? &spare : out + k * kFermiOut + j;
+        if constexpr (kPairs) RsNode<Tl>::run_pairs(pt, sites + k * max_sites, (float)s, (float)(a.m.t * s), buf, lane, to);
+        else RsNode<Tl>::run(hd[k], sites + k * max_sites, hop + (uniform ? 0 : k * Tl::NS * Tl::NS), (float)s,
+                             (float)(a.m.t * s), buf, lane, to);
     }
     __syncthreads();
     constexpr int DL = Tl::NS <= 4 ? 16 : 32;
@@ -1023,13 +1343,13 @@ __device__ __forceinline__ void rs_visits(const StageArgs& a, const StageVar& v,
             for (int k0 = 2 * warp; k0 < nv; k0 += 2 * nw) {
                 const int k = k0 + lane / 16;
                 const bool on = k < nv;
-                rs_decide<float, kMode, 16>(a, v, hd[on ? k : nv - 1], tm[on ? k : nv - 1], out + (on ? k : nv - 1) * kFermiOut,
+                rs_decide<float, 16>(mode, a, v, hd[on ? k : nv - 1], tm[on ? k : nv - 1], out + (on ? k : nv - 1) * kFermiOut,
                                             lane & 15, on);
             }
             return;
         }
     }
-    for (int k = warp; k < nv; k += nw) rs_decide<float, kMode, 32>(a, v, hd[k], tm[k], out + k * kFermiOut, lane, true);
+    for (int k = warp; k < nv; k += nw) rs_decide<float, 32>(mode, a, v, hd[k], tm[k], out + k * kFermiOut, lane, true);
 }
 
 // One visit by a thread-block cluster of node groups: node j goes to
@@ -1037,18 +1357,18 @@ __device__ __forceinline__ void rs_visits(const StageArgs& a, const StageVar& v,
 template <typename T, class Gp> struct RsGroupLayout { size_t terms, out, site, hop, buf, total; };
 template <typename T, class Gp> __host__ __device__ inline RsGroupLayout<T, Gp> rs_group_layout(int max_sites, int max_layer, int groups) {
     RsGroupLayout<T, Gp> L;
-    size_t o = align16(sizeof(RsVisit));
+    size_t o = align16(sizeof(RsVisit)) + align16(sizeof(RsPairs));
     L.terms = o; o = align16(o + sizeof(RsTerms));
     L.out = o;   o = align16(o + kFermiMaxNodes * sizeof(RsOut<T>));
     L.site = o;  o = align16(o + (size_t)max_sites * sizeof(RsSite<T>));
     L.hop = o;   o = align16(o + (size_t)max_layer * max_layer * sizeof(T));
-    L.buf = o;   o = align16(o + (size_t)groups * sizeof(typename RsGroup<T, Gp>::Smem));
+    L.buf = o;   o = align16(o + (size_t)groups * RsGroup<T, Gp>::bytes(2 * max_sites));
     L.total = o;
     return L;
 }
 
-template <typename T, class Gp, RsMode kMode>
-__device__ __forceinline__ void rs_visit_groups(const StageArgs& a, const StageVar& v, int c, int max_sites, int max_layer,
+template <typename T, class Gp, bool kPairs>
+__device__ __forceinline__ void rs_visit_groups(RsMode mode, const StageArgs& a, const StageVar& v, int c, int max_sites, int max_layer,
                                                 unsigned char* smem) {
     namespace cg = cooperative_groups;
     const cg::cluster_group cl = cg::this_cluster();
@@ -1057,12 +1377,14 @@ __device__ __forceinline__ void rs_visit_groups(const StageArgs& a, const StageV
     const int g = threadIdx.x / Gp::TPN, t = threadIdx.x % Gp::TPN;
     const auto lay = rs_group_layout<T, Gp>(max_sites, max_layer, groups);
     RsVisit& h = *reinterpret_cast<RsVisit*>(smem);
+    RsPairs& pt = *reinterpret_cast<RsPairs*>(smem + align16(sizeof(RsVisit)));
     RsTerms& tm = *reinterpret_cast<RsTerms*>(smem + lay.terms);
     RsOut<T>* out = reinterpret_cast<RsOut<T>*>(smem + lay.out);
     RsSite<T>* sites = reinterpret_cast<RsSite<T>*>(smem + lay.site);
     T* hop = reinterpret_cast<T*>(smem + lay.hop);
-    auto& sm = reinterpret_cast<typename RsGroup<T, Gp>::Smem*>(smem + lay.buf)[g];
+    auto& sm = *reinterpret_cast<typename RsGroup<T, Gp>::Smem*>(smem + lay.buf + (size_t)g * RsGroup<T, Gp>::bytes(2 * max_sites));
     if (warp == 0) rs_gather<T, 32>(a.m, v.S_in, c, v.sites[c], h, tm, sites, hop, max_layer, lane);
+    if (kPairs && warp == (blockDim.x > 32 ? 1 : 0)) rs_pairs(a.m, v.sites[c], pt, lane);
     __syncthreads();
     // Nodes of this group, then (one thread of the first CTA's last group, which
     // has the fewest) the proposal.
@@ -1071,7 +1393,8 @@ __device__ __forceinline__ void rs_visit_groups(const StageArgs& a, const StageV
         const FermiNodes& f = RsFermi<T>::tab(h.cls);
         for (int j = (size - 1 - rank) + size * g; j < f.M; j += size * groups) {
             const double s = 1.0 / (a.m.T * f.y[j]);
-            RsGroup<T, Gp>::run(h, sites, hop, max_layer, T(s), T(a.m.t * s), sm, t, 1 + g, out0 + j);
+            if constexpr (kPairs) RsGroup<T, Gp>::run_pairs(pt, sites, T(s), T(a.m.t * s), sm, t, 1 + g, out0 + j);
+            else RsGroup<T, Gp>::run(h, sites, hop, max_layer, T(s), T(a.m.t * s), sm, t, 1 + g, out0 + j);
         }
     }
     if (rank == 0 && threadIdx.x == blockDim.x - 1) {
@@ -1083,13 +1406,13 @@ __device__ __forceinline__ void rs_visit_groups(const StageArgs& a, const StageV
     if (size > 1) cl.sync();
     else __syncthreads();
     if (rank != 0) return;
-    if constexpr (kMode == RS_RESOLVE) {
+    if constexpr (sizeof(T) == 8) {   // the re-solve
         if (h.cls < 0) {
-            rs_exact(a, v, h, tm, smem + lay.out);
+            rs_exact(a, v, h, tm, blockIdx.x / size, smem + lay.out);
             return;
         }
     }
-    if (warp == 0) rs_decide<T, kMode, 32>(a, v, h, tm, out, lane, true);
+    if (warp == 0) rs_decide<T, 32>(mode, a, v, h, tm, out, lane, true);
 }
 
 }  // namespace ptca
