@@ -303,7 +303,7 @@ static void free_ctx(ptca_ctx* c) {
     void* ptrs[] = {c->d_sites, c->d_S[0], c->d_S[1], c->d_S[2], c->d_S[3], c->d_split, c->d_gL, c->d_F, c->d_fill, c->d_ticket, c->d_rec_site,
                     c->d_rec_Fold, c->d_rec_Fnew, c->d_rec_lnu, c->d_rec_acc, c->d_rec_Facc, c->d_rec_fill,
                     c->d_rec_n, c->d_counters, c->d_err, c->d_obs, c->d_stage_start, c->d_perm, c->d_queue,
-                    c->d_bar, c->d_sweep_ctr, c->d_flag_list, c->d_flag_count, c->d_gA,
+                    c->d_bar, c->d_sweep_ctr, c->d_flag_list, c->d_flag_count, c->d_gA, c->d_rs, c->d_prop,
                     c->d_chk_eig, c->d_chk_F, c->d_chk_out, c->d_sub, c->d_sub_spins};
     for (void* q : ptrs)
         if (q) cudaFree(q);
@@ -485,12 +485,14 @@ ptca_status ptca_init(const ptca_lattice* lattice, const ptca_params* params, pt
             for (int nw : {4, 1})
                 if (ptca::sweep_width_supported(c->prec, nw, c->nA))
                     widest = std::max(widest, sms * ptca::persistent_blocks_per_sm(c->prec, nw, c->nA));
-            const int slots = std::max(std::max(widest, c->resolve_grid), c->large ? c->large_grid : 0);
+            const int slots = std::max(std::max(widest, 2 * c->resolve_grid), c->large ? c->large_grid : 0);
             c->gA_stride = (int64_t)c->nA * (c->nA + 1) / 2;
             // + 64 elements: the fused pass may load up to 31 elements past a
             // slot (masked lanes of the diagonal chunk), also past the last.
             ce = dalloc(&c->d_gA, (size_t)slots * (size_t)c->gA_stride + 64);
             default_margin(c);
+            if (ce == cudaSuccess) ce = cudaMalloc(&c->d_rs, ptca::resolvent_scratch_bytes(sms));
+            if (ce == cudaSuccess && c->max_stage <= ptca::kFewVisits) ce = dalloc(&c->d_prop, (size_t)N);
         }
     }
     if (ce == cudaSuccess) ce = cudaMemset(c->d_rec_acc, 0, N);
@@ -627,6 +629,8 @@ static StageArgs base_args(ptca_ctx* ctx) {
     a.flag_count = ctx->d_flag_count;
     a.gA = ctx->d_gA;
     a.gA_stride = ctx->gA_stride;
+    a.rs_scratch = ctx->d_rs;
+    a.invT = 1.0 / ctx->p.T;
     a.gL = ctx->d_gL;
     a.gL_stride = ctx->gL_stride;
     return a;
@@ -645,9 +649,10 @@ static bool on_determinants(const ptca_ctx* ctx) {
     return ptca::resolvent_supported(to_model(ctx->p));
 }
 
-// Stages of at most this many visits run the latency-bound form: a group of
-// threads per node instead of one warp.
-static bool few_visits(const ptca_ctx* ctx) { return ctx->max_stage <= 64; }
+// Stages of at most kFewVisits visits run the latency-bound form: a group of
+// threads per node instead of one warp (45 against 110 us for 16 visits of 8x8
+// clusters; 215 against 123 us for 100 of 10x10).
+static bool few_visits(const ptca_ctx* ctx) { return ctx->max_stage <= ptca::kFewVisits; }
 
 // A stage launch and a re-solve launch in the context's configuration
 // (shared-memory kernels, or the large-cluster kernels).
@@ -721,6 +726,14 @@ static cudaError_t sweep_stages(ptca_ctx* ctx, int32_t n_sweeps, cudaStream_t st
             a.sg_center = col->center + (size_t)sw * ctx->N;
             a.sg_dF = col->dF + (size_t)sw * ctx->N;
         }
+        // Small stages wait for each visit's FP64 draws (4 of 49 us for 16 visits of
+        // 8x8 clusters): all of the sweep's at once.  The configuration is whole in
+        // buffer g mod 2 here.
+        a.prop = nullptr;
+        if (on_determinants(ctx) && few_visits(ctx)) {
+            e = ptca::launch_proposals(a, ctx->d_S[g & 1], ctx->N, ctx->d_prop, st);
+            a.prop = ctx->d_prop;
+        }
         for (int s = 0; s < ctx->nstages && e == cudaSuccess; ++s, ++g) {
             a.S_in = ctx->d_S[g & 1];
             a.S_out = ctx->d_S[(g + 1) & 1];
@@ -760,6 +773,7 @@ static void use_half(const ptca_ctx* ctx, StageArgs& a, int h) {
     a.ticket = ctx->d_ticket + h * ms;
     a.flag_list = ctx->d_flag_list + h * ms;
     a.flag_count = ctx->d_flag_count + h;
+    a.rs_half = h;
 }
 
 // Resources of the overlapped pipeline, made on first use.

@@ -100,6 +100,8 @@ struct ptca_ctx {
     int32_t* d_flag_list = nullptr;       // [2][max_stage]
     unsigned int* d_flag_count = nullptr; // [2]
     double2* d_gA = nullptr;
+    double4* d_prop = nullptr;            // proposals of a sweep (lattices of small stages)
+    void* d_rs = nullptr;                 // determinant kernels' node results (resolvent_scratch_bytes)
     int64_t gA_stride = 0;
     int resolve_grid = 0;
     // large traveling clusters (orders above the shared-memory kernels'):

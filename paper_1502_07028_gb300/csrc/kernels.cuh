@@ -369,6 +369,12 @@ struct StageArgs {
     // packed matrix of gL_stride elements (float2 or double2) per CTA.
     void* gL;
     int64_t gL_stride;
+    // Determinant kernels: node results passed between CTAs, in two halves by
+    // stage parity.
+    void* rs_scratch;
+    int32_t rs_half;
+    double invT;              // 1 / T (the host's: an FP64 division takes a microsecond of latency here)
+    const double4* prop;      // proposal and ln u by lattice site for this sweep, or null
     // Delayed acceptance: work list (perm) length on the device, and the
     // stage-1 surrogate dF~ per stage index (stage 2 accepts iff
     // ln u < -(dF - dF~)/T).  Null when screening is off.

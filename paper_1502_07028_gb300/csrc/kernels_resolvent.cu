@@ -28,6 +28,25 @@ __global__ void __launch_bounds__(Tl::MAXT, Tl::MINB) k_stage_rs(const __grid_co
                           uniform, smem, &s_task);
 }
 
+// Proposals and ln u of a whole sweep, one thread per site.  A site's variable
+// changes in its own stage alone, so that its value at the sweep's start is the one
+// its visit finds.
+__global__ void k_proposals(Model m, const double* __restrict__ S, int N, uint64_t sweep, const unsigned long long* sweep_dev,
+                            double4* __restrict__ out) {
+    const int site = blockIdx.x * blockDim.x + threadIdx.x;
+    if (site >= N) return;
+    const uint64_t sw = sweep + (sweep_dev ? *sweep_dev : 0);
+    double sn[3], u0, u1;
+    propose(m, sw, (uint32_t)site, S + 3 * (int64_t)site, sn);
+    uniform2(m.seed, sw, (uint32_t)site, RNG_ACCEPT, u0, u1);
+    out[site] = make_double4(sn[0], sn[1], sn[2], log(u0));
+}
+
+cudaError_t launch_proposals(const StageArgs& a, const double* S, int N, double4* out, cudaStream_t st) {
+    k_proposals<<<(N + 63) / 64, 64, 0, st>>>(a.m, S, N, a.sweep, a.sweep_dev, out);
+    return cudaGetLastError();
+}
+
 // f(tile, split by parity) with the tile of the problem's windows.
 template <typename F> static auto with_tile(const Model& m, F f) {
     const int np = pair_sites(m), ns = layer_sites(m);
@@ -99,7 +118,7 @@ static cudaError_t launch(RsMode mode, const StageArgs& a, int c0, int sms, cuda
 
 cudaError_t launch_stage_resolvent(const StageArgs& a, bool few, int sms, cudaStream_t st) {
     if (a.count <= 0) return cudaSuccess;
-    return few ? launch_groups(RS_STAGE, a, 0, st) : launch(RS_STAGE, a, 0, sms, st);
+    return few ? launch_groups(RS_STAGE, a, 0, sms, st) : launch(RS_STAGE, a, 0, sms, st);
 }
 
 cudaError_t launch_check_resolvent(const StageArgs& a, bool few, int c0, int count, double* F, int sms,
@@ -111,7 +130,7 @@ cudaError_t launch_check_resolvent(const StageArgs& a, bool few, int c0, int cou
     b.perm = nullptr;
     b.count_dev = nullptr;
     b.prev_count = b.prev2_count = 0;
-    return few ? launch_groups(RS_CHECK, b, c0, st) : launch(RS_CHECK, b, c0, sms, st);
+    return few ? launch_groups(RS_CHECK, b, c0, sms, st) : launch(RS_CHECK, b, c0, sms, st);
 }
 
 }  // namespace ptca

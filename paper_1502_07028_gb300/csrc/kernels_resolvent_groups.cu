@@ -1,6 +1,6 @@
-// kernels_resolvent_groups.cu -- determinant kernels with a group of threads per
-// node (resolvent.cuh): stages of few visits in FP32, and the double-float
-// re-solve.
+// kernels_resolvent_groups.cu -- determinant kernels that spread a visit over
+// several CTAs (resolvent.cuh): stages of few visits in FP32, and the
+// double-float re-solve.
 #include <algorithm>
 #include <type_traits>
 
@@ -9,33 +9,39 @@
 
 namespace ptca {
 
-// Deferred decisions of a stage, the same elimination in double-float: one
-// thread-block cluster per visit, a group of threads per node (a stage defers
-// some tens of visits, and the next stage waits for them).
+// Deferred decisions of a stage, the same elimination in double-float.  A stage
+// defers a handful to some tens of visits and the next stage waits for
+// them, so the CTAs share each visit's nodes while there are fewer visits than
+// CTAs, and take whole visits in turn beyond that.  scratch: node results, one
+// set per CTA of the grid.
 template <class Gp, bool kPairs>
-__global__ void __launch_bounds__(Gp::TPN * Gp::DFG, 1) k_resolve_rs(const __grid_constant__ StageArgs a, int max_sites,
-                                                                    int max_layer) {
+__global__ void __launch_bounds__(Gp::TPN * Gp::DFG + 32, 1) k_resolve_rs(const __grid_constant__ StageArgs a, int max_sites,
+                                                                         int max_layer, RsOut<dfl>* scratch, int max_parts) {
     extern __shared__ __align__(16) unsigned char smem[];
-    namespace cg = cooperative_groups;
-    const cg::cluster_group cl = cg::this_cluster();
-    const int size = (int)cl.num_blocks();
     const int nflag = (int)*(volatile unsigned int*)a.flag_count;
     if (nflag == 0) return;
-    cl.sync();       // every CTA of the cluster runs before its shared memory is written
-    for (int i = blockIdx.x / size; i < nflag; i += gridDim.x / size) {
-        rs_visit_groups<dfl, Gp, kPairs>(RS_RESOLVE, a, stage_var(a), a.flag_list[i], max_sites, max_layer, smem);
-        cl.sync();   // the first CTA's results are read before the next visit overwrites them
+    int parts = (int)gridDim.x / nflag;
+    parts = parts < 1 ? 1 : parts > max_parts ? max_parts : parts;
+    const StageVar v = stage_var(a);
+    if (parts > 1) {
+        const int i = blockIdx.x % nflag, part = blockIdx.x / nflag;
+        if (part >= parts) return;
+        rs_visit_part<RsGroups<Gp, kPairs>, kPairs>(RS_RESOLVE, a, v, a.flag_list[i], part, parts, scratch + (size_t)i * kFermiMaxNodes,
+                                       max_sites, max_layer, smem);
+        return;
     }
+    for (int i = blockIdx.x; i < nflag; i += gridDim.x)
+        rs_visit_part<RsGroups<Gp, kPairs>, kPairs>(RS_RESOLVE, a, v, a.flag_list[i], 0, 1, scratch + (size_t)blockIdx.x * kFermiMaxNodes,
+                                       max_sites, max_layer, smem);
 }
 
-// A stage of few visits: one cluster per visit, a group of threads per FP32 node.
-template <class Gp, bool kPairs>
-__global__ void __launch_bounds__(Gp::TPN * Gp::SPG, 1) k_stage_rs_few(const __grid_constant__ StageArgs a, int max_sites,
-                                                                      int max_layer, RsMode mode, int c0) {
+// A stage of few visits, `parts` CTAs each, FP32 nodes.  scratch: node results by
+// stage index.
+template <class Tl, bool kPairs>
+__global__ void __launch_bounds__(Tl::MAXT, Tl::MINB) k_stage_rs_few(const __grid_constant__ StageArgs a, int max_sites,
+                                                                           int max_layer, RsOut<float>* scratch, int parts,
+                                                                           RsMode mode, int c0) {
     extern __shared__ __align__(16) unsigned char smem[];
-    namespace cg = cooperative_groups;
-    const cg::cluster_group cl = cg::this_cluster();
-    const int size = (int)cl.num_blocks();
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < a.prev_count + a.prev2_count; k += gridDim.x * blockDim.x) {
         const int s = k < a.prev_count ? a.prev_sites[k] : a.prev2_sites[k - a.prev_count];
         a.S_out[3 * s] = a.S_in[3 * s];
@@ -43,10 +49,11 @@ __global__ void __launch_bounds__(Gp::TPN * Gp::SPG, 1) k_stage_rs_few(const __g
         a.S_out[3 * s + 2] = a.S_in[3 * s + 2];
     }
     const int count = a.count_dev ? (int)*a.count_dev : a.count;
-    const int i = blockIdx.x / size;
+    const int i = blockIdx.x / parts;
     if (i >= count) return;
-    if (size > 1) cl.sync();
-    rs_visit_groups<float, Gp, kPairs>(mode, a, stage_var(a), a.perm ? a.perm[i] : c0 + i, max_sites, max_layer, smem);
+    const int c = a.perm ? a.perm[i] : c0 + i;
+    rs_visit_part<RsWarps<Tl, kPairs>, kPairs>(mode, a, stage_var(a), c, blockIdx.x % parts, parts, scratch + (size_t)c * kFermiMaxNodes,
+                                     max_sites, max_layer, smem);
 }
 
 template <typename F> static auto with_group(const Model& m, F f) {
@@ -59,12 +66,28 @@ template <typename F> static auto with_group(const Model& m, F f) {
     return f(RsG32{}, std::false_type{});
 }
 
+template <typename F> static auto with_latency_tile(const Model& m, F f) {
+    const int np = pair_sites(m), ns = layer_sites(m);
+    if (np > 0 && np <= 4) return f(RsL4{}, std::true_type{});
+    if (np > 4) return f(RsT16{}, std::true_type{});
+    if (ns <= 4) return f(RsL4{}, std::false_type{});
+    if (ns <= 8) return f(RsL8{}, std::false_type{});
+    return f(RsT16{}, std::false_type{});
+}
+
 cudaError_t configure_resolvent_groups(size_t smem_limit) {
     cudaError_t e = cudaSuccess;
     auto group = [&](auto g, auto pairs) {
         if (e == cudaSuccess) e = allow_smem(k_resolve_rs<decltype(g), decltype(pairs)::value>, smem_limit);
-        if (e == cudaSuccess) e = allow_smem(k_stage_rs_few<decltype(g), decltype(pairs)::value>, smem_limit);
     };
+    auto tile = [&](auto t, auto pairs) {
+        if (e == cudaSuccess) e = allow_smem(k_stage_rs_few<decltype(t), decltype(pairs)::value>, smem_limit);
+    };
+    tile(RsL4{}, std::true_type{});
+    tile(RsT16{}, std::true_type{});
+    tile(RsL4{}, std::false_type{});
+    tile(RsL8{}, std::false_type{});
+    tile(RsT16{}, std::false_type{});
     group(RsG8{}, std::true_type{});
     group(RsG32{}, std::true_type{});
     group(RsG8{}, std::false_type{});
@@ -74,37 +97,28 @@ cudaError_t configure_resolvent_groups(size_t smem_limit) {
     return e;
 }
 
-template <typename K, typename... A>
-static cudaError_t launch_clusters(K kernel, int grid, int threads, size_t smem, int size, cudaStream_t st, A... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(threads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute at;
-    at.id = cudaLaunchAttributeClusterDimension;
-    at.val.clusterDim.x = size;
-    at.val.clusterDim.y = at.val.clusterDim.z = 1;
-    cfg.attrs = &at;
-    cfg.numAttrs = size > 1 ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kernel, args...);
+size_t resolvent_scratch_bytes(int sms) {
+    return (size_t)2 * sms * kFermiMaxNodes * sizeof(RsOut<dfl>) + 2 * (size_t)kFewVisits * kFermiMaxNodes * sizeof(RsOut<float>);
 }
 
-// The smallest cluster of up to 8 CTAs that holds a group for every node.
-static int cluster_for(int nodes, int groups) {
-    int size = 1;
-    while (size < 8 && size * groups < nodes) size *= 2;
-    return size;
-}
-
-cudaError_t launch_groups(RsMode mode, const StageArgs& a, int c0, cudaStream_t st) {
+cudaError_t launch_groups(RsMode mode, const StageArgs& a, int c0, int sms, cudaStream_t st) {
     static const FermiNodes tab[kFermiClasses] = {PTCA_FERMI_NODES};
     const int M = class_nodes(tab, unit_bound(a.m)), ms = window_sites(a.m), ml = layer_sites(a.m);
-    return with_group(a.m, [&](auto group, auto pairs) {
-        using Gp = decltype(group);
-        const int size = cluster_for(M, Gp::SPG), groups = std::min((M + size - 1) / size, Gp::SPG);
-        return launch_clusters(k_stage_rs_few<Gp, decltype(pairs)::value>, a.count * size, Gp::TPN * groups,
-                               rs_group_layout<float, Gp>(ms, ml, groups).total, size, st, a, ms, ml, mode, c0);
+    // node results by stage index: one set per stage parity (a.rs_half), as the
+    // other per-visit scratch
+    unsigned char* base = static_cast<unsigned char*>(a.rs_scratch) + (size_t)2 * sms * kFermiMaxNodes * sizeof(RsOut<dfl>);
+    RsOut<float>* scratch = reinterpret_cast<RsOut<float>*>(base) + (size_t)a.rs_half * kFewVisits * kFermiMaxNodes;
+    return with_latency_tile(a.m, [&](auto tile, auto pairs) {
+        using Tl = decltype(tile);
+        constexpr bool kPairs = decltype(pairs)::value;
+        using E = RsWarps<Tl, kPairs>;
+        // a visit's warps over as many CTAs as give four per SM
+        const int warps = (M + Tl::NPW - 1) / Tl::NPW;
+        const int parts = std::max(1, std::min(warps, 4 * sms / a.count));
+        const int threads = std::min(32 * ((warps + parts - 1) / parts) + 32, Tl::MAXT);
+        k_stage_rs_few<Tl, kPairs><<<a.count * parts, threads, rs_part_layout<E>(ms, ml, threads).total, st>>>(
+            a, ms, ml, scratch, parts, mode, c0);
+        return cudaGetLastError();
     });
 }
 
@@ -113,12 +127,12 @@ cudaError_t launch_resolve_resolvent(const StageArgs& a, int sms, cudaStream_t s
     const int M = class_nodes(tab, unit_bound(a.m)), ms = window_sites(a.m), ml = layer_sites(a.m);
     return with_group(a.m, [&](auto group, auto pairs) {
         using Gp = decltype(group);
-        const int size = cluster_for(M, Gp::DFG);
-        const int per_sm = Gp::TPN == 32 ? 2 : 1;   // CTAs that fit on an SM beside each other
-        const auto lay = rs_group_layout<dfl, Gp>(ms, ml, Gp::DFG);
-        const size_t smem = std::max(lay.total, lay.out + rs_exact_bytes(2 * ms));
-        return launch_clusters(k_resolve_rs<Gp, decltype(pairs)::value>, per_sm * sms / size * size, Gp::TPN * Gp::DFG, smem,
-                               size, st, a, ms, ml);
+        const auto lay = rs_part_layout<RsGroups<Gp, decltype(pairs)::value>>(ms, ml, Gp::TPN * Gp::DFG + 32);
+        const size_t smem = std::max(lay.total, lay.site + rs_exact_bytes(2 * ms));
+        const int grid = (Gp::TPN == 32 ? 2 : 1) * sms;   // one warp per node: two CTAs fit on an SM
+        k_resolve_rs<Gp, decltype(pairs)::value><<<grid, Gp::TPN * Gp::DFG + 32, smem, st>>>(
+            a, ms, ml, static_cast<RsOut<dfl>*>(a.rs_scratch), M);
+        return cudaGetLastError();
     });
 }
 

@@ -137,7 +137,12 @@ cudaError_t launch_stage_resolvent(const StageArgs& a, bool few, int sms, cudaSt
 cudaError_t launch_check_resolvent(const StageArgs& a, bool few, int c0, int count, double* F, int sms,
                                    cudaStream_t st);
 cudaError_t launch_resolve_resolvent(const StageArgs& a, int sms, cudaStream_t st);
+cudaError_t launch_proposals(const StageArgs& a, const double* S, int N, double4* out, cudaStream_t st);
 enum RsMode : int;
-cudaError_t launch_groups(RsMode mode, const StageArgs& a, int c0, cudaStream_t st);
+cudaError_t launch_groups(RsMode mode, const StageArgs& a, int c0, int sms, cudaStream_t st);
+// Node results that CTAs pass to one another (StageArgs::rs_scratch); stages of
+// at most kFewVisits visits have room for theirs.
+constexpr int kFewVisits = 64;
+size_t resolvent_scratch_bytes(int sms);
 
 }  // namespace ptca

@@ -39,8 +39,6 @@
 // padded by two elements so that the row groups hit different banks.
 #pragma once
 
-#include <cooperative_groups.h>
-
 #include "fermi_nodes.cuh"
 #include "kernels.cuh"
 
@@ -102,6 +100,9 @@ template <typename V> __device__ __forceinline__ V rs_det_g(V p00, V p01, V p10,
     return m;
 }
 
+__device__ __forceinline__ void rs_get(float& x, const volatile float* p) { x = *p; }
+__device__ __forceinline__ void rs_get(dfl& x, const volatile dfl* p) { x = dfl(p->hi, p->lo); }
+
 // Running sum of a lane's logarithms or phases: a float pair in FP32 (the
 // pivots' own rounding is all that is left), FP64 in double-float.
 template <typename T> struct RsSum;
@@ -123,7 +124,7 @@ template <> struct RsSum<dfl> {
 
 // On-site terms of a window site: mu - H = [[d + z, x - iy], [x + iy, d - z]].
 template <typename T> struct RsSite { T d, x, y, z; };
-template <typename T> struct RsOut { double lnd, th; T P[8]; };  // P: the last pivot block, without its i
+template <typename T> struct RsOut { double lnd, th; T P[8], s; };  // P: the last pivot block, without its i; s = 1 / (T y)
 
 // Window of a visit in layer order.
 struct RsVisit {
@@ -136,12 +137,12 @@ struct RsVisit {
 struct RsPairs {
     int na, nb, ne;                 // sites of block 0, of block 1, eliminated
     int kept[32], gone[32];         // window sites (layer order); kept: block 0, then block 1
-    uint32_t near[32];
+    uint32_t near[32], place[32];   // place: coordinates of the eliminated sites, packed
 };
 constexpr int kPairSites = 64;      // largest window
 
 // Sums over the window, FP64.
-struct RsTerms { double x1, x2, cl, sn[3], lnu; };
+struct RsTerms { double x1, x2, cl, sn[3], lnu; float dv[4]; };  // dv: change of (d, x, y, z) of RsSite, rounded
 
 template <int GR_, int GC_, int SR_, int SC_, int MAXT_, int MINB_> struct RsTile {
     static constexpr int GR = GR_, GC = GC_, SR = SR_, SC = SC_;
@@ -159,6 +160,9 @@ using RsT4 = RsTile<2, 2, 2, 2, 256, 2>;    // up to 4 sites per layer: 4x4 per 
 using RsT8 = RsTile<4, 4, 2, 2, 224, 2>;    // two nodes per warp
 using RsT12 = RsTile<4, 4, 3, 3, 224, 1>;   // 6x6 per lane
 using RsT16 = RsTile<8, 4, 2, 4, 256, 1>;   // 4x8 per lane, one node per warp
+// Stages of few visits: more lanes per node.
+using RsL4 = RsTile<4, 4, 1, 1, 256, 1>;
+using RsL8 = RsTile<8, 4, 1, 2, 256, 1>;
 
 template <class Tl> struct RsNode {
     using V = float2;
@@ -420,8 +424,8 @@ template <class Tl> struct RsNode {
             }
     }
 
-    static __device__ __forceinline__ void finish(const Tile& a, int us, RsSum<float>& lnd, RsSum<float>& th, int r, int c,
-                                                  int nl, RsOut<float>* out) {
+    static __device__ __forceinline__ void finish(const Tile& a, int us, float s, RsSum<float>& lnd, RsSum<float>& th, int r,
+                                                  int c, int nl, RsOut<float>* out) {
         // last pivot block: the lane holding rows and columns of the update site
 #pragma unroll
         for (int i = 0; i < SR; ++i)
@@ -441,6 +445,7 @@ template <class Tl> struct RsNode {
         if (nl == 0) {
             out->lnd = 0.5 * lnd.value();
             out->th = th.value();
+            out->s = s;
         }
         __syncwarp();
     }
@@ -485,7 +490,7 @@ template <class Tl> struct RsNode {
 #pragma unroll
                 for (int j = 0; j < 2 * SC; ++j) a[i][j] = csub(S[i][j], a[i][j]);
         }
-        finish(a, pt.nb - 1, lnd, th, r, c, nl, out);
+        finish(a, pt.nb - 1, s, lnd, th, r, c, nl, out);
     }
 
     // One node of one visit: the sums over all pivots but the update site's,
@@ -573,31 +578,31 @@ template <class Tl> struct RsNode {
                 __syncwarp();
             }
         }
-        finish(a, v.us, lnd, th, r, c, nl, out);
+        finish(a, v.us, s, lnd, th, r, c, nl, out);
     }
 };
 
 // ---------------------------------------------------------------------------
-// The same elimination by a group of GR x GC threads per node, for stages with
-// too few visits to fill the GPU and for the re-solve: there the time of one
-// node counts, not the throughput.  Thread (r, c) holds rows r + GR i and columns
-// c + GC j (a row is 2 site + spin); one row is pivoted at a time, its
-// row and column broadcast through double-buffered shared memory (one barrier of
-// the group per pivot), and nothing is padded.  Against one warp per node
-// with a 2x4 tile per lane: 45 us instead of 400 us per node in double-float
-// at n = 128.
+// The same elimination by a group of GR x GC threads per node, for the
+// double-float re-solve: the next stage waits for it, so the time of one node
+// counts.  Thread (r, c) holds rows r + GR i of column c (a row is 2 site + spin);
+// one row is pivoted at a time, its row, column and inverse pivot broadcast
+// through double-buffered shared memory (one barrier of the group per pivot),
+// and nothing is padded.  One column per thread: the scaled pivot row element
+// serves all its rows, so that a step is one product and R updates.  (In FP32
+// one warp per node is faster: 49 against 66 us for a stage of 16 visits of 8x8
+// clusters -- the barriers and the broadcast outweigh the arithmetic.)
 // ---------------------------------------------------------------------------
-template <int GR_, int GC_, int R_, int C_, int DFG_, int SPG_> struct RsGroupShape {
-    static constexpr int SPG = SPG_;                              // ... and at most of the FP32 stage kernel
-    static constexpr int DFG = DFG_;                              // groups per CTA of the re-solve
-    static constexpr int GR = GR_, GC = GC_, R = R_, C = C_, TPN = GR * GC;
-    static constexpr int B = GR * R > GC * C ? GR * R : GC * C;   // largest block order
-    static constexpr int RS = B + 1;                              // elements per matrix row
+template <int GR_, int GC_, int R_, int DFG_> struct RsGroupShape {
+    static constexpr int GR = GR_, GC = GC_, R = R_, C = 1, TPN = GR * GC;
+    static constexpr int DFG = DFG_;                              // groups per CTA
+    static constexpr int B = GC, RS = B + 1;                      // largest block order, elements per matrix row
+    static_assert(GR * R == GC, "square blocks");
 };
-using RsG8 = RsGroupShape<8, 4, 1, 2, 4, 8>;       // one warp, up to 4 sites per layer
-using RsG16 = RsGroupShape<16, 8, 1, 2, 3, 4>;     // four warps, up to 8 sites
-using RsG24 = RsGroupShape<16, 8, 2, 3, 3, 4>;     // ... 12 sites
-using RsG32 = RsGroupShape<16, 16, 2, 2, 2, 2>;    // eight warps, up to 16 sites
+using RsG8 = RsGroupShape<4, 8, 2, 3>;       // one warp, up to 4 sites per layer
+using RsG16 = RsGroupShape<8, 16, 2, 3>;     // four warps, up to 8 sites
+using RsG24 = RsGroupShape<8, 24, 3, 2>;     // six warps, 12 sites
+using RsG32 = RsGroupShape<8, 32, 4, 2>;     // eight warps, 16 sites
 
 template <typename T, class Gp> struct RsGroup {
     using V = cplx_t<T>;
@@ -605,7 +610,7 @@ template <typename T, class Gp> struct RsGroup {
     using Tile = V[R][C];
     // Shared memory of a group: three matrices, two broadcast buffers of a pivot
     // row and column; the node's pivots follow (bytes() with n of them).
-    struct Smem { V X[Gp::B * RS], C[Gp::B * RS], E[Gp::B * RS], row[2][Gp::B], col[2][Gp::B]; };
+    struct Smem { V X[Gp::B * RS], C[Gp::B * RS], E[Gp::B * RS], row[2][Gp::B], col[2][Gp::B], inv[2]; };
     static __host__ __device__ constexpr size_t bytes(int n) { return sizeof(Smem) + (size_t)n * sizeof(V); }
 
     static __device__ __forceinline__ void sync(int id) {
@@ -670,31 +675,30 @@ template <typename T, class Gp> struct RsGroup {
             if ((p >> 1) == skip) continue;
             V* row = sm.row[p & 1];
             V* col = sm.col[p & 1];
-#pragma unroll
-            for (int i = 0; i < R; ++i)
-#pragma unroll
-                for (int j = 0; j < C; ++j) {
-                    if (r + GR * i == p && c + GC * j < b) row[c + GC * j] = a[i][j];
-                    if (c + GC * j == p && r + GR * i < b) col[r + GR * i] = a[i][j];
-                }
-            sync(id);
-            const V pv = row[p];
-            if (r == 0 && c == 0) piv[p] = pv;
-            const T im = pv.y + T(1.f), rq = rs_rcp(pv.x * pv.x + im * im);
-            const V w = mk(pv.x * rq, -(im * rq));     // 1/(pivot + i)
             const V zero = mk(T(0.f), T(0.f));
-            V rv[C];
-#pragma unroll
-            for (int j = 0; j < C; ++j) rv[j] = c + GC * j < b ? row[c + GC * j] : zero;
+            const bool pc = c == p;
 #pragma unroll
             for (int i = 0; i < R; ++i) {
-                const bool pr = r + GR * i == p;
-                const V q = pr ? mk(-w.x, -w.y) : cfma(r + GR * i < b ? col[r + GR * i] : zero, w, zero);
-#pragma unroll
-                for (int j = 0; j < C; ++j) {
-                    const V x = cfms(q, rv[j], pr ? zero : a[i][j]);
-                    a[i][j] = c + GC * j == p ? mk(-q.x, -q.y) : x;
+                const int x = r + GR * i;
+                if (x == p) {
+                    if (c < b) row[c] = a[i][0];
+                    if (pc) {
+                        const V pv = a[i][0];
+                        piv[p] = pv;
+                        const T im = pv.y + T(1.f), rq = rs_rcp(pv.x * pv.x + im * im);
+                        sm.inv[p & 1] = mk(pv.x * rq, -(im * rq));     // 1/(pivot + i)
+                    }
                 }
+                if (pc && x < b) col[x] = a[i][0];
+            }
+            sync(id);
+            const V w = sm.inv[p & 1];
+            const V s = pc ? w : c < b ? cfma(row[c], w, zero) : zero;
+#pragma unroll
+            for (int i = 0; i < R; ++i) {
+                const int x = r + GR * i;
+                const V q = x < b ? col[x] : zero;
+                a[i][0] = x == p ? s : cfms(q, s, pc ? zero : a[i][0]);
             }
         }
     }
@@ -762,7 +766,7 @@ template <typename T, class Gp> struct RsGroup {
                 sync(id);
             }
         }
-        finish(a, sm, piv, b * L, b * (L - 1) + 2 * v.us, v.us, lnd, th, r, c, t, id, out);
+        finish(a, sm, piv, b * L, b * (L - 1) + 2 * v.us, v.us, s, lnd, th, r, c, t, id, out);
     }
 
     // o = P^t Q with P^t the block transpose of P (2x2 blocks stay as they are)
@@ -869,12 +873,12 @@ template <typename T, class Gp> struct RsGroup {
                 for (int j = 0; j < C; ++j) a[i][j] = csub(S[i][j], a[i][j]);
             sync(id);
         }
-        finish(a, sm, piv, ba + bb, ba + bb - 2, pt.nb - 1, lnd, th, r, c, t, id, out);
+        finish(a, sm, piv, ba + bb, ba + bb - 2, pt.nb - 1, s, lnd, th, r, c, t, id, out);
     }
 
     // Results of a node: the last pivot block, and the sums over the np pivots
     // but the update site's two, on top of what lnd and th hold already.
-    static __device__ __forceinline__ void finish(const Tile& a, Smem& sm, const V* piv, int np, int skip, int us, RsSum<T>& lnd,
+    static __device__ __forceinline__ void finish(const Tile& a, Smem& sm, const V* piv, int np, int skip, int us, T s, RsSum<T>& lnd,
                                                   RsSum<T>& th, int r, int c, int t, int id, RsOut<T>* out) {
         const T one = T(1.f);
 #pragma unroll
@@ -911,6 +915,7 @@ template <typename T, class Gp> struct RsGroup {
             for (int k = 1; k < Gp::TPN / 32; ++k) { l += part[k].x; h += part[k].y; }
             out->lnd = 0.5 * l;
             out->th = h;
+            out->s = s;
         }
         sync(id);
     }
@@ -937,6 +942,7 @@ __host__ __device__ inline RsLayout rs_layout(int vb, int max_sites, int nw, boo
     return L;
 }
 
+static __constant__ float c_fermi_x[kFermiClasses] = {PTCA_FERMI_X};
 static __constant__ FermiNodes c_fermi[kFermiClasses] = {PTCA_FERMI_NODES};
 static __constant__ FermiNodes c_fermi_df[kFermiClasses] = {PTCA_FERMI_NODES_DF};
 
@@ -945,40 +951,127 @@ template <typename T> struct RsFermi {
     static __device__ __forceinline__ const FermiNodes& tab(int cls) { return sizeof(T) == 4 ? c_fermi[cls] : c_fermi_df[cls]; }
 };
 
-// Window of a visit in layer order (layers along its longest axis, so that a
-// layer has the fewest sites), gathered by GL lanes of a warp: the on-site
-// terms, the in-layer hopping (when hop is given), Tr x and Tr x^2 over the
-// window, the classical energy, and the node class from Gershgorin's bound on
-// |mu - H|.
-template <typename T, int GL>
-__device__ __forceinline__ void rs_gather(const Model& m, const double* S, int c, int site, RsVisit& h, RsTerms& w,
-                                          RsSite<T>* sites, T* hop, int hs, int gl) {
-    const Window win = make_window(m, site);
-    const int ext[3] = {win.ex, win.ey, win.ez}, up[3] = {win.uwx, win.uwy, win.uwz};
-    int ax = 0;
-    if (ext[1] > ext[0]) ax = 1;
-    if (ext[2] > (ax ? ext[1] : ext[0])) ax = 2;
-    const int L = ax == 0 ? ext[0] : ax == 1 ? ext[1] : ext[2];
-    const int e0 = ax == 0 ? ext[1] : ext[0], e1 = ax == 2 ? ext[1] : ext[2];  // the other axes, in order
-    const int u0 = ax == 0 ? up[1] : up[0], u1 = ax == 2 ? up[1] : up[2];
-    const int ns = e0 * e1, nsite = ns * L, per = m.cluster_periodic;
+// A window in layer order: layers along its longest axis (a layer then has the
+// fewest sites), e0 x e1 sites each; window site k is site k % ns of layer k / ns.
+struct RsFrame {
+    Window win;
+    int ax, L, e0, e1, ns, u, us;   // u, us: layer and in-layer index of the update site
+    __device__ __forceinline__ int site(const Model& m, int k) const {
+        const int l = k / ns, q = k % ns, q0 = q % e0, q1 = q / e0;
+        return window_site(m, win, ax == 0 ? l : q0, ax == 1 ? l : (ax == 0 ? q0 : q1), ax == 2 ? l : q1);
+    }
+};
+__device__ __forceinline__ RsFrame rs_frame(const Model& m, int site) {
+    RsFrame f;
+    f.win = make_window(m, site);
+    const Window& w = f.win;
+    f.ax = w.ez > max(w.ex, w.ey) ? 2 : w.ey > w.ex ? 1 : 0;
+    f.L = f.ax == 0 ? w.ex : f.ax == 1 ? w.ey : w.ez;
+    f.e0 = f.ax == 0 ? w.ey : w.ex;                 // the other axes, in order
+    f.e1 = f.ax == 2 ? w.ey : w.ez;
+    f.ns = f.e0 * f.e1;
+    f.u = f.ax == 0 ? w.uwx : f.ax == 1 ? w.uwy : w.uwz;
+    f.us = (f.ax == 2 ? w.uwy : w.uwz) * f.e0 + (f.ax == 0 ? w.uwy : w.uwx);
+    return f;
+}
+
+// Tr x, Tr x^2 (on-site sums x1, x2 plus the hopping) and the classical energy.
+__device__ __forceinline__ void rs_terms_out(const StageArgs& a, const RsFrame& f, double x1, double x2, double cl, RsTerms& w) {
+    const int per = a.m.cluster_periodic, nsite = f.ns * f.L;
+    int pairs = 0;
+    for (int e : {f.L, f.e0, f.e1}) pairs += e < 2 ? 0 : nsite / e * (per ? (e == 2 ? 4 : e) : e - 1);
+    w.x1 = x1 * a.invT;
+    w.x2 = (x2 + 4.0 * a.m.t * a.m.t * (double)pairs) * a.invT * a.invT;
+    w.cl = cl;
+}
+
+// A visit's window, gathered by GL lanes of a warp: the on-site terms, the node
+// class from Gershgorin's bound on |mu - H|, and (kTerms) rs_terms.
+template <typename T, int GL, bool kTerms>
+__device__ __forceinline__ void rs_gather(const StageArgs& a, const double* S, int c, int site, RsVisit& h, RsTerms& w,
+                                          RsSite<T>* sites, int gl) {
+    const Model& m = a.m;
+    const RsFrame f = rs_frame(m, site);
+    const int nsite = f.ns * f.L, per = m.cluster_periodic;
     const double mus = m.mu - m.e0;
     double x1 = 0.0, x2 = 0.0, cl = 0.0;
     float bound = 0.f;
     for (int k = gl; k < nsite; k += GL) {
-        const int l = k / ns, q = k % ns, q0 = q % e0, q1 = q / e0;
-        const int wx = ax == 0 ? l : q0, wy = ax == 1 ? l : (ax == 0 ? q0 : q1), wz = ax == 2 ? l : q1;
-        const double* v = S + 3 * (int64_t)window_site(m, win, wx, wy, wz);
-        const double v0 = v[0], v1 = v[1], v2 = v[2], m2 = v0 * v0 + v1 * v1 + v2 * v2;
-        const double d = mus - m.lam * v0;
+        const double* v = S + 3 * (int64_t)f.site(m, k);
+        const double v0 = v[0], v1 = v[1], v2 = v[2], d = mus - m.lam * v0;
         sites[k].d = T(d); sites[k].x = T(m.JH * v0); sites[k].y = T(m.JH * v1); sites[k].z = T(m.JH * v2);
+        if constexpr (kTerms) {
+            const double m2 = v0 * v0 + v1 * v1 + v2 * v2;
+            x1 -= 2.0 * d;
+            x2 += 2.0 * (d * d + m.JH * m.JH * m2);
+            if (m.cls_on) cl += m.ca * m2 + m.cb * v0 + m.cc;
+        }
+        const float g0 = (float)v0, g1 = (float)v1, g2 = (float)v2;
+        bound = fmaxf(bound, fabsf((float)d) + fabsf((float)m.JH) * sqrtf(g0 * g0 + g1 * g1 + g2 * g2));
+    }
+#pragma unroll
+    for (int o = GL / 2; o > 0; o >>= 1) {
+        if constexpr (kTerms) {
+            x1 += __shfl_xor_sync(FULL_MASK, x1, o);
+            x2 += __shfl_xor_sync(FULL_MASK, x2, o);
+            if (m.cls_on) cl += __shfl_xor_sync(FULL_MASK, cl, o);
+        }
+        bound = fmaxf(bound, __shfl_xor_sync(FULL_MASK, bound, o));
+    }
+    if (gl == 0) {
+        float deg = 0.f;
+        for (int e : {f.L, f.e0, f.e1}) deg += e < 2 ? 0.f : e == 2 && !per ? 1.f : 2.f;
+        const float X = (bound + deg * fabsf((float)m.t)) * (float)a.invT * (1.f + 1e-6f);
+        int cls = 0;
+        while (cls < kFermiClasses && !(X <= c_fermi_x[cls])) ++cls;
+        h.c = c; h.site = site; h.n = 2 * nsite; h.L = f.L; h.ns = f.ns; h.per = per;
+        h.u = f.u;
+        h.us = f.us;
+        h.cls = cls < kFermiClasses ? cls : -1;
+        if constexpr (kTerms) rs_terms_out(a, f, x1, x2, cl, w);
+    }
+}
+
+// rs_terms_out of a window, by one warp.
+__device__ __forceinline__ void rs_terms(const StageArgs& a, const double* S, int site, RsTerms& w, int lane) {
+    const Model& m = a.m;
+    const RsFrame f = rs_frame(m, site);
+    const double mus = m.mu - m.e0;
+    double x1 = 0.0, x2 = 0.0, cl = 0.0;
+    for (int k = lane; k < f.ns * f.L; k += 32) {
+        const double* v = S + 3 * (int64_t)f.site(m, k);
+        const double v0 = v[0], d = mus - m.lam * v0, m2 = v0 * v0 + v[1] * v[1] + v[2] * v[2];
         x1 -= 2.0 * d;
         x2 += 2.0 * (d * d + m.JH * m.JH * m2);
         if (m.cls_on) cl += m.ca * m2 + m.cb * v0 + m.cc;
-        bound = fmaxf(bound, fabsf((float)d) + fabsf((float)m.JH) * sqrtf((float)m2));
     }
-    // in-layer bonds (an axis of extent 2 of a periodic cluster has two)
-    if (hop) for (int k = gl; k < hs * hs; k += GL) {
+    x1 = warp_sum(x1);
+    x2 = warp_sum(x2);
+    if (m.cls_on) cl = warp_sum(cl);
+    if (lane == 0) rs_terms_out(a, f, x1, x2, cl, w);
+}
+
+// The proposal and ln u of a visit (one thread): drawn here, or from the sweep's
+// table where the caller drew them all at once.
+__device__ __forceinline__ void rs_proposal(const StageArgs& a, const StageVar& v, int site, RsTerms& w) {
+    if (a.prop) {
+        const double4 p = a.prop[site];
+        w.sn[0] = p.x; w.sn[1] = p.y; w.sn[2] = p.z;
+        w.lnu = p.w;
+        return;
+    }
+    double u0, u1;
+    propose(a.m, v.sweep, (uint32_t)site, v.S_in + 3 * (int64_t)site, w.sn);
+    uniform2(a.m.seed, v.sweep, (uint32_t)site, RNG_ACCEPT, u0, u1);
+    w.lnu = log(u0);
+}
+
+// In-layer hopping of a window between sites a and b of a layer, at [a hs + b]
+// (an axis of extent 2 of a periodic cluster has two bonds), by one warp.
+template <typename T> __device__ __forceinline__ void rs_hopping(const Model& m, int site, T* hop, int hs, int lane) {
+    const RsFrame f = rs_frame(m, site);
+    const int e0 = f.e0, e1 = f.e1, ns = f.ns, per = m.cluster_periodic;
+    for (int k = lane; k < hs * hs; k += 32) {
         const int a = k / hs, b = k % hs;
         double bonds = 0.0;
         if (a < ns && b < ns) {
@@ -988,54 +1081,24 @@ __device__ __forceinline__ void rs_gather(const Model& m, const double* S, int c
         }
         hop[k] = T(m.t * bonds);
     }
-#pragma unroll
-    for (int o = GL / 2; o > 0; o >>= 1) {
-        x1 += __shfl_xor_sync(FULL_MASK, x1, o);
-        x2 += __shfl_xor_sync(FULL_MASK, x2, o);
-        if (m.cls_on) cl += __shfl_xor_sync(FULL_MASK, cl, o);
-        bound = fmaxf(bound, __shfl_xor_sync(FULL_MASK, bound, o));
-    }
-    if (gl == 0) {
-        double pairs = 0.0, deg = 0.0;
-        for (int k = 0; k < 3; ++k) {
-            const int e = k == 0 ? L : k == 1 ? e0 : e1;
-            if (e < 2) continue;
-            const double lines = (double)(nsite / e);
-            pairs += lines * (per ? (e == 2 ? 4.0 : (double)e) : (double)(e - 1));
-            deg += e == 2 && !per ? 1.0 : 2.0;
-        }
-        x2 += 4.0 * m.t * m.t * pairs;
-        const double X = ((double)bound * (1.0 + 1e-6) + deg * fabs(m.t)) / m.T;
-        int cls = 0;
-        while (cls < kFermiClasses && !(X <= c_fermi[cls].X)) ++cls;
-        h.c = c; h.site = site; h.n = 2 * nsite; h.L = L; h.ns = ns; h.per = per;
-        h.u = ax == 0 ? up[0] : ax == 1 ? up[1] : up[2];
-        h.us = u1 * e0 + u0;
-        h.cls = cls < kFermiClasses ? cls : -1;
-        w.x1 = x1 / m.T;
-        w.x2 = x2 / (m.T * m.T);
-        w.cl = cl;
-    }
 }
 
 // The parity split of a periodic lattice's windows (all alike), by one warp.
 // Window sites in layer order, as rs_gather places them.
 __device__ __forceinline__ void rs_pairs(const Model& m, int site, RsPairs& t, int lane) {
-    const Window win = make_window(m, site);
-    const int ext[3] = {win.ex, win.ey, win.ez}, up[3] = {win.uwx, win.uwy, win.uwz};
-    int ax = 0;
-    if (ext[1] > ext[0]) ax = 1;
-    if (ext[2] > (ax ? ext[1] : ext[0])) ax = 2;
-    const int e0 = ax == 0 ? ext[1] : ext[0], e1 = ax == 2 ? ext[1] : ext[2], e2 = ext[ax];
-    const int u0 = ax == 0 ? up[1] : up[0], u1 = ax == 2 ? up[1] : up[2], u2 = up[ax];
-    const int ns = e0 * e1, n = ns * e2, per = m.cluster_periodic;
-    const int u = u2 * ns + u1 * e0 + u0;
-    auto parity = [&](int k) { return (k % e0 + k / e0 % e1 + k / ns) & 1; };
-    auto bond = [&](int a, int b) {
-        const int d0 = abs(a % e0 - b % e0), d1 = abs(a / e0 % e1 - b / e0 % e1), d2 = abs(a / ns - b / ns);
-        const int h0 = d0 == 1 || (per && d0 == e0 - 1 && d0 > 0), h1 = d1 == 1 || (per && d1 == e1 - 1 && d1 > 0),
-                  h2 = d2 == 1 || (per && d2 == e2 - 1 && d2 > 0);
-        return (h0 && !d1 && !d2) || (h1 && !d0 && !d2) || (h2 && !d0 && !d1);
+    const RsFrame f = rs_frame(m, site);
+    const int e0 = f.e0, e1 = f.e1, e2 = f.L, ns = f.ns, n = ns * e2, per = m.cluster_periodic, u = f.u * ns + f.us;
+    // coordinates of a window site, packed (8 bits each); parity; bonds
+    auto place = [&](int k) { return (uint32_t)(k % e0) | (uint32_t)(k / e0 % e1) << 8 | (uint32_t)(k / ns) << 16; };
+    auto parity = [&](int k) {
+        const uint32_t x = place(k);
+        return (int)((x ^ (x >> 8) ^ (x >> 16)) & 1u);
+    };
+    auto next = [&](int d, int e) { return d == 1 || (per && d == e - 1); };
+    auto bond = [&](uint32_t x, uint32_t y) {
+        const int d0 = abs((int)(x & 255) - (int)(y & 255)), d1 = abs((int)(x >> 8 & 255) - (int)(y >> 8 & 255)),
+                  d2 = abs((int)(x >> 16) - (int)(y >> 16));
+        return (d0 && !d1 && !d2 && next(d0, e0)) || (!d0 && d1 && !d2 && next(d1, e1)) || (!d0 && !d1 && d2 && next(d2, e2));
     };
     const int pu = parity(u);
     // kept and eliminated sites in order, the update site last
@@ -1045,7 +1108,10 @@ __device__ __forceinline__ void rs_pairs(const Model& m, int site, RsPairs& t, i
         const bool in = k < n, keep = in && k != u && parity(k) == pu, drop = in && parity(k) != pu;
         const unsigned bk = __ballot_sync(FULL_MASK, keep), bd = __ballot_sync(FULL_MASK, drop), below = (1u << lane) - 1u;
         if (keep) t.kept[nk + __popc(bk & below)] = k;
-        if (drop) t.gone[ne + __popc(bd & below)] = k;
+        if (drop) {
+            t.gone[ne + __popc(bd & below)] = k;
+            t.place[ne + __popc(bd & below)] = place(k);
+        }
         nk += __popc(bk);
         ne += __popc(bd);
     }
@@ -1057,8 +1123,9 @@ __device__ __forceinline__ void rs_pairs(const Model& m, int site, RsPairs& t, i
     }
     __syncwarp();
     if (lane <= nk) {
+        const uint32_t x = place(t.kept[lane]);
         uint32_t near = 0;
-        for (int e = 0; e < ne; ++e) near |= (uint32_t)bond(t.kept[lane], t.gone[e]) << e;
+        for (int e = 0; e < ne; ++e) near |= (uint32_t)bond(x, t.place[e]) << e;
         t.near[lane] = near;
     }
 }
@@ -1085,13 +1152,13 @@ __device__ __forceinline__ void rs_commit(RsMode mode, const StageArgs& a, const
     const double dFe = stage2_dF(a, c, dF);
     if (mode == RS_STAGE) {
         // near the threshold, or a window beyond the last node class
-        if (!fine || (a.margin > 0.0 && fabs(w.lnu + dFe / m.T) < a.margin)) {
+        if (!fine || (a.margin > 0.0 && fabs(w.lnu + dFe * a.invT) < a.margin)) {
             a.flag_list[atomicAdd(a.flag_count, 1u)] = c;
             atomicAdd(&a.counters[2], 1ull);
             return;
         }
     }
-    const bool acc = w.lnu < -dFe / m.T;
+    const bool acc = w.lnu < -dFe * a.invT;
     if (a.sg_feat) collect_sample(a, v.S_in, make_window(m, site), v.rec_base + c, w.sn, dF);
     double* dst = v.S_out + 3 * (int64_t)site;
 #pragma unroll
@@ -1109,71 +1176,93 @@ __device__ __forceinline__ void rs_commit(RsMode mode, const StageArgs& a, const
     atomicAdd(&a.counters[1], 2ull);
 }
 
-// Free energies, filling and decision of a visit from its nodes' results (DL
-// lanes of a warp, one per node; `on` is false for lanes beyond the last visit).
-template <typename T, int DL>
-__device__ __forceinline__ void rs_decide(RsMode mode, const StageArgs& a, const StageVar& v, const RsVisit& h, const RsTerms& w,
-                                          const RsOut<T>* out, int lane, bool on) {
+// A node's results, past the L1 (another SM may have written them).
+template <typename T> __device__ __forceinline__ void rs_load(RsOut<T>& r, const RsOut<T>* p) {
+    const volatile RsOut<T>* q = p;
+    r.lnd = q->lnd;
+    r.th = q->th;
+#pragma unroll
+    for (int k = 0; k < 8; ++k) rs_get(r.P[k], &q->P[k]);
+    rs_get(r.s, &q->s);
+}
+
+// The last pivot of a node: lq = ln|det| and t0 = phase (against i^2) of the
+// update site's block, and dl, dt their changes under the proposal, which adds
+// [[dd + jz, jx - i jy], [jx + i jy, dd - jz]] (times s already) to the block.
+template <typename T, typename L>
+__device__ __forceinline__ void rs_last_pivot(const RsOut<T>& r, T dd, T jx, T jy, T jz, L& lq, L& t0, L& dl, L& dt) {
+    const auto p00 = mk(r.P[0], r.P[1]), p01 = mk(r.P[2], r.P[3]), p10 = mk(r.P[4], r.P[5]), p11 = mk(r.P[6], r.P[7]);
+    const auto g = rs_det_g(p00, p01, p10, p11);
+    const auto gn = rs_det_g(mk(p00.x + dd + jz, p00.y), mk(p01.x + jx, p01.y - jy), mk(p10.x + jx, p10.y + jy),
+                             mk(p11.x + dd - jz, p11.y));
+    const T q = (g.x + g.x) + (g.x * g.x + g.y * g.y), qn = (gn.x + gn.x) + (gn.x * gn.x + gn.y * gn.y);
+    // det_new / det_old = 1 + z, with det_new - det_old formed from the
+    // change of the block (no cancellation between the two determinants)
+    const auto zero = mk(T(0.f), T(0.f));
+    const T ax = dd + jz, bx = dd - jz;
+    auto num = cfma(p11, mk(ax, T(0.f)), cfma(p00, mk(bx, T(0.f)), zero));
+    num = cfms(p01, mk(jx, jy), num);
+    num = cfms(p10, mk(jx, -jy), num);
+    // (P + i): the i of the two diagonal entries; minus det of the change
+    num = mk(num.x + ax * bx - (jx * jx + jy * jy), num.y + ax + bx);
+    const T gr = T(1.f) + g.x, rq = rs_rcp(gr * gr + g.y * g.y);
+    // z = num / det_old, det_old = -(1 + g)
+    const auto z = cfms(num, mk(gr * rq, -(g.y * rq)), zero);
+    const T zq = (z.x + z.x) + (z.x * z.x + z.y * z.y);
+    const L l0 = rs_log1p(q), half = (L)0.5;
+    lq = half * l0;
+    dl = zq < T(1.f) && T(-0.5f) < zq ? half * rs_log1p(zq) : half * (rs_log1p(qn) - l0);
+    t0 = rs_phase(g.y, T(1.f) + g.x);
+    dt = rs_phase(gn.y, T(1.f) + gn.x) - t0;
+}
+
+// Free energies, filling and decision of a visit (one thread) from its weighted
+// sums over the nodes: ln|det| and phases of the old matrix, and their changes.
+__device__ __forceinline__ void rs_final(RsMode mode, const StageArgs& a, const StageVar& v, const RsVisit& h, const RsTerms& w,
+                                         const FermiNodes& f, double Lo, double Th, double dL, double dT) {
     const Model& m = a.m;
     const double* so = v.S_in + 3 * (int64_t)h.site;
-    const double invT = 1.0 / m.T;
-    const double dx = w.sn[0] - so[0], dy = w.sn[1] - so[1], dz = w.sn[2] - so[2];
-    const double oo = so[0] * so[0] + so[1] * so[1] + so[2] * so[2];
-    const double nn = w.sn[0] * w.sn[0] + w.sn[1] * w.sn[1] + w.sn[2] * w.sn[2];
-    double Lo = 0.0, Th = 0.0, dL = 0.0, dT = 0.0, ce = 0.0, cc = 0.0;
-    const bool fine = on && h.cls >= 0;
-    if (fine) {
-        const FermiNodes& f = RsFermi<T>::tab(h.cls);
-        ce = f.e;
-        cc = f.c;
-        if (lane < f.M) {
-            const RsOut<T>& r = out[lane];
-            const double s = 1.0 / (m.T * f.y[lane]);
-            const T dd = T(-m.lam * dx * s), jx = T(m.JH * dx * s), jy = T(m.JH * dy * s), jz = T(m.JH * dz * s);
-            const auto p00 = mk(r.P[0], r.P[1]), p01 = mk(r.P[2], r.P[3]), p10 = mk(r.P[4], r.P[5]), p11 = mk(r.P[6], r.P[7]);
-            const auto g = rs_det_g(p00, p01, p10, p11);
-            const auto gn = rs_det_g(mk(p00.x + dd + jz, p00.y), mk(p01.x + jx, p01.y - jy), mk(p10.x + jx, p10.y + jy),
-                                     mk(p11.x + dd - jz, p11.y));
-            const T q = (g.x + g.x) + (g.x * g.x + g.y * g.y), qn = (gn.x + gn.x) + (gn.x * gn.x + gn.y * gn.y);
-            // det_new / det_old = 1 + z, with det_new - det_old formed from the
-            // change of the block (no cancellation between the two determinants)
-            const auto zero = mk(T(0.f), T(0.f));
-            const T ax = dd + jz, bx = dd - jz;
-            auto num = cfma(p11, mk(ax, T(0.f)), cfma(p00, mk(bx, T(0.f)), zero));
-            num = cfms(p01, mk(jx, jy), num);
-            num = cfms(p10, mk(jx, -jy), num);
-            // (P + i): the i of the two diagonal entries; minus det of the change
-            num = mk(num.x + ax * bx - (jx * jx + jy * jy), num.y + ax + bx);
-            const T gr = T(1.f) + g.x, rq = rs_rcp(gr * gr + g.y * g.y);
-            // z = num / det_old, det_old = -(1 + g)
-            const auto z = cfms(num, mk(gr * rq, -(g.y * rq)), zero);
-            const T zq = (z.x + z.x) + (z.x * z.x + z.y * z.y);
-            const double dl = zq < T(1.f) && T(-0.5f) < zq ? 0.5 * (double)rs_log1p(zq)
-                                                           : 0.5 * ((double)rs_log1p(qn) - (double)rs_log1p(q));
-            const double t0 = (double)rs_phase(g.y, T(1.f) + g.x), t1 = (double)rs_phase(gn.y, T(1.f) + gn.x);
-            Lo = f.a[lane] * (r.lnd + 0.5 * (double)rs_log1p(q));
-            Th = f.b[lane] * (r.th + t0);
-            dL = f.a[lane] * dl;
-            dT = f.b[lane] * (t1 - t0);
-        }
-    }
-#pragma unroll
-    for (int o = DL / 2; o > 0; o >>= 1) {
-        Lo += __shfl_xor_sync(FULL_MASK, Lo, o);
-        Th += __shfl_xor_sync(FULL_MASK, Th, o);
-        dL += __shfl_xor_sync(FULL_MASK, dL, o);
-        dT += __shfl_xor_sync(FULL_MASK, dT, o);
-    }
-    if (lane != 0 || !on) return;
+    const bool fine = h.cls >= 0;
+    const double invT = a.invT, dx = w.sn[0] - so[0];
+    // |v|^2 of the site, new minus old
+    const double dn = (w.sn[0] - so[0]) * (w.sn[0] + so[0]) + (w.sn[1] - so[1]) * (w.sn[1] + so[1]) +
+                      (w.sn[2] - so[2]) * (w.sn[2] + so[2]);
     const double dx1 = 2.0 * m.lam * dx * invT;
     // d(d^2 + J^2 |v|^2) of the site's two rows, d = mu - e0 - lam v_x
     const double mus = m.mu - m.e0, d0 = mus - m.lam * so[0], d1 = mus - m.lam * w.sn[0];
-    const double dx2 = 2.0 * (d1 * d1 - d0 * d0 + m.JH * m.JH * (nn - oo)) * invT * invT;
-    const double Fo = -m.T * (h.n * (0.69314718055994530942 + cc) + 0.5 * ce * w.x2 + Lo - 0.5 * w.x1) + w.cl;
-    double dF = -m.T * (0.5 * ce * dx2 + dL - 0.5 * dx1);
-    if (m.cls_on) dF += m.ca * (nn - oo) + m.cb * dx;
+    const double dx2 = 2.0 * ((d1 - d0) * (d1 + d0) + m.JH * m.JH * dn) * invT * invT;
+    const double Fo = -m.T * (h.n * (0.69314718055994530942 + f.c) + 0.5 * f.e * w.x2 + Lo - 0.5 * w.x1) + w.cl;
+    double dF = -m.T * (0.5 * f.e * dx2 + dL - 0.5 * dx1);
+    if (m.cls_on) dF += m.ca * dn + m.cb * dx;
     const double fo = 0.5 * h.n - Th;
     rs_commit(mode, a, v, h, w, fine, Fo, dF, fo, fo - dT);
+}
+
+// One visit by one warp, lane = node.
+template <typename T>
+__device__ __forceinline__ void rs_decide(RsMode mode, const StageArgs& a, const StageVar& v, const RsVisit& h, const RsTerms& w,
+                                          const RsOut<T>* out, int lane) {
+    const Model& m = a.m;
+    const double* so = v.S_in + 3 * (int64_t)h.site;
+    const FermiNodes& f = RsFermi<T>::tab(h.cls >= 0 ? h.cls : 0);
+    double Lo = 0.0, Th = 0.0, dL = 0.0, dT = 0.0;
+    if (h.cls >= 0 && lane < f.M) {
+        RsOut<T> r;
+        rs_load(r, out + lane);
+        const T dd = T(-m.lam * (w.sn[0] - so[0])) * r.s, jx = T(m.JH * (w.sn[0] - so[0])) * r.s,
+                jy = T(m.JH * (w.sn[1] - so[1])) * r.s, jz = T(m.JH * (w.sn[2] - so[2])) * r.s;
+        decltype(rs_log1p(r.s)) lq, t0, dl, dt;
+        rs_last_pivot(r, dd, jx, jy, jz, lq, t0, dl, dt);
+        Lo = f.a[lane] * (r.lnd + (double)lq);
+        Th = f.b[lane] * (r.th + (double)t0);
+        dL = f.a[lane] * (double)dl;
+        dT = f.b[lane] * (double)dt;
+    }
+    Lo = warp_sum(Lo);
+    Th = warp_sum(Th);
+    dL = warp_sum(dL);
+    dT = warp_sum(dT);
+    if (lane == 0) rs_final(mode, a, v, h, w, f, Lo, Th, dL, dT);
 }
 
 // A window beyond the last node class (fields thousands of T long): both
@@ -1286,9 +1375,11 @@ __device__ __forceinline__ void rs_visits(RsMode mode, const StageArgs& a, const
     for (int k0 = warp * (32 / GL); k0 < nv; k0 += nw * (32 / GL)) {
         const int k = k0 + lane / GL < nv ? k0 + lane / GL : nv - 1;   // lanes past the end repeat the last visit
         const int c = list ? list[first + k] : first + k;
-        float* hk = uniform ? (k == 0 ? hop : nullptr) : hop + k * Tl::NS * Tl::NS;
-        rs_gather<float, GL>(a.m, v.S_in, c, v.sites[c], hd[k], tm[k], sites + k * max_sites, hk, Tl::NS, lane % GL);
+        rs_gather<float, GL, true>(a, v.S_in, c, v.sites[c], hd[k], tm[k], sites + k * max_sites, lane % GL);
     }
+    if (!kPairs)
+        for (int k = nw - 1 - warp; k < (uniform ? 1 : nv); k += nw)
+            rs_hopping(a.m, v.sites[list ? list[first + k] : first + k], hop + k * Tl::NS * Tl::NS, Tl::NS, lane);
     if (kPairs && warp == nw - 1) rs_pairs(a.m, v.sites[list ? list[first] : first], pt, lane);
     if (threadIdx.x == 0) *s_task = 0;
     __syncthreads();
@@ -1296,10 +1387,13 @@ __device__ __forceinline__ void rs_visits(RsMode mode, const StageArgs& a, const
         // proposals and uniforms of the CTA's visits, one lane each, beside
         // the other warps' eliminations
         const int site = hd[lane].site;
-        double u0, u1;
-        propose(a.m, v.sweep, (uint32_t)site, v.S_in + 3 * (int64_t)site, tm[lane].sn);
-        uniform2(a.m.seed, v.sweep, (uint32_t)site, RNG_ACCEPT, u0, u1);
-        tm[lane].lnu = log(u0);
+        rs_proposal(a, v, site, tm[lane]);
+        const double* so = v.S_in + 3 * (int64_t)site;
+        const double dx = tm[lane].sn[0] - so[0];
+        tm[lane].dv[0] = (float)(-a.m.lam * dx);
+        tm[lane].dv[1] = (float)(a.m.JH * dx);
+        tm[lane].dv[2] = (float)(a.m.JH * (tm[lane].sn[1] - so[1]));
+        tm[lane].dv[3] = (float)(a.m.JH * (tm[lane].sn[2] - so[2]));
     }
     __syncwarp();
     // Tasks: NPW nodes per warp, of one visit unless the windows are uniform.
@@ -1326,7 +1420,7 @@ __device__ __forceinline__ void rs_visits(RsMode mode, const StageArgs& a, const
             idle = j >= M;
             if (idle) j = M - 1;
         }
-        const double s = 1.0 / (a.m.T * c_fermi[hd[k].cls].y[j]);
+        const double s = a.invT / c_fermi[hd[k].cls].y[j];
         RsOut<float> spare;
         RsOut<float>* const to = idle ? &spare : out + k * kFermiOut + j;
         if constexpr (kPairs) RsNode<Tl>::run_pairs(pt, sites + k * max_sites, (float)s, (float)(a.m.t * s), buf, lane, to);
@@ -1334,85 +1428,143 @@ __device__ __forceinline__ void rs_visits(RsMode mode, const StageArgs& a, const
                              (float)(a.m.t * s), buf, lane, to);
     }
     __syncthreads();
-    constexpr int DL = Tl::NS <= 4 ? 16 : 32;
-    const bool half = DL == 16 && uniform;   // 16 lanes per visit hold the nodes of the classes up to |x| = 1024
-    if (half) {
-        bool wide = false;
-        for (int k = 0; k < nv; ++k) wide |= hd[k].cls >= 0 && c_fermi[hd[k].cls].M > 16;
-        if (!wide) {
-            for (int k0 = 2 * warp; k0 < nv; k0 += 2 * nw) {
-                const int k = k0 + lane / 16;
-                const bool on = k < nv;
-                rs_decide<float, 16>(mode, a, v, hd[on ? k : nv - 1], tm[on ? k : nv - 1], out + (on ? k : nv - 1) * kFermiOut,
-                                            lane & 15, on);
-            }
-            return;
+    if constexpr (Tl::NS <= 4) {
+        // Many visits: the nodes' last pivots spread over the CTA in FP32, then a
+        // lane per visit for the FP64 sums (a warp's FP64 instruction holds the
+        // pipe for 17 cycles, whatever its lanes: one visit per warp took half
+        // the time of a chain's stage).
+        for (int q = threadIdx.x; q < nv * kFermiOut; q += blockDim.x) {
+            const int k = q / kFermiOut, j = q % kFermiOut;
+            if (hd[k].cls < 0 || j >= c_fermi[hd[k].cls].M) continue;
+            RsOut<float>& r = out[q];
+            float lq, t0, dl, dt;
+            rs_last_pivot(r, tm[k].dv[0] * r.s, tm[k].dv[1] * r.s, tm[k].dv[2] * r.s, tm[k].dv[3] * r.s, lq, t0, dl, dt);
+            r.P[0] = lq; r.P[1] = t0; r.P[2] = dl; r.P[3] = dt;
         }
+        __syncthreads();
+        if (warp == 0 && lane < nv) {
+            const FermiNodes& f = c_fermi[hd[lane].cls >= 0 ? hd[lane].cls : 0];
+            double Lo = 0.0, Th = 0.0, dL = 0.0, dT = 0.0;
+            if (hd[lane].cls >= 0)
+                for (int j = 0; j < f.M; ++j) {
+                    const RsOut<float>& r = out[lane * kFermiOut + j];
+                    Lo += f.a[j] * (r.lnd + (double)r.P[0]);
+                    Th += f.b[j] * (r.th + (double)r.P[1]);
+                    dL += f.a[j] * (double)r.P[2];
+                    dT += f.b[j] * (double)r.P[3];
+                }
+            rs_final(mode, a, v, hd[lane], tm[lane], f, Lo, Th, dL, dT);
+        }
+    } else {
+        for (int k = warp; k < nv; k += nw) rs_decide<float>(mode, a, v, hd[k], tm[k], out + k * kFermiOut, lane);
     }
-    for (int k = warp; k < nv; k += nw) rs_decide<float, 32>(mode, a, v, hd[k], tm[k], out + k * kFermiOut, lane, true);
 }
 
-// One visit by a thread-block cluster of node groups: node j goes to
-// group j mod (groups of the cluster), results to the first CTA.
-template <typename T, class Gp> struct RsGroupLayout { size_t terms, out, site, hop, buf, total; };
-template <typename T, class Gp> __host__ __device__ inline RsGroupLayout<T, Gp> rs_group_layout(int max_sites, int max_layer, int groups) {
-    RsGroupLayout<T, Gp> L;
+// One visit, its nodes dealt to `parts` CTAs: each leaves its nodes' results in
+// out (global memory), and the CTA that arrives last (the visit's ticket)
+// decides.  Nobody waits for another CTA.  The CTA's last warp draws the
+// proposal meanwhile.  Nodes are done by RsNode's lanes (FP32) or by RsGroup's
+// threads (double-float): RsWarps and RsGroups below say how.
+struct RsPartLayout { size_t terms, site, hop, buf, total; };
+template <class E> __host__ __device__ inline RsPartLayout rs_part_layout(int max_sites, int max_layer, int threads) {
+    RsPartLayout L;
     size_t o = align16(sizeof(RsVisit)) + align16(sizeof(RsPairs));
     L.terms = o; o = align16(o + sizeof(RsTerms));
-    L.out = o;   o = align16(o + kFermiMaxNodes * sizeof(RsOut<T>));
-    L.site = o;  o = align16(o + (size_t)max_sites * sizeof(RsSite<T>));
-    L.hop = o;   o = align16(o + (size_t)max_layer * max_layer * sizeof(T));
-    L.buf = o;   o = align16(o + (size_t)groups * RsGroup<T, Gp>::bytes(2 * max_sites));
+    L.site = o;  o = align16(o + (size_t)max_sites * sizeof(RsSite<typename E::Real>));
+    L.hop = o;   o = align16(o + (size_t)E::hop_stride(max_layer) * E::hop_stride(max_layer) * sizeof(typename E::Real));
+    L.buf = o;   o = align16(o + (size_t)(threads - 32) / E::LANES * E::bytes(max_sites));
     L.total = o;
     return L;
 }
 
-template <typename T, class Gp, bool kPairs>
-__device__ __forceinline__ void rs_visit_groups(RsMode mode, const StageArgs& a, const StageVar& v, int c, int max_sites, int max_layer,
-                                                unsigned char* smem) {
-    namespace cg = cooperative_groups;
-    const cg::cluster_group cl = cg::this_cluster();
-    const int size = (int)cl.num_blocks(), rank = (int)cl.block_rank();
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, groups = blockDim.x / Gp::TPN;
-    const int g = threadIdx.x / Gp::TPN, t = threadIdx.x % Gp::TPN;
-    const auto lay = rs_group_layout<T, Gp>(max_sites, max_layer, groups);
+// FP32 nodes on LPN lanes of a warp.  LANES: threads that share one `unit`
+// index; a unit takes one node.
+template <class Tl, bool kPairs> struct RsWarps {
+    using Real = float;
+    static constexpr int LANES = Tl::LPN;
+    static constexpr bool kFullWarp = true;   // the warp's nodes run together
+    static __host__ __device__ constexpr int hop_stride(int) { return Tl::NS; }
+    static __host__ __device__ constexpr size_t bytes(int) { return Tl::node(kPairs) * sizeof(float2); }
+    static __device__ __forceinline__ void run(const RsVisit& h, const RsPairs& pt, const RsSite<float>* site, const float* hop,
+                                               int, float s, float tp, unsigned char* buf, int, RsOut<float>* out) {
+        if constexpr (kPairs) RsNode<Tl>::run_pairs(pt, site, s, tp, reinterpret_cast<float2*>(buf), threadIdx.x & 31, out);
+        else RsNode<Tl>::run(h, site, hop, s, tp, reinterpret_cast<float2*>(buf), threadIdx.x & 31, out);
+    }
+};
+template <class Gp, bool kPairs> struct RsGroups {
+    using Real = dfl;
+    static constexpr int LANES = Gp::TPN;
+    static constexpr bool kFullWarp = false;
+    static __host__ __device__ constexpr int hop_stride(int max_layer) { return max_layer; }
+    static __host__ __device__ constexpr size_t bytes(int max_sites) { return RsGroup<dfl, Gp>::bytes(2 * max_sites); }
+    static __device__ __forceinline__ void run(const RsVisit& h, const RsPairs& pt, const RsSite<dfl>* site, const dfl* hop,
+                                               int hs, dfl s, dfl tp, unsigned char* buf, int unit, RsOut<dfl>* out) {
+        using G = RsGroup<dfl, Gp>;
+        auto& sm = *reinterpret_cast<typename G::Smem*>(buf);
+        const int t = threadIdx.x % Gp::TPN;
+        if constexpr (kPairs) G::run_pairs(pt, site, s, tp, sm, t, 1 + unit, out);
+        else G::run(h, site, hop, hs, s, tp, sm, t, 1 + unit, out);
+    }
+};
+
+template <class E, bool kPairs>
+__device__ __forceinline__ void rs_visit_part(RsMode mode, const StageArgs& a, const StageVar& v, int c, int part, int parts,
+                                              RsOut<typename E::Real>* out, int max_sites, int max_layer, unsigned char* smem) {
+    using T = typename E::Real;
+    __shared__ int s_last;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, units = (blockDim.x - 32) / E::LANES;
+    const bool extra = threadIdx.x >= blockDim.x - 32;
+    const auto lay = rs_part_layout<E>(max_sites, max_layer, blockDim.x);
     RsVisit& h = *reinterpret_cast<RsVisit*>(smem);
     RsPairs& pt = *reinterpret_cast<RsPairs*>(smem + align16(sizeof(RsVisit)));
     RsTerms& tm = *reinterpret_cast<RsTerms*>(smem + lay.terms);
-    RsOut<T>* out = reinterpret_cast<RsOut<T>*>(smem + lay.out);
     RsSite<T>* sites = reinterpret_cast<RsSite<T>*>(smem + lay.site);
     T* hop = reinterpret_cast<T*>(smem + lay.hop);
-    auto& sm = *reinterpret_cast<typename RsGroup<T, Gp>::Smem*>(smem + lay.buf + (size_t)g * RsGroup<T, Gp>::bytes(2 * max_sites));
-    if (warp == 0) rs_gather<T, 32>(a.m, v.S_in, c, v.sites[c], h, tm, sites, hop, max_layer, lane);
-    if (kPairs && warp == (blockDim.x > 32 ? 1 : 0)) rs_pairs(a.m, v.sites[c], pt, lane);
+    const int hs = E::hop_stride(max_layer), site = v.sites[c];
+    if (warp == 0) rs_gather<T, 32, false>(a, v.S_in, c, site, h, tm, sites, lane);
+    if (extra) {
+        if constexpr (kPairs) rs_pairs(a.m, site, pt, lane);
+        else rs_hopping(a.m, site, hop, hs, lane);
+    }
     __syncthreads();
-    // Nodes of this group, then (one thread of the first CTA's last group, which
-    // has the fewest) the proposal.
-    RsOut<T>* const out0 = size > 1 ? cl.map_shared_rank(out, 0) : out;
-    if (h.cls >= 0) {
+    if (extra) {
+        if (lane == 0) rs_proposal(a, v, site, tm);
+        rs_terms(a, v.S_in, site, tm, lane);
+    } else if (h.cls >= 0) {
         const FermiNodes& f = RsFermi<T>::tab(h.cls);
-        for (int j = (size - 1 - rank) + size * g; j < f.M; j += size * groups) {
-            const double s = 1.0 / (a.m.T * f.y[j]);
-            if constexpr (kPairs) RsGroup<T, Gp>::run_pairs(pt, sites, T(s), T(a.m.t * s), sm, t, 1 + g, out0 + j);
-            else RsGroup<T, Gp>::run(h, sites, hop, max_layer, T(s), T(a.m.t * s), sm, t, 1 + g, out0 + j);
+        // nodes part, part + parts, ... of the visit, in turn over the units
+        const int unit = threadIdx.x / E::LANES, mine = (f.M - part + parts - 1) / parts;
+        for (int u0 = 0; u0 < mine; u0 += units) {
+            int u = u0 + unit;
+            const bool idle = u >= mine;
+            if (idle && !E::kFullWarp) break;
+            if (idle) u = mine - 1;
+            if (E::kFullWarp && __all_sync(FULL_MASK, idle)) break;
+            const int j = part + parts * u;
+            const double s = a.invT / f.y[j];
+            RsOut<T> spare;
+            E::run(h, pt, sites, hop, hs, T(s), T(a.m.t * s), smem + lay.buf + (size_t)unit * E::bytes(max_sites), unit,
+                   idle ? &spare : out + j);
         }
     }
-    if (rank == 0 && threadIdx.x == blockDim.x - 1) {
-        double u0, u1;
-        propose(a.m, v.sweep, (uint32_t)h.site, v.S_in + 3 * (int64_t)h.site, tm.sn);
-        uniform2(a.m.seed, v.sweep, (uint32_t)h.site, RNG_ACCEPT, u0, u1);
-        tm.lnu = log(u0);
-    }
-    if (size > 1) cl.sync();
-    else __syncthreads();
-    if (rank != 0) return;
     if constexpr (sizeof(T) == 8) {   // the re-solve
         if (h.cls < 0) {
-            rs_exact(a, v, h, tm, blockIdx.x / size, smem + lay.out);
+            __syncthreads();
+            if (part == 0) rs_exact(a, v, h, tm, blockIdx.x, smem + lay.site);
+            __syncthreads();
             return;
         }
     }
-    if (warp == 0) rs_decide<T, 32>(mode, a, v, h, tm, out, lane, true);
+    __threadfence();   // this thread's node results, before the ticket
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        s_last = parts == 1 || atomicAdd(&a.ticket[c], 1) == parts - 1;
+        if (parts > 1 && s_last) a.ticket[c] = 0;
+        __threadfence();
+    }
+    __syncthreads();
+    if (s_last && warp == 0) rs_decide<T>(mode, a, v, h, tm, out, lane);
+    __syncthreads();
 }
 
 }  // namespace ptca
