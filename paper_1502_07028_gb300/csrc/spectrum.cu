@@ -6,11 +6,11 @@
 //   1. the dense matrix is built as its packed lower triangle (row-major:
 //      element (i, j <= i) at i(i+1)/2 + j) in global memory;
 //   2. a Householder reduction to real tridiagonal form spread over the whole
-//      GPU: per reflector, one tiled pass applies the previous reflector's
-//      deferred rank-2 update to the trailing block and accumulates the
-//      Hermitian matrix-vector product with the current reflector (row and
-//      column partial sums per 64 x 64 tile, in a fixed order), a reduction
-//      combines the partials, and one CTA forms w, the explicit update of the
+//      GPU: per reflector, one pass applies the previous reflector's deferred
+//      rank-2 update to the trailing block and accumulates the Hermitian
+//      matrix-vector product with the current reflector (row and column partial
+//      sums per strip of 64 columns, in a fixed order), and one thread-block
+//      cluster adds the partials up and forms w, the explicit update of the
 //      next pivot column and the next reflector -- the algorithm of the
 //      cluster kernels (cluster_solve.cuh), with the matrix too large for one
 //      SM;
@@ -32,10 +32,15 @@ namespace ptca {
 
 __host__ __device__ __forceinline__ int64_t tri64(int64_t r) { return r * (r + 1) / 2; }
 
-constexpr int FS_TB = 64;          // tile edge of the reduction pass
-constexpr int FS_PASS_THREADS = 256;
+constexpr int FS_TB = 64;            // columns of a strip of the reduction pass
+constexpr int FS_PASS_THREADS = 256, FS_PASS_WARPS = FS_PASS_THREADS / 32;
+constexpr int FS_PASS_CTAS = 2;      // resident per SM
+constexpr int FS_GROUP = 4;          // rows that a warp loads and reduces at a time
+constexpr int FS_MIN_ROWS = 16, FS_MAX_ROWS = 128;  // rows of a chunk
 constexpr int FS_RED_THREADS = 256;  // 8 warps; each CTA sums the partials of FS_RED_ROWS rows
 constexpr int FS_RED_ROWS = 32;
+constexpr int FS_CL = 8;             // CTAs of the step cluster (the portable size)
+constexpr int FS_STEP_THREADS = 1024, FS_STEP_PARTS = 4, FS_STEP_ROWS = FS_STEP_THREADS / FS_STEP_PARTS;
 constexpr int FS_SCALAR_THREADS = 1024;
 constexpr int FS_EIG_THREADS = 128;
 
@@ -81,12 +86,196 @@ __device__ __forceinline__ double fs_d(dfl x) { return (double)x; }
 template <typename R> __device__ __forceinline__ R fs_r(float x);
 template <> __device__ __forceinline__ double fs_r<double>(float x) { return (double)x; }
 template <> __device__ __forceinline__ dfl fs_r<dfl>(float x) { return dfl(x, 0.f); }
+__device__ __forceinline__ double shfl_xor_r(double v, int o) { return __shfl_xor_sync(FULL_MASK, v, o); }
+__device__ __forceinline__ dfl shfl_xor_r(dfl v, int o) { return shfl_xor_dfl(v, o); }
+
+// Pairs of floats for the two-wide FP32 instructions.
+using fs_f2 = unsigned long long;
+__device__ __forceinline__ fs_f2 f2_pack(float a, float b) {
+    fs_f2 r;
+    asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(a), "f"(b));
+    return r;
+}
+__device__ __forceinline__ float2 f2_split(fs_f2 v) {
+    float2 r;
+    asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
+    return r;
+}
+__device__ __forceinline__ fs_f2 f2_dup(float a) { return f2_pack(a, a); }
+__device__ __forceinline__ fs_f2 f2_add(fs_f2 a, fs_f2 b) {
+    fs_f2 r;
+    asm("add.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ fs_f2 f2_sub(fs_f2 a, fs_f2 b) {
+    fs_f2 r;
+    asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ fs_f2 f2_mul(fs_f2 a, fs_f2 b) {
+    fs_f2 r;
+    asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
+    return r;
+}
+__device__ __forceinline__ fs_f2 f2_fma(fs_f2 a, fs_f2 b, fs_f2 c) {
+    fs_f2 r;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
+    return r;
+}
+
+// A complex double-float in memory: the leading parts of (re, im), then the
+// trailing ones, so that the pass works on pairs; and its accumulators.
+struct __align__(16) DfPair { fs_f2 hi, lo; };
+// c += p + (the product's error and cross terms), not renormalised: TwoSum on the
+// leading parts, everything below into the trailing ones.
+__device__ __forceinline__ void df_add(DfPair& c, fs_f2 hi, fs_f2 lo) {
+    const fs_f2 s = f2_add(c.hi, hi), t = f2_sub(s, c.hi);
+    const fs_f2 e = f2_add(f2_sub(c.hi, f2_sub(s, t)), f2_sub(hi, t));
+    c.hi = s;
+    c.lo = f2_add(c.lo, f2_add(e, lo));
+}
+// a b elementwise: the rounded product, and its error and cross terms in lo.
+__device__ __forceinline__ fs_f2 df_mul(const DfPair& a, const DfPair& b, fs_f2& lo) {
+    const fs_f2 p = f2_mul(a.hi, b.hi);
+    const float2 x = f2_split(a.hi), y = f2_split(b.hi), q = f2_split(p);
+    lo = f2_fma(a.lo, b.hi, f2_fma(a.hi, b.lo, f2_pack(__fmaf_rn(x.x, y.x, -q.x), __fmaf_rn(x.y, y.y, -q.y))));
+    return p;
+}
+__device__ __forceinline__ void df_fma(DfPair& c, const DfPair& a, const DfPair& b) {
+    fs_f2 lo;
+    const fs_f2 p = df_mul(a, b, lo);
+    df_add(c, p, lo);
+}
+__device__ __forceinline__ DfPair df_norm(const DfPair& c) {
+    DfPair r;
+    r.hi = f2_add(c.hi, c.lo);
+    r.lo = f2_sub(c.lo, f2_sub(r.hi, c.hi));
+    return r;
+}
+__device__ __forceinline__ DfPair df_dup(dfl v) { return {f2_dup(v.hi), f2_dup(v.lo)}; }
+__device__ __forceinline__ DfPair df_pack(dfl x, dfl y) { return {f2_pack(x.hi, y.hi), f2_pack(x.lo, y.lo)}; }
+
+// The memory form of a complex entry and its conversions.
+template <typename R> struct FsMem { using type = cplx_t<R>; };
+template <> struct FsMem<dfl> { using type = DfPair; };
+template <typename R> using fs_mem = typename FsMem<R>::type;
+__device__ __forceinline__ double2 fs_get(const double2& v) { return v; }
+__device__ __forceinline__ dfl2 fs_get(const DfPair& v) {
+    const float2 h = f2_split(v.hi), l = f2_split(v.lo);
+    return mk(dfl(h.x, l.x), dfl(h.y, l.y));
+}
+// s += v on memory forms, without the renormalisation (fs_sum does it once).
+__device__ __forceinline__ void fs_acc(double2& s, const double2& v) { s = cadd(s, v); }
+__device__ __forceinline__ void fs_acc(DfPair& s, const DfPair& v) { df_add(s, v.hi, v.lo); }
+__device__ __forceinline__ double2 fs_sum(const double2& s) { return s; }
+__device__ __forceinline__ dfl2 fs_sum(const DfPair& s) { return fs_get(df_norm(s)); }
+__device__ __forceinline__ void fs_acc(double& s, double v) { s += v; }
+__device__ __forceinline__ void fs_acc(dfl& s, dfl v) {
+    const dfl t = two_sum(s.hi, v.hi);
+    s = dfl(t.hi, __fadd_rn(__fadd_rn(t.lo, v.lo), s.lo));
+}
+__device__ __forceinline__ double fs_sum(double s) { return s; }
+__device__ __forceinline__ dfl fs_sum(dfl s) { return fast_two_sum(s.hi, s.lo); }
+__device__ __forceinline__ double2 fs_xor(const double2& v, int o) { return cshfl_xor(v, o); }
+__device__ __forceinline__ DfPair fs_xor(const DfPair& v, int o) {
+    return {__shfl_xor_sync(FULL_MASK, v.hi, o), __shfl_xor_sync(FULL_MASK, v.lo, o)};
+}
+__device__ __forceinline__ void fs_put(double2& m, double2 v) { m = v; }
+__device__ __forceinline__ void fs_put(DfPair& m, dfl2 v) { m = df_pack(v.x, v.y); }
+
+// The pass's arithmetic on one element x of row i and a column c: the update
+// x - u_i w_c^* - w_i u_c^*, the row sum of x v_c and the column sum of x^* v_i.
+// `Row` and `Col` hold the operands in the form that the products take, `Sum` is
+// an accumulator; save() leaves a row sum's parts in two places of shared memory
+// and total() reads them.
+template <typename R> struct FsOps;
+template <> struct FsOps<double> {
+    struct Row { double2 u, w, v; };
+    struct Col { double2 u, w, v; };
+    using Sum = double2;
+    static __device__ __forceinline__ Sum zero() { return make_double2(0.0, 0.0); }
+    static __device__ __forceinline__ Row row(const double2* m) { return {m[0], m[1], m[2]}; }
+    static __device__ __forceinline__ Col col(double2 u, double2 w, double2 v) { return {u, w, v}; }
+    static __device__ __forceinline__ double2 update(double2 x, const Row& r, const Col& c) {
+        return cfms_conj_b(r.w, c.u, cfms_conj_b(r.u, c.w, x));
+    }
+    static __device__ __forceinline__ void real(double2& x) { x.y = 0.0; }
+    static __device__ __forceinline__ void row_add(Sum& s, double2 x, const Col& c, bool) { s = cfma(x, c.v, s); }
+    static __device__ __forceinline__ void col_add(Sum& s, double2 x, const Row& r) { s = cfma_conj_a(x, r.v, s); }
+    static __device__ __forceinline__ void save_row(double2* m, const Sum& s) { *m = s; }
+    static __device__ __forceinline__ double2 row_total(const double2* m, int n, int stride) {
+        double2 s = m[0];
+        for (int j = 1; j < n; ++j) s = cadd(s, m[j * stride]);
+        return s;
+    }
+    static __device__ __forceinline__ double2 col_total(const Sum& s) { return s; }
+};
+template <> struct FsOps<dfl> {
+    // Scalars of the row, both halves alike; the column's u and w as (-re, im) and
+    // (-im, -re), so that the update is four products into the element; v's parts
+    // alike.  The sums keep the products with v.x and v.y apart and combine them
+    // at the end: nothing is swapped or negated per element.  51 + 16 + 24
+    // two-wide operations an element (216 scalar ones before).
+    struct Row { DfPair ux, uy, wx, wy, vx, vy; };
+    struct Col { DfPair u1, u2, w1, w2, vx, vy; };
+    struct Sum { DfPair x, y; };
+    static __device__ __forceinline__ Sum zero() { return {{0, 0}, {0, 0}}; }
+    static __device__ __forceinline__ Row row(const DfPair* m) {
+        const dfl2 u = fs_get(m[0]), w = fs_get(m[1]), v = fs_get(m[2]);
+        return {df_dup(u.x), df_dup(u.y), df_dup(w.x), df_dup(w.y), df_dup(v.x), df_dup(v.y)};
+    }
+    static __device__ __forceinline__ Col col(dfl2 u, dfl2 w, dfl2 v) {
+        return {df_pack(-u.x, u.y), df_pack(-u.y, -u.x), df_pack(-w.x, w.y), df_pack(-w.y, -w.x), df_dup(v.x), df_dup(v.y)};
+    }
+    static __device__ __forceinline__ DfPair update(DfPair x, const Row& r, const Col& c) {
+        df_fma(x, r.ux, c.w1);
+        df_fma(x, r.uy, c.w2);
+        df_fma(x, r.wx, c.u1);
+        df_fma(x, r.wy, c.u2);
+        return df_norm(x);
+    }
+    static __device__ __forceinline__ void real(DfPair& x) {
+        x.hi &= 0xffffffffull;
+        x.lo &= 0xffffffffull;
+    }
+    static __device__ __forceinline__ void row_add(Sum& s, const DfPair& x, const Col& c, bool first) {
+        if (first) {
+            s.x.hi = df_mul(x, c.vx, s.x.lo);
+            s.y.hi = df_mul(x, c.vy, s.y.lo);
+        } else {
+            df_fma(s.x, x, c.vx);
+            df_fma(s.y, x, c.vy);
+        }
+    }
+    static __device__ __forceinline__ void col_add(Sum& s, const DfPair& x, const Row& r) {
+        df_fma(s.x, x, r.vx);
+        df_fma(s.y, x, r.vy);
+    }
+    static __device__ __forceinline__ void save_row(DfPair* m, const Sum& s) {
+        m[0] = s.x;
+        m[32] = s.y;
+    }
+    static __device__ __forceinline__ dfl2 row_total(const DfPair* m, int n, int stride) {
+        Sum s{m[0], m[32]};
+        for (int j = 1; j < n; ++j) {
+            const DfPair a = m[j * stride], b = m[j * stride + 32];
+            df_add(s.x, a.hi, a.lo);
+            df_add(s.y, b.hi, b.lo);
+        }
+        const dfl2 x = fs_get(df_norm(s.x)), y = fs_get(df_norm(s.y));
+        return mk(x.x - y.y, x.y + y.x);
+    }
+    static __device__ __forceinline__ dfl2 col_total(const Sum& s) {
+        const dfl2 x = fs_get(df_norm(s.x)), y = fs_get(df_norm(s.y));
+        return mk(x.x + y.y, y.x - x.y);
+    }
+};
 
 // The built FP64 matrix rewritten in place as double-float pairs.
 __global__ void k_fs_to_dfl(double2* A, int64_t count) {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < count; i += (int64_t)gridDim.x * blockDim.x) {
         const double2 x = A[i];
-        reinterpret_cast<dfl2*>(A)[i] = mk(dfl(x.x), dfl(x.y));
+        fs_put(reinterpret_cast<DfPair*>(A)[i], mk(dfl(x.x), dfl(x.y)));
     }
 }
 
@@ -94,7 +283,7 @@ __global__ void k_fs_to_dfl(double2* A, int64_t count) {
 // its first entry is stored at index k+1 like the others.
 template <typename R>
 struct FsArgs {
-    using C = cplx_t<R>;
+    using C = fs_mem<R>;
     int n;
     C* A;
     const C* U;   // v_{k-1} (zero at k = 0)
@@ -102,157 +291,212 @@ struct FsArgs {
     C* Vn;        // v_{k+1}, written by the scalar phase of step k
     const C* W;   // w_{k-1} (zero at k = 0)
     C* Wn;        // w_k, written by the scalar phase of step k
-    C* pr;        // [T][n] row partial sums of A v_k, by tile column
-    C* pc;        // [T][n] column partial sums, by tile row
+    C* pr;        // [strips][n]  row partial sums of A v_k, by strip
+    C* pc;        // [chunks][n]  column partial sums, by chunk of the column's strip
     C* p;         // [n]    tau A v_k
-    R* red;       // [blocks of the reduction] partial sums of Re(v^H p)
     R* tau;       // [2]    tau_k in tau[k & 1]
     double* d;    // [n]
     double* e2;   // [n]
 };
 
-// Step k's pass over the trailing block (rows and columns j0 = k+1 .. n-1),
-// one 64 x 64 tile of its lower triangle per CTA: A <- A - u w^H - w u^H
-// with step k-1's (u, w), then the tile's row sums of A v (into pr[tile
-// column][row]) and, below the diagonal, column sums of A^H v (into
-// pc[tile row][column]).  Warp q takes rows q, q+8, ...; lanes take columns
-// lane and lane + 32 of the tile.  The tile's row entries of u, w and v are
-// staged in shared memory, and a warp loads its next row's elements before
-// it updates the current one (the pass is bound by instruction issue once
-// the loads are in flight early).  Each lane's row partials go to shared
-// memory and four threads per row add them up (eight each, then across the
-// four), in a fixed order.
-constexpr int FS_RS_LD = 33;  // row stride of the row partials (16-byte entries)
+// Chunks of a strip (64 columns) of `rows` rows, q rows each.
+__host__ __device__ __forceinline__ int fs_chunks(int rows, int q) { return (rows + q - 1) / q; }
+
+__device__ __forceinline__ void fs_copy16(void* smem, const void* gmem) {
+    const unsigned d = (unsigned)__cvta_generic_to_shared(smem);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(gmem) : "memory");
+}
+// The launches of the reduction follow one another with programmatic dependence:
+// a kernel starts while its predecessor drains and waits here for its results.
+__device__ __forceinline__ void fs_launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void fs_wait_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// Step k's pass over the trailing block (rows and columns j0 = k+1 .. n-1): A <-
+// A - u w^H - w u^H with step k-1's (u, w), then row sums of A v (into
+// pr[strip][row]) and, below the diagonal, column sums of A^H v (into
+// pc[chunk][column]).  The lower triangle is cut into strips of 64 columns and
+// each strip into chunks of q rows, one per CTA; q is the smallest multiple of
+// eight for which the chunks fit on the chip at once, so that every step is one
+// wave of nearly equal CTAs however large its block is (64 x 64 tiles left a
+// second wave of 40 tiles at order 1950, and one tile per SM at order 1050).
+// Warp w takes rows w, w+8, ... of its chunk; lanes take columns lane and lane +
+// 32.  A warp copies its rows' elements and their entries of u, w and v to its
+// own part of shared memory two groups of four rows ahead; a consumed element's
+// place takes the lane's row partial, and eight lanes per row add these up, in a
+// fixed order.
+// In double-float bound by the FP32 pipe (55 % issue, most of it two-wide): 232
+// instructions an element, 362 with scalar arithmetic, 23 against 29 us at order
+// 1950; 10 us at order 1050 and 5.5 at 150, most of it latency.  Two CTAs per SM
+// leave the 128 registers that the columns' operands take.
+template <typename R> struct FsPassBuf {
+    fs_mem<R> x[2][FS_GROUP][FS_TB];
+    fs_mem<R> uwv[2][FS_GROUP][3];
+};
 template <typename R>
-__global__ void __launch_bounds__(FS_PASS_THREADS, 3) k_fs_pass(FsArgs<R> a, int k) {
+__global__ void __launch_bounds__(FS_PASS_THREADS, FS_PASS_CTAS) k_fs_pass(FsArgs<R> a, int k, int q) {
     using C = cplx_t<R>;
-    __shared__ C rsum[FS_TB][FS_RS_LD];
-    __shared__ C csum[FS_PASS_THREADS / 32][FS_TB];
-    __shared__ C svec[3][FS_TB];
+    using M = fs_mem<R>;
+    using Op = FsOps<R>;
+    extern __shared__ __align__(16) unsigned char fs_smem[];
+    FsPassBuf<R>* const bufs = reinterpret_cast<FsPassBuf<R>*>(fs_smem);
     const int n = a.n, j0 = k + 1, m = n - j0;
-    const int64_t b = blockIdx.x;
-    int TR = (int)((sqrtf(8.f * (float)b + 1.f) - 1.f) * 0.5f);  // corrected below
-    while (tri64(TR + 1) <= b) ++TR;
-    while (tri64(TR) > b) --TR;
-    const int TC = (int)(b - tri64(TR));
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const R r0 = fs_r<R>(0.f);
-    const C zero = mk(r0, r0);
+    fs_launch_next();
+    // strip and chunk of this CTA: a scan over the strips' chunk counts
+    int strip = 0, chunk = 0;
+    for (int base = 0, before = 0;; base += 32) {
+        const int rows = m - FS_TB * (base + lane);
+        int incl = rows > 0 ? fs_chunks(rows, q) : 0;
+        const int own = incl;
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const int t = __shfl_up_sync(FULL_MASK, incl, o);
+            if (lane >= o) incl += t;
+        }
+        const unsigned hit = __ballot_sync(FULL_MASK, (int)blockIdx.x < before + incl);
+        const int f = hit ? __ffs(hit) - 1 : 31;
+        if (hit) {
+            strip = base + f;
+            chunk = (int)blockIdx.x - before - __shfl_sync(FULL_MASK, incl - own, f);
+            break;
+        }
+        before += __shfl_sync(FULL_MASK, incl, 31);
+        if (base > m) return;  // past the last strip: not reached with the host's grid
+    }
+    const int c0 = FS_TB * strip, r0 = c0 + chunk * q, r1 = min(m, r0 + q);
+    FsPassBuf<R>& buf = bufs[warp];
+    const R z = fs_r<R>(0.f);
+    const C zero = mk(z, z);
+    M zero_m;
+    fs_put(zero_m, zero);
     int cr[2];
-    C vc[2], uc[2], wc[2], cacc[2];
 #pragma unroll
-    for (int q = 0; q < 2; ++q) {
-        cr[q] = FS_TB * TC + lane + 32 * q;
-        const bool in = cr[q] < m;
-        const int j = j0 + cr[q];
-        vc[q] = in ? a.V[j] : zero;
-        uc[q] = in ? a.U[j] : zero;
-        wc[q] = in ? a.W[j] : zero;
-        cacc[q] = zero;
-    }
-    // the tile's row entries of u, w and v, staged once
-    for (int t = threadIdx.x; t < 3 * FS_TB; t += FS_PASS_THREADS) {
-        const int r = t % FS_TB, ri = FS_TB * TR + r;
-        const C* src = t < FS_TB ? a.U : (t < 2 * FS_TB ? a.W : a.V);
-        svec[t / FS_TB][r] = ri < m ? src[j0 + ri] : zero;
-    }
-    __syncthreads();
-    // the next row's elements are loaded before the current row is updated
-    C xa[2], xb[2] = {zero, zero};
-    {
-        const int ri = FS_TB * TR + warp;
-        const C* row = a.A + tri64(j0 + ri) + j0;
+    for (int h = 0; h < 2; ++h) cr[h] = c0 + lane + 32 * h;
+    const int nrow = r0 + warp < r1 ? (r1 - r0 - warp + FS_PASS_WARPS - 1) / FS_PASS_WARPS : 0;
+    // offset of row ri (of the block) in A: below 2^32 elements for every order
+    auto row_at = [&](int ri) { return (uint32_t)(j0 + ri) * (uint32_t)(j0 + ri + 1) / 2 + j0; };
+    // group g of this warp's rows: warp + 8 (4 g + r) of the chunk
+    auto fetch = [&](int g) {
 #pragma unroll
-        for (int q = 0; q < 2; ++q) xa[q] = (ri < m && cr[q] <= ri) ? row[cr[q]] : zero;
-    }
-    for (int rr = warp; rr < FS_TB; rr += FS_PASS_THREADS / 32) {
-        const int ri = FS_TB * TR + rr;
-        if (ri >= m) break;
-        const int rn = ri + FS_PASS_THREADS / 32;
-        if (rr + FS_PASS_THREADS / 32 < FS_TB && rn < m) {
-            const C* rown = a.A + tri64(j0 + rn) + j0;
+        for (int r = 0; r < FS_GROUP; ++r) {
+            const int ri = r0 + warp + FS_PASS_WARPS * (FS_GROUP * g + r);
+            if (ri < r1) {
+                const M* row = a.A + row_at(ri);
 #pragma unroll
-            for (int q = 0; q < 2; ++q) xb[q] = cr[q] <= rn ? rown[cr[q]] : zero;
-        }
-        const C ui = svec[0][rr], wi = svec[1][rr], vi = svec[2][rr];
-        C* row = a.A + tri64(j0 + ri) + j0;
-        C racc = zero;
-#pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            const int c = cr[q];
-            if (c <= ri) {
-                C x = xa[q];
-                x = cfms_conj_b(ui, wc[q], x);
-                x = cfms_conj_b(wi, uc[q], x);
-                if (c == ri) x.y = r0;  // the diagonal stays real
-                row[c] = x;
-                racc = cfma(x, vc[q], racc);
-                if (c < ri) cacc[q] = cfma_conj_a(x, vi, cacc[q]);
+                for (int h = 0; h < 2; ++h)
+                    if (cr[h] <= ri) fs_copy16(&buf.x[g & 1][r][lane + 32 * h], row + cr[h]);
+                if (lane < 3) fs_copy16(&buf.uwv[g & 1][r][lane], (lane == 0 ? a.U : lane == 1 ? a.W : a.V) + j0 + ri);
             }
-            xa[q] = xb[q];
         }
-        rsum[rr][lane] = racc;
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    fs_wait_previous();
+    fetch(0);
+    fetch(1);
+    typename Op::Col col[2];
+    typename Op::Sum csum[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const bool in = cr[h] < m;
+        const int j = j0 + cr[h];
+        col[h] = Op::col(in ? fs_get(a.U[j]) : zero, in ? fs_get(a.W[j]) : zero, in ? fs_get(a.V[j]) : zero);
+        csum[h] = Op::zero();
     }
-    csum[warp][lane] = cacc[0];
-    csum[warp][lane + 32] = cacc[1];
+    for (int g = 0; FS_GROUP * g < nrow; ++g) {
+        asm volatile("cp.async.wait_group 1;" ::: "memory");
+        __syncwarp();
+        const int nr = min(FS_GROUP, nrow - FS_GROUP * g);
+        for (int r = 0; r < nr; ++r) {
+            const int ri = r0 + warp + FS_PASS_WARPS * (FS_GROUP * g + r);
+            const typename Op::Row rw = Op::row(buf.uwv[g & 1][r]);
+            M* row = a.A + row_at(ri);
+            typename Op::Sum rsum = Op::zero();
+            if (ri >= c0 + FS_TB) {  // below the strip's diagonal block: every lane, no conditions
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const M x = Op::update(buf.x[g & 1][r][lane + 32 * h], rw, col[h]);
+                    row[cr[h]] = x;
+                    Op::row_add(rsum, x, col[h], h == 0);
+                    Op::col_add(csum[h], x, rw);
+                }
+            } else {
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    if (cr[h] <= ri) {
+                        M x = Op::update(buf.x[g & 1][r][lane + 32 * h], rw, col[h]);
+                        if (cr[h] == ri) Op::real(x);  // the diagonal stays real
+                        row[cr[h]] = x;
+                        Op::row_add(rsum, x, col[h], h == 0);
+                        if (cr[h] < ri) Op::col_add(csum[h], x, rw);
+                    }
+                }
+            }
+            Op::save_row(&buf.x[g & 1][r][lane], rsum);
+        }
+        __syncwarp();
+        {
+            const int r = lane >> 3, part = lane & 7;
+            M sum = zero_m;
+            if (r < nr) fs_put(sum, Op::row_total(&buf.x[g & 1][r][part], 4, 8));
+#pragma unroll
+            for (int o = 1; o < 8; o <<= 1) fs_acc(sum, fs_xor(sum, o));
+            if (part == 0 && r < nr)
+                fs_put(a.pr[(int64_t)strip * n + r0 + warp + FS_PASS_WARPS * (FS_GROUP * g + r)], fs_sum(sum));
+        }
+        __syncwarp();
+        fetch(g + 2);
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncwarp();
+#pragma unroll
+    for (int h = 0; h < 2; ++h) fs_put(buf.x[0][0][lane + 32 * h], Op::col_total(csum[h]));
     __syncthreads();
-    {
-        const int rr = threadIdx.x >> 2, part = threadIdx.x & 3, ri = FS_TB * TR + rr;
-        C sum = zero;
-        if (ri < m) {
-            sum = rsum[rr][part];
-#pragma unroll
-            for (int j = 1; j < 8; ++j) sum = cadd(sum, rsum[rr][part + 4 * j]);
-        }
-        sum = cadd(sum, cshfl_xor(sum, 1));
-        sum = cadd(sum, cshfl_xor(sum, 2));
-        if (part == 0 && ri < m) a.pr[(int64_t)TC * n + ri] = sum;
-    }
     if (threadIdx.x < FS_TB) {
-        C sum = csum[0][threadIdx.x];
+        M sum = bufs[0].x[0][0][threadIdx.x];
 #pragma unroll
-        for (int w = 1; w < FS_PASS_THREADS / 32; ++w) sum = cadd(sum, csum[w][threadIdx.x]);
-        const int c = FS_TB * TC + threadIdx.x;
-        if (c < m) a.pc[(int64_t)TR * n + c] = sum;
+        for (int w = 1; w < FS_PASS_WARPS; ++w) fs_acc(sum, bufs[w].x[0][0][threadIdx.x]);
+        const int c = c0 + threadIdx.x;
+        if (c < m) fs_put(a.pc[(int64_t)chunk * n + c], fs_sum(sum));
     }
 }
 
-// p = tau (A v): for row ri of band B (its tile row), the row partials of
-// tiles (B, 0 .. B) plus the column partials of tiles (B .. T-1, B) (the
-// diagonal tile's column sums hold the elements below the diagonal); and
-// each CTA's partial sum of Re(v^H p).  A CTA takes 32 consecutive rows, one
-// per lane; warp q adds the partials q, q+8, ... of that list, and warp 0
-// adds the eight warps' sums, in a fixed order.
+// Partial `j` of row ri of A v: the row partials of strips 0 .. band (the row's own
+// band), then the column partials of the band's chunks (a diagonal block's column
+// sums hold the elements below the diagonal).
+template <typename R> __device__ __forceinline__ fs_mem<R> fs_partial(const FsArgs<R>& a, int j, int band, int ri) {
+    const fs_mem<R>* src = j <= band ? a.pr + (int64_t)j * a.n : a.pc + (int64_t)(j - band - 1) * a.n;
+    return src[ri];
+}
+
+// p = tau (A v) of large blocks, spread over the chip.  A CTA takes 32 consecutive
+// rows, one per lane; warp q adds the partials q, q+8, ..., and warp 0 adds the
+// eight warps' sums, in a fixed order.
 template <typename R>
-__global__ void __launch_bounds__(FS_RED_THREADS) k_fs_reduce(FsArgs<R> a, int k) {
+__global__ void __launch_bounds__(FS_RED_THREADS) k_fs_reduce(FsArgs<R> a, int k, int q) {
     using C = cplx_t<R>;
-    __shared__ C part[FS_RED_THREADS / 32][FS_RED_ROWS];
-    const int n = a.n, j0 = k + 1, m = n - j0, T = (m + FS_TB - 1) / FS_TB;
+    using M = fs_mem<R>;
+    __shared__ M part[FS_RED_THREADS / 32][FS_RED_ROWS];
+    const int n = a.n, j0 = k + 1, m = n - j0;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int ri = blockIdx.x * FS_RED_ROWS + lane;
-    const R r0 = fs_r<R>(0.f);
-    C s = mk(r0, r0);
+    const R z = fs_r<R>(0.f);
+    M s;
+    fs_put(s, mk(z, z));
+    fs_launch_next();
+    fs_wait_previous();
     if (ri < m) {
-        const int band = ri / FS_TB;
-        for (int q = warp; q <= T; q += FS_RED_THREADS / 32)
-            s = cadd(s, q <= band ? a.pr[(int64_t)q * n + ri] : a.pc[(int64_t)(q - 1) * n + ri]);
+        const int band = ri / FS_TB, np = band + 1 + fs_chunks(m - FS_TB * band, q);
+#pragma unroll 4
+        for (int j = warp; j < np; j += FS_RED_THREADS / 32) fs_acc(s, fs_partial(a, j, band, ri));
     }
     part[warp][lane] = s;
     __syncthreads();
-    if (warp != 0) return;
+    if (warp != 0 || ri >= m) return;
 #pragma unroll
-    for (int w = 1; w < FS_RED_THREADS / 32; ++w) s = cadd(s, part[w][lane]);
-    R sp = r0;
-    if (ri < m) {
-        const R tau = a.tau[k & 1];
-        s.x = s.x * tau;
-        s.y = s.y * tau;
-        a.p[j0 + ri] = s;
-        const C v = a.V[j0 + ri];
-        sp = v.x * s.x + v.y * s.y;
-    }
-    sp = warp_sum<R>(sp);
-    if (lane == 0) a.red[blockIdx.x] = sp;
+    for (int w = 1; w < FS_RED_THREADS / 32; ++w) fs_acc(s, part[w][lane]);
+    const R tau = a.tau[k & 1];
+    const C t = fs_sum(s);
+    fs_put(a.p[j0 + ri], mk(t.x * tau, t.y * tau));
 }
 
 // Sum over the FS_SCALAR_THREADS threads of a scalar-phase CTA; every thread
@@ -276,64 +520,202 @@ __global__ void __launch_bounds__(FS_SCALAR_THREADS) k_fs_setup(FsArgs<R> a) {
     const int n = a.n;
     R s2 = fs_r<R>(0.f);
     for (int i = 1 + threadIdx.x; i < n; i += blockDim.x) {
-        const C x = a.A[tri64(i)];
+        const C x = fs_get(a.A[tri64(i)]);
         s2 = s2 + cabs2(x);
-        if (i >= 2) a.Vn[i] = x;
+        if (i >= 2) fs_put(a.Vn[i], x);
         if (i == 1) s_x0 = x;
     }
     s2 = fs_block_sum<R>(s2, red);
     if (threadIdx.x == 0) {
-        a.d[0] = fs_d(a.A[0].x);
+        a.d[0] = fs_d(fs_get(a.A[0]).x);
         a.e2[0] = fs_d(s2);
         C f;
         R tau;
         reflector_head<R>(s2, s_x0, f, tau);
-        a.Vn[1] = f;
+        fs_put(a.Vn[1], f);
         a.tau[0] = tau;
     }
 }
 
-// Step k's scalar phase (one CTA): w = p - (tau/2)(v^H p) v; the explicit
-// update of pivot column j0 = k+1 with (v_k, w_k); d_j0, e2_j0 and, unless
-// this was the last reflector, the next reflector v_{k+1} and tau_{k+1}.
-template <typename R>
-__global__ void __launch_bounds__(FS_SCALAR_THREADS) k_fs_scalar(FsArgs<R> a, int k, int nred) {
-    using C = cplx_t<R>;
-    __shared__ R red[FS_SCALAR_THREADS / 32];
-    __shared__ R s_K;
-    __shared__ C s_x0;
-    const int n = a.n, j0 = k + 1;
-    R sp = fs_r<R>(0.f);
-    for (int b = threadIdx.x; b < nred; b += blockDim.x) sp = sp + a.red[b];
-    sp = fs_block_sum<R>(sp, red);
-    if (threadIdx.x == 0) s_K = fs_r<R>(0.5f) * a.tau[k & 1] * sp;
-    __syncthreads();
-    const R K = s_K;
-    const C vf = a.V[j0];
-    const C p0 = a.p[j0];
-    const C w0 = mk(p0.x - K * vf.x, p0.y - K * vf.y);
-    R s2 = fs_r<R>(0.f);
-    for (int i = j0 + threadIdx.x; i < n; i += blockDim.x) {
-        const C v = a.V[i], pi = a.p[i];
-        const C w = mk(pi.x - K * v.x, pi.y - K * v.y);
-        a.Wn[i] = w;
-        C x = a.A[tri64(i) + j0];
-        x = cfms_conj_b(v, w0, x);
-        x = cfms_conj_b(w, vf, x);
-        if (i == j0) a.d[j0] = fs_d(x.x);
-        if (i >= j0 + 1) s2 = s2 + cabs2(x);
-        if (i >= j0 + 2) a.Vn[i] = x;
-        if (i == j0 + 1) s_x0 = x;
+// Step k's scalar phase: p = tau A v (its partials added up here, or by
+// k_fs_reduce: `reduced`); w = p - (tau/2)(v^H p) v; the explicit update of pivot
+// column j0 = k+1 with (v_k, w_k); d_j0, e2_j0 and, unless this was the last
+// reflector, the next reflector v_{k+1} and tau_{k+1}.
+// One cluster of eight CTAs: the two sums over all rows that it needs (v^H p and
+// the next column's norm) cross between the CTAs through distributed shared memory
+// and the hardware's cluster barrier.  Bound by latency: the loads of the partials
+// (1 MB at order 1950, in flight at once), two barriers and the reflector's head.
+// 9.3 us at order 1950, 7.4 at 150, where a reduction over the chip and one CTA
+// took 16.
+// CTA r takes blocks r, r + 8, ... of 256 rows: four threads of four warps add a
+// row's partials, one of them keeps the row.
+template <typename R> struct FsXch {
+    R sum[2][FS_CL];
+    cplx_t<R> p0;
+};
+__device__ __forceinline__ void fs_cluster_arrive() {
+    __syncwarp();
+    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
+}
+__device__ __forceinline__ void fs_cluster_wait() {
+    __syncwarp();
+    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// 16 or 8 bytes into the same place of CTA `rank`'s shared memory.
+__device__ __forceinline__ unsigned fs_remote(const void* p, int rank) {
+    unsigned d;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(d) : "r"((unsigned)__cvta_generic_to_shared(p)), "r"(rank));
+    return d;
+}
+__device__ __forceinline__ void fs_remote_store(void* p, int rank, double v) {
+    asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(fs_remote(p, rank)), "d"(v) : "memory");
+}
+__device__ __forceinline__ void fs_remote_store(void* p, int rank, dfl v) {
+    asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(fs_remote(p, rank)), "f"(v.hi), "f"(v.lo) : "memory");
+}
+// Sum over the cluster's row-keeping threads (warps 0 .. 7 of each CTA) of v, into
+// every CTA's x.sum[which]; the caller passes the cluster barrier before it reads it.
+template <typename R> __device__ __forceinline__ void fs_cluster_sum(R v, R* red, FsXch<R>& x, int which, int rank) {
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    if (warp < FS_STEP_ROWS / 32) {
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) fs_acc(v, shfl_xor_r(v, o));
+        if (lane == 0) red[warp] = v;
     }
-    s2 = fs_block_sum<R>(s2, red);
-    if (threadIdx.x == 0) {
+    __syncthreads();
+    if (warp == 0) {
+        v = red[lane % (FS_STEP_ROWS / 32)];
+#pragma unroll
+        for (int o = FS_STEP_ROWS / 64; o > 0; o >>= 1) fs_acc(v, shfl_xor_r(v, o));
+        if (lane < FS_CL) fs_remote_store(&x.sum[which][rank], lane, fs_sum(v));
+    }
+}
+template <typename R> __device__ __forceinline__ R fs_sum8(const R* s) {
+    R a = s[0], b = s[2], c = s[4], d = s[6];
+    fs_acc(a, s[1]);
+    fs_acc(b, s[3]);
+    fs_acc(c, s[5]);
+    fs_acc(d, s[7]);
+    fs_acc(a, b);
+    fs_acc(c, d);
+    fs_acc(a, c);
+    return fs_sum(a);
+}
+template <typename R>
+__global__ void __cluster_dims__(FS_CL, 1, 1) __launch_bounds__(FS_STEP_THREADS) k_fs_step(FsArgs<R> a, int k, int q,
+                                                                                         bool reduced) {
+    using C = cplx_t<R>;
+    using M = fs_mem<R>;
+    __shared__ M part[FS_STEP_PARTS][FS_STEP_ROWS];
+    __shared__ R red[2][FS_STEP_ROWS / 32];
+    __shared__ FsXch<R> xch;
+    __shared__ C s_p0;
+    const int n = a.n, j0 = k + 1, m = n - j0, rank = blockIdx.x;
+    const int slot = threadIdx.x % FS_STEP_ROWS, pt = threadIdx.x / FS_STEP_ROWS;
+    const bool keeper = pt == 0;
+    const R z = fs_r<R>(0.f);
+    const C zero = mk(z, z);
+    fs_launch_next();
+    fs_cluster_arrive();  // every CTA runs before any writes into another's memory
+    fs_wait_previous();
+    const R tau = a.tau[k & 1];
+    // the first block's entries, loaded ahead of the partials
+    const int ri0 = rank * FS_STEP_ROWS + slot;
+    C v1 = zero, x1 = zero, p1 = zero;
+    if (keeper && ri0 < m) {
+        v1 = fs_get(a.V[j0 + ri0]);
+        x1 = fs_get(a.A[tri64(j0 + ri0) + j0]);
+    }
+    const C vf = fs_get(a.V[j0]);
+    R sp = z;
+    for (int rb = ri0 - slot; rb < m; rb += FS_CL * FS_STEP_ROWS) {
+        const int ri = rb + slot;
+        const bool first = ri == ri0;
+        C s = zero;
+        M acc;
+        fs_put(acc, zero);
+        if (!reduced) {
+            if (ri < m) {
+                const int band = ri / FS_TB, np = band + 1 + fs_chunks(m - FS_TB * band, q);
+#pragma unroll 4
+                for (int j = pt; j < np; j += FS_STEP_PARTS) fs_acc(acc, fs_partial(a, j, band, ri));
+            }
+            part[pt][slot] = acc;
+            __syncthreads();
+        }
+        if (keeper && ri < m) {
+            if (reduced) {
+                s = fs_get(a.p[j0 + ri]);
+            } else {
+#pragma unroll
+                for (int t = 1; t < FS_STEP_PARTS; ++t) fs_acc(acc, part[t][slot]);
+                s = fs_sum(acc);
+                s = mk(s.x * tau, s.y * tau);
+                if (!first) fs_put(a.p[j0 + ri], s);
+            }
+            const C v = first ? v1 : fs_get(a.V[j0 + ri]);
+            sp = sp + (v.x * s.x + v.y * s.y);
+            if (first) p1 = s;
+            if (ri == 0) s_p0 = s;
+        }
+        if (!reduced) __syncthreads();
+    }
+    fs_cluster_wait();
+    fs_cluster_sum<R>(sp, red[0], xch, 0, rank);  // (its __syncthreads covers s_p0)
+    if (rank == 0 && threadIdx.x < 2 * FS_CL) {
+        const int to = threadIdx.x >> 1;
+        if (threadIdx.x & 1) fs_remote_store(&xch.p0.y, to, s_p0.y);
+        else fs_remote_store(&xch.p0.x, to, s_p0.x);
+    }
+    fs_cluster_arrive();
+    fs_cluster_wait();
+    const R K = fs_r<R>(0.5f) * tau * fs_sum8(xch.sum[0]);
+    const C p0 = xch.p0;
+    const C w0 = mk(p0.x - K * vf.x, p0.y - K * vf.y);
+    R s2 = z;
+    C w1 = zero;
+    if (keeper) {
+        for (int ri = ri0; ri < m; ri += FS_CL * FS_STEP_ROWS) {
+            const bool first = ri == ri0;
+            const int i = j0 + ri;
+            const C v = first ? v1 : fs_get(a.V[i]), pi = first ? p1 : fs_get(a.p[i]);
+            const C w = mk(pi.x - K * v.x, pi.y - K * v.y);
+            if (first) w1 = w;
+            else fs_put(a.Wn[i], w);
+            C x = first ? x1 : fs_get(a.A[tri64(i) + j0]);
+            x = cfms_conj_b(v, w0, x);
+            x = cfms_conj_b(w, vf, x);
+            if (ri >= 1) s2 = s2 + cabs2(x);
+            if (first) x1 = x;
+            else fs_put(a.Vn[i], x);
+        }
+    }
+    fs_cluster_sum<R>(s2, red[1], xch, 1, rank);
+    fs_cluster_arrive();
+    // the first block's results go out while the barrier fills (ahead of it, its
+    // release would wait for them)
+    if (keeper && ri0 < m) {
+        fs_put(a.Wn[j0 + ri0], w1);
+        if (ri0 >= 2) fs_put(a.Vn[j0 + ri0], x1);
+        if (ri0 == 0) a.d[j0] = fs_d(x1.x);
+    }
+    // row j0 + 1's keeper forms the reflector's head (reflector_head), the part
+    // without the norm first
+    const bool head = rank == 0 && threadIdx.x == 1;
+    R ax0 = z;
+    C ph = zero;
+    if (head) {
+        ax0 = sqroot(cabs2(x1));
+        ph = ax0 > z ? mk(x1.x / ax0, x1.y / ax0) : mk(fs_r<R>(1.f), z);
+    }
+    fs_cluster_wait();
+    if (head) {
+        s2 = fs_sum8(xch.sum[1]);
         a.e2[j0] = fs_d(s2);
         if (k + 1 <= n - 3) {
-            C f;
-            R tau;
-            reflector_head<R>(s2, s_x0, f, tau);
-            a.Vn[j0 + 1] = f;
-            a.tau[(k + 1) & 1] = tau;
+            const R sigma = sqroot(s2);
+            fs_put(a.Vn[j0 + 1], mk(x1.x + ph.x * sigma, x1.y + ph.y * sigma));
+            a.tau[(k + 1) & 1] = sigma > z ? fs_r<R>(1.f) / (sigma * (sigma + ax0)) : z;
         }
     }
 }
@@ -343,8 +725,8 @@ __global__ void __launch_bounds__(FS_SCALAR_THREADS) k_fs_scalar(FsArgs<R> a, in
 template <typename R>
 __global__ void k_fs_finish(FsArgs<R> a) {
     const int n = a.n;
-    const auto v = a.V[n - 1], w = a.W[n - 1];
-    a.d[n - 1] = fs_d(a.A[tri64(n - 1) + n - 1].x - fs_r<R>(2.f) * (v.x * w.x + v.y * w.y));
+    const auto v = fs_get(a.V[n - 1]), w = fs_get(a.W[n - 1]);
+    a.d[n - 1] = fs_d(fs_get(a.A[tri64(n - 1) + n - 1]).x - fs_r<R>(2.f) * (v.x * w.x + v.y * w.y));
 }
 
 // Gershgorin bracket and Sturm-count guards of the tridiagonal (d, e2), and
@@ -405,21 +787,54 @@ __global__ void __launch_bounds__(FS_EIG_THREADS) k_fs_eig(int n, const float* _
     eig[k] = eig_df_bracketed(n, df, dlo, e2f, e2lo, k, a, b, 8.0 * FLT_EPSILON * nrm, lo, hi, pivminf, nrm);
 }
 
+// Rows of a chunk of the pass over a block of order m, and the chunks' number.
+struct FsPlan { int q, chunks; };
+static FsPlan fs_plan(int m, int slots) {
+    auto count = [&](int q) {
+        int c = 0;
+        for (int rows = m; rows > 0; rows -= FS_TB) c += fs_chunks(rows, q);
+        return c;
+    };
+    const int64_t rows = (int64_t)m * ((m + FS_TB - 1) / FS_TB) / 2;
+    int q = std::clamp((int)(rows / slots) / 8 * 8, FS_MIN_ROWS, FS_MAX_ROWS), c = count(q);
+    while (q < FS_MAX_ROWS && c > slots) c = count(q += 8);
+    return {q, c};
+}
+// Blocks above this order have their partials added up by k_fs_reduce: the step
+// cluster's eight SMs read 16 bytes per row and partial, 1 MB at order 2000.
+constexpr int FS_FUSED_MAX = 4096;
+
+// A launch that may start while its predecessor on the stream drains (the kernel
+// waits for it before it reads or writes anything).
+template <typename... P, typename... A>
+static cudaError_t fs_launch(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, A... args) {
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 // Reduction of the packed matrix A (in R's complex form) to the real
 // tridiagonal (d, e2), enqueued on st.  The buffers are those of FsArgs, as
 // raw device memory; v_k sits in vb[k mod 3] and w_k in wb[k mod 2], and
 // v_{-1} = vb[2] and w_{-1} = wb[1] start at zero.
 template <typename R>
-static cudaError_t fs_tridiagonalise(int n, void* A, void* vb_, void* wb_, void* pr, void* pc, void* p, void* red,
-                                     void* tau, double* d, double* e2, cudaStream_t st) {
-    using C = cplx_t<R>;
+static cudaError_t fs_tridiagonalise(int n, int slots, void* A, void* vb_, void* wb_, void* pr, void* pc, void* p, void* tau,
+                                     double* d, double* e2, cudaStream_t st) {
+    using C = fs_mem<R>;
     FsArgs<R> a;
     a.n = n;
     a.A = static_cast<C*>(A);
     a.pr = static_cast<C*>(pr);
     a.pc = static_cast<C*>(pc);
     a.p = static_cast<C*>(p);
-    a.red = static_cast<R*>(red);
     a.tau = static_cast<R*>(tau);
     a.d = d;
     a.e2 = e2;
@@ -438,20 +853,24 @@ static cudaError_t fs_tridiagonalise(int n, void* A, void* vb_, void* wb_, void*
     a.W = wb + n;
     a.V = vb;
     a.Wn = wb;
+    const size_t smem = FS_PASS_WARPS * sizeof(FsPassBuf<R>);
+    cudaError_t e = cudaFuncSetAttribute(k_fs_pass<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
     k_fs_setup<R><<<1, FS_SCALAR_THREADS, 0, st>>>(a);
-    cudaError_t e = cudaGetLastError();
+    e = cudaGetLastError();
     for (int k = 0; k <= n - 3 && e == cudaSuccess; ++k) {
-        const int mm = n - k - 1, T = (mm + FS_TB - 1) / FS_TB;
+        const int mm = n - k - 1;
+        const FsPlan pl = fs_plan(mm, slots);
+        const bool reduced = mm > FS_FUSED_MAX;
         a.U = vb + (size_t)((k + 2) % 3) * n;
         a.V = vb + (size_t)(k % 3) * n;
         a.Vn = vb + (size_t)((k + 1) % 3) * n;
         a.W = wb + (size_t)((k + 1) & 1) * n;
         a.Wn = wb + (size_t)(k & 1) * n;
-        k_fs_pass<R><<<(unsigned)tri64(T), FS_PASS_THREADS, 0, st>>>(a, k);
-        const int nred = (mm + FS_RED_ROWS - 1) / FS_RED_ROWS;
-        k_fs_reduce<R><<<nred, FS_RED_THREADS, 0, st>>>(a, k);
-        k_fs_scalar<R><<<1, FS_SCALAR_THREADS, 0, st>>>(a, k, nred);
-        e = cudaGetLastError();
+        e = fs_launch(k_fs_pass<R>, (unsigned)pl.chunks, FS_PASS_THREADS, smem, st, a, k, pl.q);
+        if (e == cudaSuccess && reduced)
+            e = fs_launch(k_fs_reduce<R>, (unsigned)((mm + FS_RED_ROWS - 1) / FS_RED_ROWS), FS_RED_THREADS, 0, st, a, k, pl.q);
+        if (e == cudaSuccess) e = fs_launch(k_fs_step<R>, FS_CL, FS_STEP_THREADS, 0, st, a, k, pl.q, reduced);
     }
     if (e != cudaSuccess) return e;
     a.V = vb + (size_t)((n - 3) % 3) * n;
@@ -471,10 +890,11 @@ extern "C" ptca_status ptca_full_spectrum(ptca_ctx* ctx, double* eig_out, void* 
     const int N = ctx->N;
     if (N > 16384) return ptca_internal_fail(PTCA_ERR_INVALID, "ptca_full_spectrum covers lattices of up to 16384 sites");
     const int n = 2 * N;
-    const int Tmax = (n - 1 + FS_TB - 1) / FS_TB;
+    const int Tmax = std::max((n - 1 + FS_TB - 1) / FS_TB, 1), slots = FS_PASS_CTAS * ctx->sms;
+    int cmax = 1;  // most chunks of a strip (its first) in any step
+    for (int mm = n - 1; mm >= 2; --mm) cmax = std::max(cmax, fs_chunks(mm, fs_plan(mm, slots).q));
     cudaError_t es = ptca_internal_settle(ctx, static_cast<cudaStream_t>(stream), true);
     if (es != cudaSuccess) return ptca_internal_fail(PTCA_ERR_CUDA, cudaGetErrorString(es));
-    const int red_max = (n + FS_RED_ROWS - 1) / FS_RED_ROWS;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
 
     std::vector<void*> owned;
@@ -493,15 +913,14 @@ extern "C" ptca_status ptca_full_spectrum(ptca_ctx* ctx, double* eig_out, void* 
     double2* vb = static_cast<double2*>(alloc(3 * (size_t)n * sizeof(double2)));
     double2* wb = static_cast<double2*>(alloc(2 * (size_t)n * sizeof(double2)));
     double2* p = static_cast<double2*>(alloc((size_t)n * sizeof(double2)));
-    double2* pr = static_cast<double2*>(alloc((size_t)(Tmax > 0 ? Tmax : 1) * n * sizeof(double2)));
-    double2* pc = static_cast<double2*>(alloc((size_t)(Tmax > 0 ? Tmax : 1) * n * sizeof(double2)));
-    double* red = static_cast<double*>(alloc((size_t)red_max * sizeof(double)));
+    double2* pr = static_cast<double2*>(alloc((size_t)Tmax * n * sizeof(double2)));
+    double2* pc = static_cast<double2*>(alloc((size_t)cmax * n * sizeof(double2)));
     double* tau = static_cast<double*>(alloc(2 * sizeof(double)));
     double* d = static_cast<double*>(alloc((size_t)n * sizeof(double)));
     double* e2 = static_cast<double*>(alloc((size_t)n * sizeof(double)));
     float* f32 = static_cast<float*>(alloc(4 * (size_t)n * sizeof(float)));
     double* prm = static_cast<double*>(alloc(4 * sizeof(double)));
-    for (void* q : {(void*)A, (void*)vb, (void*)wb, (void*)p, (void*)pr, (void*)pc, (void*)red, (void*)tau, (void*)d,
+    for (void* q : {(void*)A, (void*)vb, (void*)wb, (void*)p, (void*)pr, (void*)pc, (void*)tau, (void*)d,
                     (void*)e2, (void*)f32, (void*)prm})
         if (!q) {
             release();
@@ -526,9 +945,9 @@ extern "C" ptca_status ptca_full_spectrum(ptca_ctx* ctx, double* eig_out, void* 
         // PTCA_MIXED: the reduction in double-float
         const int64_t cnt = tri64(n) + 64;
         k_fs_to_dfl<<<(unsigned)std::min<int64_t>((cnt + 255) / 256, 152 * 16), 256, 0, st>>>(A, cnt);
-        e = fs_tridiagonalise<dfl>(n, A, vb, wb, pr, pc, p, red, tau, d, e2, st);
+        e = fs_tridiagonalise<dfl>(n, slots, A, vb, wb, pr, pc, p, tau, d, e2, st);
     } else {
-        e = fs_tridiagonalise<double>(n, A, vb, wb, pr, pc, p, red, tau, d, e2, st);
+        e = fs_tridiagonalise<double>(n, slots, A, vb, wb, pr, pc, p, tau, d, e2, st);
     }
     if (e != cudaSuccess) return fail(e, "reducing to tridiagonal form");
     float* df = f32;

@@ -94,3 +94,22 @@ def test_full_spectrum_at_order_2048_matches_lapack(precision):
     # trace and Frobenius norm of the spectrum against the matrix
     assert abs(got.sum() - np.trace(H).real) <= 1e-9 * cfg.N
     assert abs(np.sum(got ** 2) - np.sum(np.abs(H) ** 2)) <= 1e-9 * np.sum(np.abs(H) ** 2)
+
+
+# Uniform spins on an open lattice: -2 cos(k_x) - 2 cos(k_y) +- J_H with k =
+# pi i / (L + 1).  Orders at the edges of the reduction: one strip of 64 columns
+# and its neighbours, blocks of the pass above one wave, a second block of rows in
+# the step cluster (above 2048), partial sums added by their own kernel (above 4096).
+@pytest.mark.parametrize("Lx, Ly, precision", [
+    (2, 1, P.MIXED), (8, 4, P.MIXED), (8, 4, P.FP64), (11, 3, P.MIXED), (11, 3, P.FP64), (13, 10, P.MIXED),
+    (33, 32, P.MIXED), (33, 32, P.FP64), (46, 45, P.MIXED)])
+def test_full_spectrum_of_uniform_spins(Lx, Ly, precision):
+    J = 3.0
+    cfg = P.Config(Lx=Lx, Ly=Ly, L_c=2, periodic=0, J_H=J, precision=precision,
+                   schedule=P.SCHEDULE_BLOCK if min(Lx, Ly) > 1 else P.SCHEDULE_TILED)
+    got = _spectrum(cfg, np.tile([0.48, -0.6, 0.64], (cfg.N, 1)))
+    hop = np.zeros(1)
+    for L in (Lx, Ly):
+        hop = (hop[:, None] - 2.0 * np.cos(np.pi * np.arange(1, L + 1) / (L + 1))[None, :] * (L > 1)).ravel()
+    ref = np.sort(np.concatenate([hop - J, hop + J]))
+    assert np.max(np.abs(got - ref)) <= 1e-10 * 14.0
