@@ -745,13 +745,19 @@ static cudaError_t sweep_stages(ptca_ctx* ctx, int32_t n_sweeps, cudaStream_t st
             a.perm = nullptr;
             a.count_dev = nullptr;
             a.sg_dFt = nullptr;
+            if (on_determinants(ctx)) {
+                a.flag_count = ctx->d_flag_count + (g & 1);
+                a.flag_next = ctx->d_flag_count + (~g & 1);
+            }
             if (ctx->checker) e = check_stage(ctx, a, s, st);
             if (e == cudaSuccess && ctx->sg.enabled && !col) e = ptca_screen_stage(ctx, a, st);
             if (e == cudaSuccess)
                 e = launched(0, 2 * (int64_t)a.count, [&] { return launch_stage_ctx(ctx, a, st); });
             if (e == cudaSuccess && (a.margin > 0.0 || on_determinants(ctx))) {
                 e = launched(1, 0, [&] { return launch_resolve_ctx(ctx, a, st); });
-                if (e == cudaSuccess) e = cudaMemsetAsync(ctx->d_flag_count, 0, sizeof(unsigned int), st);
+                // (on determinants the re-solve clears the next stage's counter itself)
+                if (e == cudaSuccess && !on_determinants(ctx))
+                    e = cudaMemsetAsync(ctx->d_flag_count, 0, sizeof(unsigned int), st);
             }
             prev_s = s;
         }
@@ -759,6 +765,7 @@ static cudaError_t sweep_stages(ptca_ctx* ctx, int32_t n_sweeps, cudaStream_t st
     if (e == cudaSuccess && g > 0)
         e = ptca::launch_copy_sites(ctx->d_S[g & 1], ctx->d_S[(g + 1) & 1], ctx->d_sites + ctx->h_start[prev_s],
                                     ctx->h_start[prev_s + 1] - ctx->h_start[prev_s], st);
+    if (e == cudaSuccess && on_determinants(ctx)) e = cudaMemsetAsync(ctx->d_flag_count, 0, 2 * sizeof(unsigned int), st);
     if (e == cudaSuccess)
         e = captured ? ptca::launch_add_u64(ctx->d_sweep_ctr, (unsigned long long)n_sweeps, st)
                      : ptca::launch_set_u64(ctx->d_sweep_ctr, (unsigned long long)(ctx->sweeps + n_sweeps), st);

@@ -169,4 +169,9 @@ __device__ __forceinline__ void propose_spin(uint64_t seed, uint64_t sweep, uint
     sn[0] = r0 * inv; sn[1] = r1 * inv; sn[2] = r2 * inv;
 }
 
+// A chained launch (launch_chained): lets the next one start; waits until the
+// previous one, and so everything before it, is done and its writes are visible.
+__device__ __forceinline__ void launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 }  // namespace ptca

@@ -374,6 +374,7 @@ struct StageArgs {
     void* rs_scratch;
     int32_t rs_half;
     double invT;              // 1 / T (the host's: an FP64 division takes a microsecond of latency here)
+    unsigned int* flag_next;  // counter that the re-solve clears for the next stage, or null
     const double4* prop;      // proposal and ln u by lattice site for this sweep, or null
     // Delayed acceptance: work list (perm) length on the device, and the
     // stage-1 surrogate dF~ per stage index (stage 2 accepts iff

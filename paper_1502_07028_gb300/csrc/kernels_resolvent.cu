@@ -15,6 +15,8 @@ __global__ void __launch_bounds__(Tl::MAXT, Tl::MINB) k_stage_rs(const __grid_co
                                                                  bool uniform, RsMode mode, int c0) {
     extern __shared__ __align__(16) unsigned char smem[];
     __shared__ int s_task;
+    launch_next();
+    wait_previous();
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < a.prev_count + a.prev2_count; k += gridDim.x * blockDim.x) {
         const int s = k < a.prev_count ? a.prev_sites[k] : a.prev2_sites[k - a.prev_count];
         a.S_out[3 * s] = a.S_in[3 * s];
@@ -110,9 +112,8 @@ static cudaError_t launch(RsMode mode, const StageArgs& a, int c0, int sms, cuda
                 if (share > best + 0.01) { best = share; vb = v; }
             }
         }
-        k_stage_rs<Tl, kPairs><<<(a.count + vb - 1) / vb, 32 * nw, rs_layout<Tl>(vb, ms, nw, uniform, kPairs).total, st>>>(
-            a, vb, ms, uniform, mode, c0);
-        return cudaGetLastError();
+        return launch_chained(k_stage_rs<Tl, kPairs>, (a.count + vb - 1) / vb, 32 * nw,
+                              rs_layout<Tl>(vb, ms, nw, uniform, kPairs).total, st, a, vb, ms, uniform, mode, c0);
     });
 }
 

@@ -18,7 +18,12 @@ template <class Gp, bool kPairs>
 __global__ void __launch_bounds__(Gp::TPN * Gp::DFG + 32, 1) k_resolve_rs(const __grid_constant__ StageArgs a, int max_sites,
                                                                          int max_layer, RsOut<dfl>* scratch, int max_parts) {
     extern __shared__ __align__(16) unsigned char smem[];
+    // No launch_next(): the next stage's blocks, resident while these still hold
+    // their shared memory, crowd onto few SMs (32x32, 16 visits a stage: 4.9 ms a
+    // sweep instead of 3.1).  The stage does call it: 3.4 ms without chaining.
+    wait_previous();
     const int nflag = (int)*(volatile unsigned int*)a.flag_count;
+    if (a.flag_next && blockIdx.x == 0 && threadIdx.x == 0) *a.flag_next = 0;
     if (nflag == 0) return;
     int parts = (int)gridDim.x / nflag;
     parts = parts < 1 ? 1 : parts > max_parts ? max_parts : parts;
@@ -42,6 +47,8 @@ __global__ void __launch_bounds__(Tl::MAXT, Tl::MINB) k_stage_rs_few(const __gri
                                                                            int max_layer, RsOut<float>* scratch, int parts,
                                                                            RsMode mode, int c0) {
     extern __shared__ __align__(16) unsigned char smem[];
+    launch_next();
+    wait_previous();
     for (int k = blockIdx.x * blockDim.x + threadIdx.x; k < a.prev_count + a.prev2_count; k += gridDim.x * blockDim.x) {
         const int s = k < a.prev_count ? a.prev_sites[k] : a.prev2_sites[k - a.prev_count];
         a.S_out[3 * s] = a.S_in[3 * s];
@@ -116,9 +123,8 @@ cudaError_t launch_groups(RsMode mode, const StageArgs& a, int c0, int sms, cuda
         const int warps = (M + Tl::NPW - 1) / Tl::NPW;
         const int parts = std::max(1, std::min(warps, 4 * sms / a.count));
         const int threads = std::min(32 * ((warps + parts - 1) / parts) + 32, Tl::MAXT);
-        k_stage_rs_few<Tl, kPairs><<<a.count * parts, threads, rs_part_layout<E>(ms, ml, threads).total, st>>>(
-            a, ms, ml, scratch, parts, mode, c0);
-        return cudaGetLastError();
+        return launch_chained(k_stage_rs_few<Tl, kPairs>, a.count * parts, threads, rs_part_layout<E>(ms, ml, threads).total, st,
+                              a, ms, ml, scratch, parts, mode, c0);
     });
 }
 
@@ -130,9 +136,8 @@ cudaError_t launch_resolve_resolvent(const StageArgs& a, int sms, cudaStream_t s
         const auto lay = rs_part_layout<RsGroups<Gp, decltype(pairs)::value>>(ms, ml, Gp::TPN * Gp::DFG + 32);
         const size_t smem = std::max(lay.total, lay.site + rs_exact_bytes(2 * ms));
         const int grid = (Gp::TPN == 32 ? 2 : 1) * sms;   // one warp per node: two CTAs fit on an SM
-        k_resolve_rs<Gp, decltype(pairs)::value><<<grid, Gp::TPN * Gp::DFG + 32, smem, st>>>(
-            a, ms, ml, static_cast<RsOut<dfl>*>(a.rs_scratch), M);
-        return cudaGetLastError();
+        return launch_chained(k_resolve_rs<Gp, decltype(pairs)::value>, grid, Gp::TPN * Gp::DFG + 32, smem, st, a, ms, ml,
+                              static_cast<RsOut<dfl>*>(a.rs_scratch), M);
     });
 }
 

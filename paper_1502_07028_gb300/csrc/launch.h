@@ -7,6 +7,26 @@
 
 namespace ptca {
 
+// A launch that may start while its predecessor on the stream drains
+// (programmatic dependence; captured into a graph as such).  The kernel calls
+// launch_next() early and wait_previous() before it reads or writes anything that
+// another kernel touches.
+template <typename... P, typename... A>
+inline cudaError_t launch_chained(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t st,
+                                  A... args) {
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 struct Model;
 struct StageArgs;
 struct PersistArgs;

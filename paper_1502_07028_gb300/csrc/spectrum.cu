@@ -306,10 +306,6 @@ __device__ __forceinline__ void fs_copy16(void* smem, const void* gmem) {
     const unsigned d = (unsigned)__cvta_generic_to_shared(smem);
     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(d), "l"(gmem) : "memory");
 }
-// The launches of the reduction follow one another with programmatic dependence:
-// a kernel starts while its predecessor drains and waits here for its results.
-__device__ __forceinline__ void fs_launch_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-__device__ __forceinline__ void fs_wait_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // Step k's pass over the trailing block (rows and columns j0 = k+1 .. n-1): A <-
 // A - u w^H - w u^H with step k-1's (u, w), then row sums of A v (into
@@ -341,7 +337,7 @@ __global__ void __launch_bounds__(FS_PASS_THREADS, FS_PASS_CTAS) k_fs_pass(FsArg
     FsPassBuf<R>* const bufs = reinterpret_cast<FsPassBuf<R>*>(fs_smem);
     const int n = a.n, j0 = k + 1, m = n - j0;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    fs_launch_next();
+    launch_next();
     // strip and chunk of this CTA: a scan over the strips' chunk counts
     int strip = 0, chunk = 0;
     for (int base = 0, before = 0;; base += 32) {
@@ -390,7 +386,7 @@ __global__ void __launch_bounds__(FS_PASS_THREADS, FS_PASS_CTAS) k_fs_pass(FsArg
         }
         asm volatile("cp.async.commit_group;" ::: "memory");
     };
-    fs_wait_previous();
+    wait_previous();
     fetch(0);
     fetch(1);
     typename Op::Col col[2];
@@ -482,8 +478,8 @@ __global__ void __launch_bounds__(FS_RED_THREADS) k_fs_reduce(FsArgs<R> a, int k
     const R z = fs_r<R>(0.f);
     M s;
     fs_put(s, mk(z, z));
-    fs_launch_next();
-    fs_wait_previous();
+    launch_next();
+    wait_previous();
     if (ri < m) {
         const int band = ri / FS_TB, np = band + 1 + fs_chunks(m - FS_TB * band, q);
 #pragma unroll 4
@@ -615,9 +611,9 @@ __global__ void __cluster_dims__(FS_CL, 1, 1) __launch_bounds__(FS_STEP_THREADS)
     const bool keeper = pt == 0;
     const R z = fs_r<R>(0.f);
     const C zero = mk(z, z);
-    fs_launch_next();
+    launch_next();
     fs_cluster_arrive();  // every CTA runs before any writes into another's memory
-    fs_wait_previous();
+    wait_previous();
     const R tau = a.tau[k & 1];
     // the first block's entries, loaded ahead of the partials
     const int ri0 = rank * FS_STEP_ROWS + slot;
@@ -804,23 +800,6 @@ static FsPlan fs_plan(int m, int slots) {
 // cluster's eight SMs read 16 bytes per row and partial, 1 MB at order 2000.
 constexpr int FS_FUSED_MAX = 4096;
 
-// A launch that may start while its predecessor on the stream drains (the kernel
-// waits for it before it reads or writes anything).
-template <typename... P, typename... A>
-static cudaError_t fs_launch(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t st, A... args) {
-    cudaLaunchAttribute at[1];
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(block);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cfg.attrs = at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
-}
-
 // Reduction of the packed matrix A (in R's complex form) to the real
 // tridiagonal (d, e2), enqueued on st.  The buffers are those of FsArgs, as
 // raw device memory; v_k sits in vb[k mod 3] and w_k in wb[k mod 2], and
@@ -867,10 +846,10 @@ static cudaError_t fs_tridiagonalise(int n, int slots, void* A, void* vb_, void*
         a.Vn = vb + (size_t)((k + 1) % 3) * n;
         a.W = wb + (size_t)((k + 1) & 1) * n;
         a.Wn = wb + (size_t)(k & 1) * n;
-        e = fs_launch(k_fs_pass<R>, (unsigned)pl.chunks, FS_PASS_THREADS, smem, st, a, k, pl.q);
+        e = launch_chained(k_fs_pass<R>, (unsigned)pl.chunks, FS_PASS_THREADS, smem, st, a, k, pl.q);
         if (e == cudaSuccess && reduced)
-            e = fs_launch(k_fs_reduce<R>, (unsigned)((mm + FS_RED_ROWS - 1) / FS_RED_ROWS), FS_RED_THREADS, 0, st, a, k, pl.q);
-        if (e == cudaSuccess) e = fs_launch(k_fs_step<R>, FS_CL, FS_STEP_THREADS, 0, st, a, k, pl.q, reduced);
+            e = launch_chained(k_fs_reduce<R>, (unsigned)((mm + FS_RED_ROWS - 1) / FS_RED_ROWS), FS_RED_THREADS, 0, st, a, k, pl.q);
+        if (e == cudaSuccess) e = launch_chained(k_fs_step<R>, FS_CL, FS_STEP_THREADS, 0, st, a, k, pl.q, reduced);
     }
     if (e != cudaSuccess) return e;
     a.V = vb + (size_t)((n - 3) % 3) * n;
