@@ -3,9 +3,10 @@
 traveling clusters (n = 128 complex Hermitian), 30-degree cone proposals,
 t = 1, J_H = 8, mu = -6.5, T = 0.05.
 
-One step = one sweep (every site gets one proposal; 2 cluster eigensolves per
-proposal).  The headline is the mixed-precision path (FP32 reduction to
-tridiagonal form, FP64 eigenvalues and free energies); the plain FP64 GPU path
+One step = one sweep (every site gets one proposal; 2 cluster free energies per
+proposal).  The headline is the mixed-precision path (free energies from layered
+FP32 determinants at the nodes of a rational form of the Fermi functions,
+near-threshold decisions solved again in double-float); the plain FP64 GPU path
 is timed beside it on the same workload.
 
   python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
@@ -36,6 +37,11 @@ N_ORDER = 128
 # triangle once with 16 real FMA per complex element (rank-2 update + both
 # halves of the Hermitian matrix-vector product): sum_m 32 m(m+1)/2 ~ (16/3) n^3.
 HH_FLOPS = sum(32 * m * (m + 1) // 2 for m in range(1, N_ORDER))
+# Algorithmic real flops of the mixed path's free energies per cluster matrix:
+# both matrices of a visit together take about 0.42 M complex-arithmetic FMAs
+# (8 layers of 16 x 16 blocks on a ring) at each of 13 nodes (the class of
+# |mu - H| / T <= 384).
+RS_FLOPS = 13 * 2 * 0.42e6 / 2
 # DRAM bytes (read + write) per cluster matrix of each candidate dominant
 # kernel on this workload, from the ncu captures summarised under profiles/
 # (a launch's bytes / the matrices it solved; a launch's traffic is this
@@ -865,20 +871,25 @@ def main():
 
     # --- roofline of the dominant kernel: the stage kernel when a per-stage
     # pipeline is chosen, else the persistent kernel (one launch per sweep);
-    # its FP32 work is the Householder reduction.  Launches per step: one
-    # persistent launch; or the stage, dependent-visit and re-solve kernels
-    # the library timed, plus the closing counter kernel (and, one stream,
-    # the closing copy-forward kernel).
-    if kt is not None:
+    # its FP32 work is the determinants or the Householder reduction.  Launches
+    # per step: one persistent launch; the graph's stage and re-solve kernels;
+    # or the stage, dependent-visit and re-solve kernels the library timed;
+    # plus the closing counter kernel (and, one stream, the closing
+    # copy-forward kernel).
+    on_determinants = best.reduction == P.REDUCTION_ROWS and best.panel_width <= 1
+    if kt is not None and kt.stage_launches > 0:
         launches_per_step = ((kt.stage_launches + kt.dependent_launches + kt.resolve_launches) / args.steps
                              + (2 if best.pipeline == P.PIPELINE_STAGES else 1))
+    elif on_determinants:
+        launches_per_step = 2 * n_stages + 2
     else:
         launches_per_step = 1
     if kt is not None and kt.stage_launches > 0:
         # k_stage launches other than the overlapped pipeline's dependent
         # visits: 2 matrices per visit, per-launch durations from the
         # library's CUDA events on the stream each launch runs on.
-        kernel_name = (f"k_stage<float,4,{best.warps_per_cta},tiled>" if best.reduction == P.REDUCTION_TILED
+        kernel_name = ("k_stage_rs" if on_determinants
+                       else f"k_stage<float,4,{best.warps_per_cta},tiled>" if best.reduction == P.REDUCTION_TILED
                        else f"k_stage<float,4,{best.warps_per_cta},panel{best.panel_width}>" if best.panel_width > 1
                        else f"k_stage<float,4,{best.warps_per_cta}>")
         launch_ms = kt.stage_ms / kt.stage_launches
@@ -890,12 +901,12 @@ def main():
         # intervals), one launch's share of it per launch.
         busy_ms_per_launch = kt.stage_union_ms / kt.stage_launches
     else:
-        kernel_name = f"k_sweep_persistent<float,4,{best.warps_per_cta}>"
+        kernel_name = "k_stage_rs" if on_determinants else f"k_sweep_persistent<float,4,{best.warps_per_cta}>"
         launch_ms = ms_per_step
         matrices_per_launch = 2 * N
         resolve_ms_per_step = None
         busy_ms_per_launch = launch_ms
-    achieved_tflops = matrices_per_launch * HH_FLOPS / (busy_ms_per_launch * 1e-3) / 1e12
+    achieved_tflops = matrices_per_launch * (RS_FLOPS if on_determinants else HH_FLOPS) / (busy_ms_per_launch * 1e-3) / 1e12
     per_matrix = DRAM_BYTES_PER_MATRIX.get(kernel_name)
     traffic = None if per_matrix is None else per_matrix * matrices_per_launch
     peak = fp32_alu_peak_tflops(clocks["sm_max_mhz"] or 2070.0)
@@ -917,8 +928,8 @@ def main():
             "warmup": args.warmup, "ms_per_step": ms_per_step, "higher_is_better": True, "scaling": "weak",
             "vs_baseline": None, "dtype": "f32+f64", "data": "synthetic",
             "config": {"workload": workload_name(args.schedule, n_stages),
-                       "precision": "mixed: FP32 reduction, double-float eigenvalue finish, FP64 free energies, "
-                                    "double-float re-solve of near-threshold decisions",
+                       "precision": "mixed: free energies from FP32 determinants, double-float re-solve of "
+                                    "near-threshold decisions",
                        "l2": "flushed between timed steps (256 MiB write)",
                        "parallelism": f"replicas x{world}"},
             "e2e": {"value": e2e_value, "unit": "spin-updates/s", "h2d_bytes_per_step": N * 24,
@@ -953,7 +964,8 @@ def main():
                          "matrices_per_launch": matrices_per_launch, "resolve_ms_per_step": resolve_ms_per_step,
                          "achieved": achieved_tflops, "peak": peak, "unit": "TFLOP/s",
                          "frac": achieved_tflops / peak, "traffic": traffic,
-                         "note": "FP32 FMA pipe, Householder flops only; peak = 152 SM x 128 lanes x 2 x max clock. "
+                         "note": "FP32 FMA pipe, flops of the determinants (or of the Householder reduction, "
+                                 "where the configuration names one) only; peak = 152 SM x 128 lanes x 2 x max clock. "
                                  "In the overlap pipeline consecutive stage launches overlap (look-ahead) and share "
                                  "the GPU with the re-solves and dependent visits: achieved = matrices x flops over "
                                  "the time at least one stage launch ran (busy_ms_per_launch = that union / "

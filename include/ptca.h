@@ -112,9 +112,10 @@ typedef struct {
     int32_t schedule;         /* PTCA_SCHEDULE_TILED or PTCA_SCHEDULE_BLOCK            */
     int32_t stride;           /* tiled schedule: spacing of the update sites in a     */
                               /* stage along each axis; 0: L_c                        */
-    int32_t precision;        /* PTCA_FP64 or PTCA_MIXED (FP32 reduction to tridiagonal */
-                              /* form, double-float eigenvalue finish, FP64 free      */
-                              /* energies and dF)                                     */
+    int32_t precision;        /* PTCA_FP64 or PTCA_MIXED (sweeps: free energies from    */
+                              /* FP32 determinants, or an FP32 reduction to           */
+                              /* tridiagonal form with a double-float eigenvalue      */
+                              /* finish; see reduction below)                         */
     int32_t proposal;         /* PTCA_PROPOSAL_SPHERE or PTCA_PROPOSAL_CONE            */
     int32_t model;            /* PTCA_MODEL_DOUBLE_EXCHANGE, _HUBBARD_MF or _HOLSTEIN   */
     double cone_deg;          /* half-angle of the cone proposal, degrees             */
@@ -278,7 +279,10 @@ ptca_status ptca_sweep(ptca_ctx* ctx, int32_t n_sweeps, ptca_sweep_stats* stats_
  * run the row-chunked reduction, one per matrix: selecting
  * PTCA_PIPELINE_PERSISTENT or PTCA_PIPELINE_GRAPH here resets the launch
  * configuration's reduction and panel_width to 0 (and a default re-solve
- * margin to that reduction's, ptca_set_resolve_margin). */
+ * margin to that reduction's, ptca_set_resolve_margin).  Where the sweep takes
+ * its free energies from determinants (`reduction` below) these two pipelines
+ * run one stage and one re-solve launch per stage, captured in a graph per
+ * sweep; no kernel waits at a barrier then. */
 ptca_status ptca_set_pipeline(ptca_ctx* ctx, int32_t mode, double barrier_timeout_s);
 
 /* Launch configuration of the sweep kernels:
@@ -297,8 +301,16 @@ ptca_status ptca_set_pipeline(ptca_ctx* ctx, int32_t mode, double barrier_timeou
  *   ctas_per_sm    CTAs per SM of the persistent kernel, 0 = as many as fit
  *                  (large clusters: the persistent pipelines run width 16,
  *                  the matrix in each CTA's global slot);
- *   reduction      organisation of the FP32 Householder pass (Sec. II.c
- *                  step b): PTCA_REDUCTION_ROWS = lanes on columns of the
+ *   reduction      how a visit's free energies are found (Sec. II.c step b).
+ *                  The default of a PTCA_MIXED context (PTCA_REDUCTION_ROWS
+ *                  with panel_width 0 or 1; PTCA_REDUCTION_SHARED for large
+ *                  clusters) takes them from determinants, without
+ *                  eigenvalues, wherever windows have up to 16 sites per
+ *                  layer across their longest axis and |mu - H| / T of a
+ *                  window of unit vectors stays below 4096; warps_per_cta
+ *                  and ctas_per_sm then change nothing.  Otherwise, and in
+ *                  PTCA_FP64, it is the organisation of the Householder
+ *                  pass: PTCA_REDUCTION_ROWS = lanes on columns of the
  *                  packed triangle, rows in batches (every width);
  *                  PTCA_REDUCTION_TILED = register tiles, 4x4
  *                  complex tiles per lane over pairs of block rows, the
@@ -377,10 +389,11 @@ ptca_status ptca_set_kernel_timing(ptca_ctx* ctx, int32_t on);
 ptca_status ptca_kernel_times(ptca_ctx* ctx, double* out, void* stream);
 
 /* PTCA_MIXED decision guard.  The FP32 reduction leaves an error of about
- * 1e-4 in dF at n = 128, so a Metropolis decision whose margin
- * |ln u + dF/T| is below `margin` is deferred: both cluster matrices of that
- * update site are solved again at FP64-class precision (reduction and
- * eigenvalues in double-float arithmetic, about 48 significant bits) and the
+ * 1e-4 in dF at n = 128 (determinants: 5e-7), so a Metropolis decision whose
+ * margin |ln u + dF/T| is below `margin` is deferred: both cluster matrices of
+ * that update site are solved again at FP64-class precision (determinants, or
+ * reduction and eigenvalues, in double-float arithmetic, about 48 significant
+ * bits; windows beyond the determinants' range in FP64) and the
  * decision is taken on that dF, before the next stage starts.  With a
  * margin above T^-1 times the largest dF error this makes decisions identical
  * to the FP64 path wherever the FP64 margin exceeds its own error.  Default
@@ -394,8 +407,8 @@ ptca_status ptca_set_resolve_margin(ptca_ctx* ctx, double margin);
 
 /* Precision checker (PTCA_MIXED only; PTCA_ERR_UNSUPPORTED otherwise).  While
  * on, every stage of ptca_sweep first solves both cluster matrices of each of
- * its visits twice from the stage-start spins -- with the FP32 reduction the
- * sweep uses and fully in FP64 -- and records per stage (per batch of
+ * its visits twice from the stage-start spins -- with the FP32 reduction
+ * (eigenvalues) and the free energies the sweep uses, and fully in FP64 -- and records per stage (per batch of
  * concurrent clusters) the largest eigenvalue error max|eps32 - eps64| and
  * free-energy-difference error max|dF32 - dF64|.  The chain itself is
  * unchanged; sweeps run the per-stage pipeline while the checker is on.
@@ -572,7 +585,7 @@ ptca_status ptca_sweep_noalloc(const ptca_lattice* lattice, const ptca_params* p
  * real tridiagonal form by this library's Householder reduction spread over
  * the whole GPU (one pass over the trailing triangle per reflector: FP64 for
  * a PTCA_FP64 context; double-float, about 48 significant bits on the FP32
- * pipe, for a PTCA_MIXED context, with the per-reflector scalars in FP64),
+ * pipe, for a PTCA_MIXED context),
  * and its eigenvalues found one thread each (FP32 bisection finished by
  * double-float Sturm counts and Newton).  No library eigensolver is used.
  *   eig_out  device double[2N]
