@@ -591,7 +591,7 @@ ptca_status ptca_cluster_eigvals(ptca_ctx* ctx, const void* H, const int64_t* of
                                              ctx->gL_stride, ctx->large_grid, st));
         return PTCA_OK;
     }
-    PTCA_CUDA(ptca::launch_eigvals(ctx->prec, ctx->nA, H, offsets, n, m, eig_out, eig_offsets, st));
+    PTCA_CUDA(ptca::launch_eigvals(ctx->prec, ctx->sms, ctx->nA, H, offsets, n, m, eig_out, eig_offsets, st));
     return PTCA_OK;
 }
 

@@ -280,13 +280,13 @@ __global__ void __launch_bounds__(CTA) k_build(Model m, const double* __restrict
 }
 
 // All eigenvalues of m packed matrices from global memory.
-template <typename T, int NT>
-__global__ void __launch_bounds__(CTA, MinBlocks<T, NT>::value) k_eigvals(const cplx_t<T>* __restrict__ H, const int64_t* __restrict__ offsets,
+template <typename T, int NT, int NWP = NW>
+__global__ void __launch_bounds__(32 * NWP, MinBlocks<T, NT, NWP>::value) k_eigvals(const cplx_t<T>* __restrict__ H, const int64_t* __restrict__ offsets,
                                                  const int32_t* __restrict__ nin, int count, int nA,
                                                  double* __restrict__ eig, const int64_t* __restrict__ eoff) {
     extern __shared__ __align__(16) unsigned char smem[];
-    const SmemLayout L = smem_layout(nA, 32 * NT, sizeof(cplx_t<T>));
-    Carve<T> c = carve<T>(smem, L);
+    const SmemLayout L = smem_layout(nA, 32 * NT, sizeof(cplx_t<T>), NWP);
+    Carve<T> c = carve<T>(smem, L, NWP);
     const int b = blockIdx.x;
     if (b >= count) return;
     const int n = nin[b];
@@ -299,10 +299,10 @@ __global__ void __launch_bounds__(CTA, MinBlocks<T, NT>::value) k_eigvals(const 
     const int P = tri(n);
     for (int i = threadIdx.x; i < P; i += blockDim.x) c.A[i] = src[i];
     __syncthreads();
-    householder_tridiag<T, NT, NW>(n, c.A, c.hh, c.d, c.e2);
+    householder_tridiag<T, NT, NWP>(n, c.A, c.hh, c.d, c.e2);
     double s1, s2;
     int K;
-    tridiag_eig_F<T>(n, c, 0.0, 1.0, true, out, s1, s2, K);
+    tridiag_eig_F<T, NWP>(n, c, 0.0, 1.0, true, out, s1, s2, K);
 }
 
 struct StageArgs;

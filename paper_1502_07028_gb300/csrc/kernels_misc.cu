@@ -31,6 +31,10 @@ size_t cluster_smem_bytes_f32w4(int nA);
 int cluster_max_order_f32w4();
 cudaError_t configure_f32w4(size_t);
 cudaError_t launch_stage_f32w4(const StageArgs&, cudaStream_t);
+cudaError_t launch_eigvals_f32w4(int, const void*, const int64_t*, const int32_t*, int, double*, const int64_t*,
+                                 cudaStream_t);
+cudaError_t launch_eigvals_f32w1(int, const void*, const int64_t*, const int32_t*, int, double*, const int64_t*,
+                                 cudaStream_t);
 cudaError_t launch_persistent_f32w4(const PersistArgs&, int, cudaStream_t);
 int persistent_blocks_per_sm_f32w4(int);
 // one-warp FP32 sweep kernels (kernels_f32w1.cu)
@@ -72,8 +76,23 @@ cudaError_t launch_build(int prec, const Model& m, const double* S, const int32_
     return prec ? launch_build_f32(m, S, sites, count, new_spins, H, stride, offsets, nout, st)
                 : launch_build_f64(m, S, sites, count, new_spins, H, stride, offsets, nout, st);
 }
-cudaError_t launch_eigvals(int prec, int nA, const void* H, const int64_t* offsets, const int32_t* n, int count,
+cudaError_t launch_eigvals(int prec, int sms, int nA, const void* H, const int64_t* offsets, const int32_t* n, int count,
                            double* eig, const int64_t* eoff, cudaStream_t st) {
+    // FP32: 8-warp CTAs have the shortest matrices (128: 0.36 against 0.44 ms with
+    // four warps) but two to an SM; four-warp CTAs hold three (four up to order
+    // 32) and win where that saves a wave: order 128, 330 matrices 0.57 against
+    // 0.77 ms, 1500 2.03 against 2.24; 500 (two waves either way) 0.94 against
+    // 0.91.  Up to order 32 one warp per matrix leaves no second wave: order 32,
+    // 700 matrices 0.116 against 0.135 (four warps) and 0.198 ms, 1500 0.137, 0.205
+    // and 0.333.
+    if (prec && count > 2 * sms) {
+        if (nA <= cluster_max_order_f32w1())
+            return count > 4 * sms ? launch_eigvals_f32w1(nA, H, offsets, n, count, eig, eoff, st)
+                                   : launch_eigvals_f32w4(nA, H, offsets, n, count, eig, eoff, st);
+        const int waves8 = (count + 2 * sms - 1) / (2 * sms), waves4 = (count + 3 * sms - 1) / (3 * sms);
+        if (nA <= cluster_max_order_f32w4() && waves4 < waves8)
+            return launch_eigvals_f32w4(nA, H, offsets, n, count, eig, eoff, st);
+    }
     return prec ? launch_eigvals_f32(nA, H, offsets, n, count, eig, eoff, st)
                 : launch_eigvals_f64(nA, H, offsets, n, count, eig, eoff, st);
 }

@@ -52,7 +52,7 @@ cudaError_t launch_scatter_sites(const int32_t* sites, int count, const double* 
 cudaError_t launch_build(int prec, const Model& m, const double* S, const int32_t* sites, int count,
                          const double* new_spins, void* H, int64_t stride, int64_t* offsets, int32_t* nout,
                          cudaStream_t st);
-cudaError_t launch_eigvals(int prec, int nA, const void* H, const int64_t* offsets, const int32_t* n, int count,
+cudaError_t launch_eigvals(int prec, int sms, int nA, const void* H, const int64_t* offsets, const int32_t* n, int count,
                            double* eig, const int64_t* eoff, cudaStream_t st);
 cudaError_t launch_free_energy(const double* eig, const int64_t* eoff, const int32_t* n, int count, double mu,
                                double T, double* F, cudaStream_t st);
