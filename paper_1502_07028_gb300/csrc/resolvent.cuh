@@ -52,24 +52,15 @@ __device__ __forceinline__ float2 shfl_c(float2 v, int src) {
     v.y = __shfl_sync(FULL_MASK, v.y, src);
     return v;
 }
-__device__ __forceinline__ dfl2 shfl_c(dfl2 v, int src) {
-    v.x.hi = __shfl_sync(FULL_MASK, v.x.hi, src);
-    v.x.lo = __shfl_sync(FULL_MASK, v.x.lo, src);
-    v.y.hi = __shfl_sync(FULL_MASK, v.y.hi, src);
-    v.y.lo = __shfl_sync(FULL_MASK, v.y.lo, src);
-    return v;
-}
 // Two consecutive elements of a matrix row (the first at an even index).
 __device__ __forceinline__ void ld2(const float2* p, float2& a, float2& b) {
     const float4 v = *reinterpret_cast<const float4*>(p);
     a = make_float2(v.x, v.y);
     b = make_float2(v.z, v.w);
 }
-__device__ __forceinline__ void ld2(const dfl2* p, dfl2& a, dfl2& b) { a = p[0]; b = p[1]; }
 __device__ __forceinline__ void st2(float2* p, float2 a, float2 b) {
     *reinterpret_cast<float4*>(p) = make_float4(a.x, a.y, b.x, b.y);
 }
-__device__ __forceinline__ void st2(dfl2* p, dfl2 a, dfl2 b) { p[0] = a; p[1] = b; }
 
 // Scalar helpers of the two arithmetics.
 __device__ __forceinline__ float rs_rcp(float x) { return __fdividef(1.f, x); }
