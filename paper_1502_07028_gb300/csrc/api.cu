@@ -386,6 +386,7 @@ ptca_status ptca_init(const ptca_lattice* lattice, const ptca_params* params, pt
     ptca_ctx* c = new ptca_ctx();
     c->p = p;
     c->device = dev;
+    c->smem_optin = (size_t)optin;
     c->prec = p.precision == PTCA_MIXED ? 1 : 0;
     c->N = p.N();
     c->h_start = st;
@@ -657,7 +658,7 @@ static bool few_visits(const ptca_ctx* ctx) { return ctx->max_stage <= ptca::kFe
 // A stage launch and a re-solve launch in the context's configuration
 // (shared-memory kernels, or the large-cluster kernels).
 static cudaError_t launch_stage_ctx(const ptca_ctx* ctx, const StageArgs& a, cudaStream_t st) {
-    if (on_determinants(ctx)) return ptca::launch_stage_resolvent(a, few_visits(ctx), ctx->sms, st);
+    if (on_determinants(ctx)) return ptca::launch_stage_resolvent(a, few_visits(ctx), {ctx->sms, ctx->smem_optin}, st);
     if (ctx->large && ctx->reduction == 2) return ptca::launch_stage_large_shared(a, ctx->large_grid, st);
     if (ctx->large && ctx->prec == 1 && ctx->nw == 8 && ctx->cl_size > 0)
         return ptca::launch_stage_cluster(ctx->cl_size, a, ctx->cl_grid, st);
@@ -700,7 +701,7 @@ static cudaError_t check_stage(ptca_ctx* ctx, const StageArgs& a, int s, cudaStr
             if (e == cudaSuccess) e = ptca::launch_check(0, a, c0, cnt, e64, ld, F64, ctx->resolve_grid, st);
         }
         // the free energies that the sweep decides on
-        if (e == cudaSuccess && on_determinants(ctx)) e = ptca::launch_check_resolvent(a, few_visits(ctx), c0, cnt, F32, ctx->sms, st);
+        if (e == cudaSuccess && on_determinants(ctx)) e = ptca::launch_check_resolvent(a, few_visits(ctx), c0, cnt, F32, {ctx->sms, ctx->smem_optin}, st);
         if (e == cudaSuccess)
             e = ptca::launch_check_compare(a.m, a.sites + c0, cnt, e32, e64, ld, F32, F64, ctx->d_chk_out + ptca::kCheckCols * s, st);
     }

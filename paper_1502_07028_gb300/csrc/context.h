@@ -88,6 +88,7 @@ struct ptca_ctx {
     int panel = 0;           // > 1: the blocked FP32 reduction in panels of this width (8-warp stage kernels)
     int ctas_per_sm = 0;     // persistent CTAs per SM (0: as many as fit)
     int sms = 0;
+    size_t smem_optin = 0;                // shared memory that a CTA may opt into
     unsigned long long timeout_ns = 30ull * 1000000000ull;
     int grid = 0;
     cudaGraphExec_t graph = nullptr;

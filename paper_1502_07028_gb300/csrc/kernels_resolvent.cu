@@ -1,8 +1,5 @@
 // kernels_resolvent.cu -- stage kernel of PTCA_MIXED sweeps whose free energies
 // come from determinants (resolvent.cuh), nodes packed into warps.
-#include <algorithm>
-#include <type_traits>
-
 #include "launch.h"
 #include "resolvent_plan.h"
 
@@ -49,19 +46,6 @@ cudaError_t launch_proposals(const StageArgs& a, const double* S, int N, double4
     return cudaGetLastError();
 }
 
-// f(tile, split by parity) with the tile of the problem's windows.
-template <typename F> static auto with_tile(const Model& m, F f) {
-    const int np = pair_sites(m), ns = layer_sites(m);
-    if (np == 1) return f(RsT1{}, std::true_type{});
-    if (np > 0 && np <= 4) return f(RsT4{}, std::true_type{});
-    if (np > 4) return f(RsT16{}, std::true_type{});
-    if (ns <= 1) return f(RsT1{}, std::false_type{});
-    if (ns <= 4) return f(RsT4{}, std::false_type{});
-    if (ns <= 8) return f(RsT8{}, std::false_type{});
-    if (ns <= 12) return f(RsT12{}, std::false_type{});
-    return f(RsT16{}, std::false_type{});
-}
-
 cudaError_t configure_resolvent_kernels(size_t smem_limit) {
     cudaError_t e = configure_resolvent_groups(smem_limit);
     auto tile = [&](auto t, auto pairs) {
@@ -85,45 +69,26 @@ bool resolvent_supported(const Model& m) {
     return layer_sites(m) <= 16 && unit_bound(m) <= 0.5 * kFermiMaxX;
 }
 
-static cudaError_t launch(RsMode mode, const StageArgs& a, int c0, int sms, cudaStream_t st) {
+static cudaError_t launch(RsMode mode, const StageArgs& a, int c0, const RsDevice& dev, cudaStream_t st) {
     static const FermiNodes tab[kFermiClasses] = {PTCA_FERMI_NODES};
     const int M = class_nodes(tab, unit_bound(a.m)), ms = window_sites(a.m);
     const bool uniform = a.m.lattice_periodic;
     return with_tile(a.m, [&](auto tile, auto pairs) {
         using Tl = decltype(tile);
         constexpr bool kPairs = decltype(pairs)::value;
-        // Visits per CTA: enough that its warps share their nodes evenly (a
-        // warp takes NPW nodes at a time).  Small windows: eight warps, 24 or 16
-        // visits; fewer leave turns empty or repeat the CTA's start too often.
-        // Up to 8 sites per layer: two (1099 us per 2500 visits of 8x8 clusters
-        // against 1219 with four).  One node per warp and one CTA per SM: the
-        // count with the fewest idle warps (3.8 against 5.4 ms for 8000 visits of
-        // 4x4x4 clusters, 11 nodes on 8 warps).
-        int nw = std::min((M + Tl::NPW - 1) / Tl::NPW, Tl::MAXT / 32), vb = 1;
-        if (Tl::NS <= 4) {
-            nw = Tl::MAXT / 32;
-            vb = Tl::NS == 1 ? 24 : 16;
-        } else if (Tl::NS <= 8) {
-            vb = 2;
-        } else if (Tl::NPW == 1 && uniform) {
-            double best = 0.0;
-            for (int v = 1; v <= 5 && (v == 1 || a.count >= 4 * v * sms); ++v) {
-                const double share = (double)v * M / (((v * M + nw - 1) / nw) * nw);
-                if (share > best + 0.01) { best = share; vb = v; }
-            }
-        }
-        return launch_chained(k_stage_rs<Tl, kPairs>, (a.count + vb - 1) / vb, 32 * nw,
-                              rs_layout<Tl>(vb, ms, nw, uniform, kPairs).total, st, a, vb, ms, uniform, mode, c0);
+        const RsStagePlan p = rs_stage_plan<Tl, kPairs>(M, ms, uniform, a.count, dev.sms, dev.smem - kRsStatic);
+        return launch_chained(k_stage_rs<Tl, kPairs>, (a.count + p.vb - 1) / p.vb, 32 * p.nw, p.bytes, st, a, p.vb, ms,
+                              uniform, mode, c0);
     });
 }
 
-cudaError_t launch_stage_resolvent(const StageArgs& a, bool few, int sms, cudaStream_t st) {
+cudaError_t launch_stage_resolvent(const StageArgs& a, bool few, const RsDevice& dev, cudaStream_t st) {
     if (a.count <= 0) return cudaSuccess;
-    return few ? launch_groups(RS_STAGE, a, 0, sms, st) : launch(RS_STAGE, a, 0, sms, st);
+    return few ? launch_groups(RS_STAGE, a, 0, dev.sms, st) : launch(RS_STAGE, a, 0, dev, st);
 }
 
-cudaError_t launch_check_resolvent(const StageArgs& a, bool few, int c0, int count, double* F, int sms,
-                                   cudaStream_t st) {
+cudaError_t launch_check_resolvent(const StageArgs& a, bool few, int c0, int count, double* F,
+                                   const RsDevice& dev, cudaStream_t st) {
     if (count <= 0) return cudaSuccess;
     StageArgs b = a;
     b.Fbuf = F - 2 * (int64_t)c0;
@@ -131,7 +96,7 @@ cudaError_t launch_check_resolvent(const StageArgs& a, bool few, int c0, int cou
     b.perm = nullptr;
     b.count_dev = nullptr;
     b.prev_count = b.prev2_count = 0;
-    return few ? launch_groups(RS_CHECK, b, c0, sms, st) : launch(RS_CHECK, b, c0, sms, st);
+    return few ? launch_groups(RS_CHECK, b, c0, dev.sms, st) : launch(RS_CHECK, b, c0, dev, st);
 }
 
 }  // namespace ptca

@@ -1,9 +1,6 @@
 // kernels_resolvent_groups.cu -- determinant kernels that spread a visit over
 // several CTAs (resolvent.cuh): stages of few visits in FP32, and the
 // double-float re-solve.
-#include <algorithm>
-#include <type_traits>
-
 #include "launch.h"
 #include "resolvent_plan.h"
 
@@ -63,25 +60,6 @@ __global__ void __launch_bounds__(Tl::MAXT, Tl::MINB) k_stage_rs_few(const __gri
                                      max_sites, max_layer, smem);
 }
 
-template <typename F> static auto with_group(const Model& m, F f) {
-    const int np = pair_sites(m), ns = layer_sites(m);
-    if (np > 0 && np <= 4) return f(RsG8{}, std::true_type{});
-    if (np > 4) return f(RsG32{}, std::true_type{});
-    if (ns <= 4) return f(RsG8{}, std::false_type{});
-    if (ns <= 8) return f(RsG16{}, std::false_type{});
-    if (ns <= 12) return f(RsG24{}, std::false_type{});
-    return f(RsG32{}, std::false_type{});
-}
-
-template <typename F> static auto with_latency_tile(const Model& m, F f) {
-    const int np = pair_sites(m), ns = layer_sites(m);
-    if (np > 0 && np <= 4) return f(RsL4{}, std::true_type{});
-    if (np > 4) return f(RsT16{}, std::true_type{});
-    if (ns <= 4) return f(RsL4{}, std::false_type{});
-    if (ns <= 8) return f(RsL8{}, std::false_type{});
-    return f(RsT16{}, std::false_type{});
-}
-
 cudaError_t configure_resolvent_groups(size_t smem_limit) {
     cudaError_t e = cudaSuccess;
     auto group = [&](auto g, auto pairs) {
@@ -118,13 +96,9 @@ cudaError_t launch_groups(RsMode mode, const StageArgs& a, int c0, int sms, cuda
     return with_latency_tile(a.m, [&](auto tile, auto pairs) {
         using Tl = decltype(tile);
         constexpr bool kPairs = decltype(pairs)::value;
-        using E = RsWarps<Tl, kPairs>;
-        // a visit's warps over as many CTAs as give four per SM
-        const int warps = (M + Tl::NPW - 1) / Tl::NPW;
-        const int parts = std::max(1, std::min(warps, 4 * sms / a.count));
-        const int threads = std::min(32 * ((warps + parts - 1) / parts) + 32, Tl::MAXT);
-        return launch_chained(k_stage_rs_few<Tl, kPairs>, a.count * parts, threads, rs_part_layout<E>(ms, ml, threads).total, st,
-                              a, ms, ml, scratch, parts, mode, c0);
+        const RsFewPlan p = rs_few_plan<Tl, kPairs>(M, ms, ml, a.count, sms);
+        return launch_chained(k_stage_rs_few<Tl, kPairs>, a.count * p.parts, p.threads, p.bytes, st, a, ms, ml, scratch,
+                              p.parts, mode, c0);
     });
 }
 
@@ -133,8 +107,7 @@ cudaError_t launch_resolve_resolvent(const StageArgs& a, int sms, cudaStream_t s
     const int M = class_nodes(tab, unit_bound(a.m)), ms = window_sites(a.m), ml = layer_sites(a.m);
     return with_group(a.m, [&](auto group, auto pairs) {
         using Gp = decltype(group);
-        const auto lay = rs_part_layout<RsGroups<Gp, decltype(pairs)::value>>(ms, ml, Gp::TPN * Gp::DFG + 32);
-        const size_t smem = std::max(lay.total, lay.site + rs_exact_bytes(2 * ms));
+        const size_t smem = rs_resolve_bytes<Gp, decltype(pairs)::value>(ms, ml);
         const int grid = (Gp::TPN == 32 ? 2 : 1) * sms;   // one warp per node: two CTAs fit on an SM
         return launch_chained(k_resolve_rs<Gp, decltype(pairs)::value>, grid, Gp::TPN * Gp::DFG + 32, smem, st, a, ms, ml,
                               static_cast<RsOut<dfl>*>(a.rs_scratch), M);

@@ -148,14 +148,15 @@ cudaError_t launch_observables(const double* S, int Lx, int Ly, const double* re
 // the problem's windows and temperature fit them, and a stage launch.  few:
 // stages too small to fill the GPU (the same for every launch of a context, since
 // the two forms round differently).
+struct RsDevice { int sms; size_t smem; };  // SMs, opt-in shared memory of a CTA
 bool resolvent_supported(const Model& m);
 cudaError_t configure_resolvent_kernels(size_t smem_limit);
 cudaError_t configure_resolvent_groups(size_t smem_limit);
-cudaError_t launch_stage_resolvent(const StageArgs& a, bool few, int sms, cudaStream_t st);
+cudaError_t launch_stage_resolvent(const StageArgs& a, bool few, const RsDevice& dev, cudaStream_t st);
 // Their free energies of visits c0 .. c0 + count - 1 for the checker (F[2k],
 // F[2k + 1] of visit c0 + k), and the double-float re-solve.
-cudaError_t launch_check_resolvent(const StageArgs& a, bool few, int c0, int count, double* F, int sms,
-                                   cudaStream_t st);
+cudaError_t launch_check_resolvent(const StageArgs& a, bool few, int c0, int count, double* F,
+                                   const RsDevice& dev, cudaStream_t st);
 cudaError_t launch_resolve_resolvent(const StageArgs& a, int sms, cudaStream_t st);
 cudaError_t launch_proposals(const StageArgs& a, const double* S, int N, double4* out, cudaStream_t st);
 enum RsMode : int;

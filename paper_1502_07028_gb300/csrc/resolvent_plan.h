@@ -2,7 +2,9 @@
 // which problems they serve and how a window is laid out.
 #pragma once
 
+#include <algorithm>
 #include <cmath>
+#include <type_traits>
 
 #include "resolvent.cuh"
 
@@ -36,6 +38,91 @@ inline int class_nodes(const FermiNodes* tab, double X) {
     while (c + 1 < kFermiClasses && X > tab[c].X) ++c;
     return tab[c].M;
 }
+
+// f(tile, split by parity) with the tile of the problem's windows.
+template <typename F> auto with_tile(const Model& m, F f) {
+    const int np = pair_sites(m), ns = layer_sites(m);
+    if (np == 1) return f(RsT1{}, std::true_type{});
+    if (np > 0 && np <= 4) return f(RsT4{}, std::true_type{});
+    if (np > 4) return f(RsT16{}, std::true_type{});
+    if (ns <= 1) return f(RsT1{}, std::false_type{});
+    if (ns <= 4) return f(RsT4{}, std::false_type{});
+    if (ns <= 8) return f(RsT8{}, std::false_type{});
+    if (ns <= 12) return f(RsT12{}, std::false_type{});
+    return f(RsT16{}, std::false_type{});
+}
+
+// Shape of a k_stage_rs launch of `count` visits with M nodes each: warps per
+// CTA, visits per CTA, dynamic shared memory.
+struct RsStagePlan { int nw, vb; size_t bytes; };
+
+// Visits per CTA: enough that its warps share their nodes evenly (a warp takes
+// NPW nodes at a time).  Small windows: eight warps, 24 or 16 visits; fewer leave
+// turns empty or repeat the CTA's start too often.  Up to 8 sites per layer: two
+// (1099 us per 2500 visits of 8x8 clusters against 1219 with four).  One node per
+// warp and one CTA per SM: the count with the fewest idle warps (3.8 against
+// 5.4 ms for 8000 visits of 4x4x4 clusters, 11 nodes on 8 warps) of those that
+// `room` bytes hold: eight warps' blocks of 13 to 16 sites per layer take 204 KB,
+// each visit of a 16x16 window 5 KB more.
+template <class Tl, bool kPairs>
+RsStagePlan rs_stage_plan(int M, int max_sites, bool uniform, int count, int sms, size_t room) {
+    RsStagePlan p{std::min((M + Tl::NPW - 1) / Tl::NPW, Tl::MAXT / 32), 1, 0};
+    if (Tl::NS <= 4) {
+        p.nw = Tl::MAXT / 32;
+        p.vb = Tl::NS == 1 ? 24 : 16;
+    } else if (Tl::NS <= 8) {
+        p.vb = 2;
+    } else if (Tl::NPW == 1 && uniform) {
+        double best = 0.0;
+        for (int v = 1; v <= 5 && (v == 1 || count >= 4 * v * sms); ++v) {
+            if (v > 1 && rs_layout<Tl>(v, max_sites, p.nw, uniform, kPairs).total > room) break;
+            const double share = (double)v * M / (((v * M + p.nw - 1) / p.nw) * p.nw);
+            if (share > best + 0.01) { best = share; p.vb = v; }
+        }
+    }
+    p.bytes = rs_layout<Tl>(p.vb, max_sites, p.nw, uniform, kPairs).total;
+    return p;
+}
+
+// Stages of few visits: the tile, and CTAs per visit, threads and dynamic shared
+// memory of a k_stage_rs_few launch.
+template <typename F> auto with_latency_tile(const Model& m, F f) {
+    const int np = pair_sites(m), ns = layer_sites(m);
+    if (np > 0 && np <= 4) return f(RsL4{}, std::true_type{});
+    if (np > 4) return f(RsT16{}, std::true_type{});
+    if (ns <= 4) return f(RsL4{}, std::false_type{});
+    if (ns <= 8) return f(RsL8{}, std::false_type{});
+    return f(RsT16{}, std::false_type{});
+}
+struct RsFewPlan { int parts, threads; size_t bytes; };
+template <class Tl, bool kPairs> RsFewPlan rs_few_plan(int M, int max_sites, int max_layer, int count, int sms) {
+    // a visit's warps over as many CTAs as give four per SM
+    const int warps = (M + Tl::NPW - 1) / Tl::NPW;
+    RsFewPlan p;
+    p.parts = std::max(1, std::min(warps, 4 * sms / count));
+    p.threads = std::min(32 * ((warps + p.parts - 1) / p.parts) + 32, Tl::MAXT);
+    p.bytes = rs_part_layout<RsWarps<Tl, kPairs>>(max_sites, max_layer, p.threads).total;
+    return p;
+}
+
+// The re-solve: threads per node, and dynamic shared memory.
+template <typename F> auto with_group(const Model& m, F f) {
+    const int np = pair_sites(m), ns = layer_sites(m);
+    if (np > 0 && np <= 4) return f(RsG8{}, std::true_type{});
+    if (np > 4) return f(RsG32{}, std::true_type{});
+    if (ns <= 4) return f(RsG8{}, std::false_type{});
+    if (ns <= 8) return f(RsG16{}, std::false_type{});
+    if (ns <= 12) return f(RsG24{}, std::false_type{});
+    return f(RsG32{}, std::false_type{});
+}
+template <class Gp, bool kPairs> size_t rs_resolve_bytes(int max_sites, int max_layer) {
+    const auto lay = rs_part_layout<RsGroups<Gp, kPairs>>(max_sites, max_layer, Gp::TPN * Gp::DFG + 32);
+    return std::max(lay.total, lay.site + rs_exact_bytes(2 * max_sites));
+}
+
+// What the device's opt-in limit leaves for dynamic shared memory beside the
+// kernels' own few words.
+constexpr size_t kRsStatic = 256;
 
 // Allow a kernel all the dynamic shared memory of the device.
 template <class K> cudaError_t allow_smem(K kernel, size_t smem_limit) {
