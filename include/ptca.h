@@ -397,10 +397,13 @@ ptca_status ptca_kernel_times(ptca_ctx* ctx, double* out, void* stream);
  * decision is taken on that dF, before the next stage starts.  With a
  * margin above T^-1 times the largest dF error this makes decisions identical
  * to the FP64 path wherever the FP64 margin exceeds its own error.  Default
- * in PTCA_MIXED: 1e-2; 1e-4 for large clusters on the shared reduction
- * (launch configuration reduction = PTCA_REDUCTION_SHARED, their default),
- * whose dF error is about 5e-7.  The default follows the launch
- * configuration until the caller sets a margin here; 0 disables it.  The
+ * in PTCA_MIXED: two or more times T^-1 times the largest dF error measured,
+ * which is 4e-5 (|J| + |lambda| + 2 d |t|) / T for the per-matrix FP32
+ * reductions and 4e-7 (...) / T for determinants and the large clusters'
+ * shared reduction; but at least 1e-2, and for large clusters in
+ * PTCA_REDUCTION_SHARED (their default) at least 1e-4.  The default follows
+ * T, mu and the launch configuration until the caller sets a margin here; 0
+ * disables it.  The
  * count of re-solved updates is ptca_sweep_stats.resolved.  Rejected
  * (PTCA_ERR_INVALID) for PTCA_FP64. */
 ptca_status ptca_set_resolve_margin(ptca_ctx* ctx, double margin);
@@ -540,8 +543,9 @@ ptca_status ptca_surrogate_enable(ptca_ctx* ctx, int32_t on);
 /* Sweep without device allocation                                           */
 /* ----------------------------------------------------------------------- */
 
-/* One sweep as ptca_sweep runs it in the per-stage pipeline (same stage and
- * re-solve kernels, same decisions and spins), for callers that cannot
+/* One sweep as ptca_sweep runs it in the per-stage pipeline (same decisions and
+ * spins; free energies from eigenvalues, one 8-warp CTA per matrix), for callers
+ * that cannot
  * allocate device memory: hosts whose own pool owns the device memory or
  * that forbid loaded libraries to allocate, and loops that cannot afford
  * cudaMalloc/cudaFree (cudaFree synchronises the device).  The paper has no
@@ -555,9 +559,9 @@ ptca_status ptca_surrogate_enable(ptca_ctx* ctx, int32_t on);
  *                sweep, 0 or the ptca_status of a device-side failure
  *                (PTCA_ERR_NUMERIC: a free-energy difference was not finite)
  * The schedule is built and checked on the host, as ptca_init does, and
- * copied into the library's array.  In PTCA_MIXED the decisions within 1e-2
- * of the Metropolis threshold are re-solved at FP64-class precision, as
- * ptca_sweep's default margin does; that re-solve keeps its matrix in shared
+ * copied into the library's array.  In PTCA_MIXED the decisions near the
+ * Metropolis threshold are re-solved at FP64-class precision, within
+ * ptca_sweep's default margin for that reduction; that re-solve keeps its matrix in shared
  * memory, so PTCA_MIXED is limited to the orders where that fits (128 on a
  * GB300; PTCA_ERR_UNSUPPORTED above).
  * No context and no device allocation: working memory is one array of about

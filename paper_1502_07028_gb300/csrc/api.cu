@@ -355,14 +355,15 @@ ptca_status ptca_stage_split(const ptca_lattice* lattice, const ptca_params* par
     return PTCA_OK;
 }
 
-// Default re-solve margin of a PTCA_MIXED context (unless the caller set
-// one): 5 to 10 times beta times the largest FP32 dF error measured for its
-// reduction.  The per-matrix reductions leave up to about 2e-4 (n = 128 to
-// 288), hence 1e-2; the large-cluster shared reduction, whose chases run in
-// double-float, about 5e-7, hence 1e-4.
+// Re-solve margin of a PTCA_MIXED context whose caller set none, for its present
+// reduction, temperature and couplings (default_resolve_margin).
+static bool on_determinants(const ptca_ctx* ctx);
 static void default_margin(ptca_ctx* c) {
     if (c->prec != 1 || c->margin_set) return;
-    c->margin = (c->large && c->reduction == 2) ? 1e-4 : 1e-2;
+    const bool large_shared = c->large && c->reduction == 2;
+    c->margin = ptca::default_resolve_margin(to_model(c->p),
+                                             large_shared || on_determinants(c) ? ptca::kDeterminantDF : ptca::kHouseholderDF,
+                                             large_shared ? 1e-4 : 1e-2);
 }
 
 ptca_status ptca_init(const ptca_lattice* lattice, const ptca_params* params, ptca_ctx** out) {
@@ -524,6 +525,7 @@ ptca_status ptca_set_T(ptca_ctx* ctx, double T) {
     if (!(T > 0) || !std::isfinite(T)) return fail(PTCA_ERR_INVALID, "T must be finite and > 0");
     PTCA_SETTLE_SYNC(ctx);
     ctx->p.T = T;
+    default_margin(ctx);
     drop_graph(ctx);
     return PTCA_OK;
 }
@@ -533,6 +535,7 @@ ptca_status ptca_set_mu(ptca_ctx* ctx, double mu) {
     if (!std::isfinite(mu)) return fail(PTCA_ERR_INVALID, "mu must be finite");
     PTCA_SETTLE_SYNC(ctx);
     ctx->p.mu = mu;
+    default_margin(ctx);
     drop_graph(ctx);
     return PTCA_OK;
 }

@@ -238,6 +238,12 @@ __global__ void k_init_spins(Model m, double* __restrict__ S, int N) {
     S[3 * i] = s[0]; S[3 * i + 1] = s[1]; S[3 * i + 2] = s[2];
 }
 
+double default_resolve_margin(const Model& m, double rel_dF, double least) {
+    const int d = (m.Lx > 1) + (m.Ly > 1) + (m.Lz > 1);
+    const double rule = rel_dF * (std::fabs(m.JH) + std::fabs(m.lam) + 2.0 * d * std::fabs(m.t)) / m.T;
+    return rule > least ? rule : least;
+}
+
 void set_model_terms(Model& m, int model, double J_H, double U, double lam, double K, double mu, double m_step) {
     m.model = model;
     m.JH = 0.0; m.e0 = 0.0; m.lam = 0.0; m.ca = 0.0; m.cb = 0.0; m.cc = 0.0; m.m_step = 0.0; m.cls_on = 0;

@@ -44,6 +44,14 @@ cudaError_t launch_init_spins(const Model& m, double* S, int N, cudaStream_t st)
 // proposal step) for model 0 (double exchange), 1 (Hubbard mean field) or 2
 // (Holstein).
 void set_model_terms(Model& m, int model, double J_H, double U, double lam, double K, double mu, double m_step);
+// Default re-solve margin of PTCA_MIXED sweeps: beta times rel_dF couplings
+// (|J| + |lambda| + 2 d |t|, the reach of a proposal's dF), and at least `least`.
+// Largest dF errors measured at a coupling of 12: 2e-4 for the per-matrix FP32
+// reductions (kHouseholderDF: 4.8e-4), 3e-6 for FP32 determinants and 5e-7 for the
+// large-cluster shared reduction, whose chases run in double-float
+// (kDeterminantDF: 4.8e-6); their rms is ten times less.
+constexpr double kHouseholderDF = 4e-5, kDeterminantDF = 4e-7;
+double default_resolve_margin(const Model& m, double rel_dF, double least);
 cudaError_t launch_copy_sites(const double* src, double* dst, const int32_t* sites, int count, cudaStream_t st);
 // out[k] = S[sites[k]]; and S0[sites[k]] = S1[sites[k]] = in[k] (3 doubles each).
 cudaError_t launch_gather_sites(const double* S, const int32_t* sites, int count, double* out, cudaStream_t st);

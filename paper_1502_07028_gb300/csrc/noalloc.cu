@@ -38,7 +38,6 @@ namespace {
 
 constexpr int kNoAllocMaxSites = 16384;  // e.g. up to a 128 x 128 lattice
 constexpr int kNoAllocMaxDevices = 64;
-constexpr double kNoAllocMargin = 1e-2;  // re-solve band of PTCA_MIXED, as ptca_init's default
 
 // Byte layout of the scratch array (offsets are multiples of 256).
 constexpr size_t al256(size_t x) { return (x + 255) & ~size_t(255); }
@@ -133,8 +132,8 @@ extern "C" ptca_status ptca_sweep_noalloc(const ptca_lattice* lattice, const ptc
         return ptca_internal_fail(PTCA_ERR_INVALID, "ptca_sweep_noalloc: cluster matrix too large for this precision");
     e = ptca::configure_cluster_kernels((size_t)optin);
     if (e != cudaSuccess) return ptca_internal_fail(PTCA_ERR_CUDA, cudaGetErrorString(e));
-    // PTCA_MIXED re-solves the decisions within kNoAllocMargin of the
-    // threshold, as ptca_sweep does; that re-solve must keep its matrix in
+    // PTCA_MIXED re-solves the decisions near the threshold, as
+    // ptca_sweep does (default_resolve_margin); that re-solve must keep its matrix in
     // shared memory here (the global matrix slots it uses otherwise are
     // context memory).
     if (prec == 1 && !ptca::resolve_smem_fits(nA))
@@ -180,7 +179,7 @@ extern "C" ptca_status ptca_sweep_noalloc(const ptca_lattice* lattice, const ptc
     a.rec_n = reinterpret_cast<int32_t*>(base + kOffRecN);
     a.counters = counters;
     a.err = err;
-    a.margin = prec == 1 ? kNoAllocMargin : 0.0;
+    a.margin = prec == 1 ? ptca::default_resolve_margin(m, ptca::kHouseholderDF, 1e-2) : 0.0;
     a.flag_list = reinterpret_cast<int32_t*>(base + kOffFlags);
     a.flag_count = flag_count;
     for (int s = 0; s < n_stages; ++s) {
