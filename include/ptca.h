@@ -391,10 +391,11 @@ ptca_status ptca_kernel_times(ptca_ctx* ctx, double* out, void* stream);
 /* PTCA_MIXED decision guard.  The FP32 reduction leaves an error of about
  * 1e-4 in dF at n = 128 (determinants: 5e-7), so a Metropolis decision whose
  * margin |ln u + dF/T| is below `margin` is deferred: both cluster matrices of
- * that update site are solved again at FP64-class precision (determinants, or
- * reduction and eigenvalues, in double-float arithmetic, about 48 significant
- * bits; windows beyond the determinants' range in FP64) and the
- * decision is taken on that dF, before the next stage starts.  With a
+ * that update site are solved again at FP64-class precision (in double-float
+ * arithmetic, about 48 significant bits: reduction and eigenvalues to about
+ * 1e-14, or determinants, free energies then to about 1e-12 of themselves and
+ * the filling to 1e-9 per site; windows beyond the determinants' range in
+ * FP64) and the decision is taken on that dF, before the next stage starts.  With a
  * margin above T^-1 times the largest dF error this makes decisions identical
  * to the FP64 path wherever the FP64 margin exceeds its own error.  Default
  * in PTCA_MIXED: two or more times T^-1 times the largest dF error measured,

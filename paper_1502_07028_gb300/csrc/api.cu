@@ -635,6 +635,9 @@ static StageArgs base_args(ptca_ctx* ctx) {
     a.gA_stride = ctx->gA_stride;
     a.rs_scratch = ctx->d_rs;
     a.invT = 1.0 / ctx->p.T;
+    const double unit = std::fabs(a.m.t) > 1e-6 * (std::fabs(a.m.mu - a.m.e0) + std::fabs(a.m.lam) + std::fabs(a.m.JH))
+                            ? std::fabs(a.m.t) : 1.0;
+    a.unit = {(a.m.mu - a.m.e0) / unit, a.m.lam / unit, a.m.JH / unit, a.m.t / unit, unit / ctx->p.T};
     a.gL = ctx->d_gL;
     a.gL_stride = ctx->gL_stride;
     return a;

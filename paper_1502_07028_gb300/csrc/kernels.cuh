@@ -328,6 +328,10 @@ __global__ void __launch_bounds__(CTA, 1) k_check_ref(StageArgs a, int c0, int c
 // does not hold yet, copied forward from S_in (the previous stage's with two
 // rotating spin buffers, the two previous stages' with three), so S_out is
 // the full configuration after the stage.
+// Energies of the determinant kernels, in units of |t| (of 1 where t is too small):
+// mu - e0, lambda, J, t, and the unit over T.
+struct RsUnit { double mu, lam, J, t, T1; };
+
 struct StageArgs {
     Model m;
     const double* S_in;
@@ -374,6 +378,7 @@ struct StageArgs {
     void* rs_scratch;
     int32_t rs_half;
     double invT;              // 1 / T (the host's: an FP64 division takes a microsecond of latency here)
+    RsUnit unit;
     unsigned int* flag_next;  // counter that the re-solve clears for the next stage, or null
     const double4* prop;      // proposal and ln u by lattice site for this sweep, or null
     // Delayed acceptance: work list (perm) length on the device, and the

@@ -113,9 +113,11 @@ template <> struct RsSum<dfl> {
     __device__ __forceinline__ double value() const { return v; }
 };
 
-// On-site terms of a window site: mu - H = [[d + z, x - iy], [x + iy, d - z]].
+// On-site terms of a window site: mu - H = [[d + z, x - iy], [x + iy, d - z]], in
+// units of |t| (RsUnit), so that the scaled hopping is the scale s itself.
 template <typename T> struct RsSite { T d, x, y, z; };
-template <typename T> struct RsOut { double lnd, th; T P[8], s; };  // P: the last pivot block, without its i; s = 1 / (T y)
+// P: the last pivot block, without its i; s = unit / (T y), rounded; eta: its relative rounding error.
+template <typename T> struct RsOut { double lnd, th; T P[8], s; float eta; };
 
 // Window of a visit in layer order.
 struct RsVisit {
@@ -219,13 +221,14 @@ template <class Tl> struct RsNode {
         __syncwarp();
     }
 
-    // The block of layer l without its i on the diagonal, minus tt X (X in a).
-    static __device__ __forceinline__ void layer(Tile& a, const RsSite<float>* site, const float* hop, float s, float tt,
+    // The block of layer l without its i on the diagonal, minus t'^2 X (X in a); t'
+    // is applied twice, since a rounded t'^2 would be off by as much on every bond.
+    static __device__ __forceinline__ void layer(Tile& a, const RsSite<float>* site, const float* hop, float s, float tp,
                                                  int ns, int r, int c, bool chain) {
 #pragma unroll
         for (int i = 0; i < SR; ++i) {
             const int sr = r + GR * i;
-            const float f = sr < ns ? tt : 0.f;
+            const float f = sr < ns ? tp : 0.f;
 #pragma unroll
             for (int j = 0; j < SC; ++j) {
                 const int sc = csite(c, j);
@@ -241,10 +244,10 @@ template <class Tl> struct RsNode {
                 }
                 if (chain) {
                     const V x00 = a[i][j], x01 = a[i][SC + j], x10 = a[SR + i][j], x11 = a[SR + i][SC + j];
-                    uu = make_float2(uu.x - f * x00.x, -(f * x00.y));
-                    dd = make_float2(dd.x - f * x11.x, -(f * x11.y));
-                    ud = make_float2(ud.x - f * x01.x, ud.y - f * x01.y);
-                    du = make_float2(du.x - f * x10.x, du.y - f * x10.y);
+                    uu = make_float2(uu.x - f * (f * x00.x), -(f * (f * x00.y)));
+                    dd = make_float2(dd.x - f * (f * x11.x), -(f * (f * x11.y)));
+                    ud = make_float2(ud.x - f * (f * x01.x), ud.y - f * (f * x01.y));
+                    du = make_float2(du.x - f * (f * x10.x), du.y - f * (f * x10.y));
                 }
                 a[i][j] = uu;
                 a[SR + i][SC + j] = dd;
@@ -370,7 +373,7 @@ template <class Tl> struct RsNode {
     // on-site terms (without i) minus t'^2 times the pivot inverses of common
     // neighbours (inv: 4 elements per eliminated site).
     static __device__ __forceinline__ void pair_block(Tile& a, const RsPairs& pt, int row0, int nr, int col0, int nc,
-                                                      const RsSite<float>* site, const V* inv, float s, float tt, int r, int c) {
+                                                      const RsSite<float>* site, const V* inv, float s, float tp, int r, int c) {
 #pragma unroll 1
         for (int i = 0; i < SR; ++i)
 #pragma unroll 1
@@ -390,10 +393,10 @@ template <class Tl> struct RsNode {
                         du = csub(du, p);
                         dd = csub(dd, q);
                     }
-                    uu = make_float2(tt * uu.x, tt * uu.y);
-                    ud = make_float2(tt * ud.x, tt * ud.y);
-                    du = make_float2(tt * du.x, tt * du.y);
-                    dd = make_float2(tt * dd.x, tt * dd.y);
+                    uu = make_float2(tp * (tp * uu.x), tp * (tp * uu.y));
+                    ud = make_float2(tp * (tp * ud.x), tp * (tp * ud.y));
+                    du = make_float2(tp * (tp * du.x), tp * (tp * du.y));
+                    dd = make_float2(tp * (tp * dd.x), tp * (tp * dd.y));
                     if (row0 + x == col0 + y) {
                         const RsSite<float> o = site[pt.kept[row0 + x]];
                         uu.x += (o.d + o.z) * s;
@@ -446,7 +449,6 @@ template <class Tl> struct RsNode {
                                                      int lane, RsOut<float>* out) {
         const int base = lane & ~(Tl::LPN - 1), nl = lane - base;
         const int r = nl / GC, c = nl % GC;
-        const float tt = tp * tp;
         V *X = buf, *C = buf + Tl::B * RS, *inv = C + Tl::B * RS;
         RsSum<float> lnd, th;
         for (int e = nl; e < pt.ne; e += Tl::LPN) {
@@ -463,15 +465,15 @@ template <class Tl> struct RsNode {
         }
         __syncwarp();
         Tile a, S;
-        pair_block(a, pt, 0, pt.na, 0, pt.na, site, inv, s, tt, r, c);
+        pair_block(a, pt, 0, pt.na, 0, pt.na, site, inv, s, tp, r, c);
 #pragma unroll 1
         for (int o = 0;; ++o) {
             invert(a, lnd, th, o == 0 ? -1 : pt.nb - 1, o == 0 ? pt.na : pt.nb, r, c, nl, base);
             if (o) break;
             store(X, a, r, c);
-            pair_block(a, pt, 0, pt.na, pt.na, pt.nb, site, inv, s, tt, r, c);
+            pair_block(a, pt, 0, pt.na, pt.na, pt.nb, site, inv, s, tp, r, c);
             store(C, a, r, c);
-            pair_block(S, pt, pt.na, pt.nb, pt.na, pt.nb, site, inv, s, tt, r, c);
+            pair_block(S, pt, pt.na, pt.nb, pt.na, pt.nb, site, inv, s, tp, r, c);
             __syncwarp();
             mul(a, X, C, pt.na, r, c);
             put(X, a, 1.f, r, c);
@@ -485,7 +487,7 @@ template <class Tl> struct RsNode {
     }
 
     // One node of one visit: the sums over all pivots but the update site's,
-    // and that site's last pivot block.  s: 1 / (T y), tp: t / (T y).
+    // and that site's last pivot block.  s: unit / (T y), tp: t / (T y) = +-s.
     static __device__ __forceinline__ void run(const RsVisit& v, const RsSite<float>* site, const float* hop, float s, float tp,
                                                V* buf, int lane, RsOut<float>* out) {
         const int base = lane & ~(Tl::LPN - 1), nl = lane - base;
@@ -493,10 +495,9 @@ template <class Tl> struct RsNode {
         const int L = v.L, ns = v.ns;
         V *X = buf, *C = buf + Tl::B * RS, *E = C + Tl::B * RS;
         const bool ring = v.per && L >= 3;
-        const float tt = tp * tp, tau2 = (v.per && L == 2) ? 4.f * tt : tt;
         Tile a, S;
         RsSum<float> lnd, th;
-        layer(S, site + v.u * ns, hop, s, tt, ns, r, c, false);
+        layer(S, site + v.u * ns, hop, s, tp, ns, r, c, false);
 #pragma unroll 1
         for (int o = 0; o < L; ++o) {
             const bool last = o == L - 1;
@@ -511,7 +512,7 @@ template <class Tl> struct RsNode {
                 int l;
                 if (v.per) { l = v.u + 1 + o; if (l >= L) l -= L; }
                 else l = o < v.u ? o : L - 1 - (o - v.u);
-                layer(a, site + l * ns, hop, s, tt, ns, r, c, o > 0 && (v.per || o != v.u));
+                layer(a, site + l * ns, hop, s, tp, ns, r, c, o > 0 && (v.per || o != v.u));
             }
             invert(a, lnd, th, last ? v.us : -1, ns, r, c, nl, base);
             if (last) break;
@@ -549,12 +550,12 @@ template <class Tl> struct RsNode {
             if (!ring && !(o == L - 2 || (!v.per && o == v.u - 1))) continue;
             // S -= (coupling)^2 X, on real sites; the ring's first layer also
             // starts the border blocks with t' X.
-            const float cc = ring ? tt : tau2;
+            const float cc = v.per && L == 2 ? 2.f * tp : tp;
 #pragma unroll
             for (int i = 0; i < 2 * SR; ++i) {
                 const float f = (r + GR * (i % SR)) < ns ? cc : 0.f;
 #pragma unroll
-                for (int j = 0; j < 2 * SC; ++j) S[i][j] = make_float2(S[i][j].x - f * a[i][j].x, S[i][j].y - f * a[i][j].y);
+                for (int j = 0; j < 2 * SC; ++j) S[i][j] = make_float2(S[i][j].x - f * (f * a[i][j].x), S[i][j].y - f * (f * a[i][j].y));
             }
             if (ring) {
                 Tile w;
@@ -936,6 +937,7 @@ __host__ __device__ inline RsLayout rs_layout(int vb, int max_sites, int nw, boo
 static __constant__ float c_fermi_x[kFermiClasses] = {PTCA_FERMI_X};
 static __constant__ FermiNodes c_fermi[kFermiClasses] = {PTCA_FERMI_NODES};
 static __constant__ FermiNodes c_fermi_df[kFermiClasses] = {PTCA_FERMI_NODES_DF};
+static __constant__ FermiSlopes c_slope = fermi_slopes();
 
 // The nodes of an arithmetic: their approximation error is below its rounding.
 template <typename T> struct RsFermi {
@@ -971,8 +973,8 @@ __device__ __forceinline__ void rs_terms_out(const StageArgs& a, const RsFrame& 
     const int per = a.m.cluster_periodic, nsite = f.ns * f.L;
     int pairs = 0;
     for (int e : {f.L, f.e0, f.e1}) pairs += e < 2 ? 0 : nsite / e * (per ? (e == 2 ? 4 : e) : e - 1);
-    w.x1 = x1 * a.invT;
-    w.x2 = (x2 + 4.0 * a.m.t * a.m.t * (double)pairs) * a.invT * a.invT;
+    w.x1 = x1 * a.unit.T1;
+    w.x2 = (x2 + 4.0 * a.unit.t * a.unit.t * (double)pairs) * a.unit.T1 * a.unit.T1;
     w.cl = cl;
 }
 
@@ -984,21 +986,21 @@ __device__ __forceinline__ void rs_gather(const StageArgs& a, const double* S, i
     const Model& m = a.m;
     const RsFrame f = rs_frame(m, site);
     const int nsite = f.ns * f.L, per = m.cluster_periodic;
-    const double mus = m.mu - m.e0;
+    const RsUnit& u = a.unit;
     double x1 = 0.0, x2 = 0.0, cl = 0.0;
     float bound = 0.f;
     for (int k = gl; k < nsite; k += GL) {
         const double* v = S + 3 * (int64_t)f.site(m, k);
-        const double v0 = v[0], v1 = v[1], v2 = v[2], d = mus - m.lam * v0;
-        sites[k].d = T(d); sites[k].x = T(m.JH * v0); sites[k].y = T(m.JH * v1); sites[k].z = T(m.JH * v2);
+        const double v0 = v[0], v1 = v[1], v2 = v[2], d = u.mu - u.lam * v0;
+        sites[k].d = T(d); sites[k].x = T(u.J * v0); sites[k].y = T(u.J * v1); sites[k].z = T(u.J * v2);
         if constexpr (kTerms) {
             const double m2 = v0 * v0 + v1 * v1 + v2 * v2;
             x1 -= 2.0 * d;
-            x2 += 2.0 * (d * d + m.JH * m.JH * m2);
+            x2 += 2.0 * (d * d + u.J * u.J * m2);
             if (m.cls_on) cl += m.ca * m2 + m.cb * v0 + m.cc;
         }
         const float g0 = (float)v0, g1 = (float)v1, g2 = (float)v2;
-        bound = fmaxf(bound, fabsf((float)d) + fabsf((float)m.JH) * sqrtf(g0 * g0 + g1 * g1 + g2 * g2));
+        bound = fmaxf(bound, fabsf((float)d) + fabsf((float)u.J) * sqrtf(g0 * g0 + g1 * g1 + g2 * g2));
     }
 #pragma unroll
     for (int o = GL / 2; o > 0; o >>= 1) {
@@ -1012,7 +1014,7 @@ __device__ __forceinline__ void rs_gather(const StageArgs& a, const double* S, i
     if (gl == 0) {
         float deg = 0.f;
         for (int e : {f.L, f.e0, f.e1}) deg += e < 2 ? 0.f : e == 2 && !per ? 1.f : 2.f;
-        const float X = (bound + deg * fabsf((float)m.t)) * (float)a.invT * (1.f + 1e-6f);
+        const float X = (bound + deg * fabsf((float)u.t)) * (float)u.T1 * (1.f + 1e-6f);
         int cls = 0;
         while (cls < kFermiClasses && !(X <= c_fermi_x[cls])) ++cls;
         h.c = c; h.site = site; h.n = 2 * nsite; h.L = f.L; h.ns = f.ns; h.per = per;
@@ -1027,13 +1029,13 @@ __device__ __forceinline__ void rs_gather(const StageArgs& a, const double* S, i
 __device__ __forceinline__ void rs_terms(const StageArgs& a, const double* S, int site, RsTerms& w, int lane) {
     const Model& m = a.m;
     const RsFrame f = rs_frame(m, site);
-    const double mus = m.mu - m.e0;
+    const RsUnit& u = a.unit;
     double x1 = 0.0, x2 = 0.0, cl = 0.0;
     for (int k = lane; k < f.ns * f.L; k += 32) {
         const double* v = S + 3 * (int64_t)f.site(m, k);
-        const double v0 = v[0], d = mus - m.lam * v0, m2 = v0 * v0 + v[1] * v[1] + v[2] * v[2];
+        const double v0 = v[0], d = u.mu - u.lam * v0, m2 = v0 * v0 + v[1] * v[1] + v[2] * v[2];
         x1 -= 2.0 * d;
-        x2 += 2.0 * (d * d + m.JH * m.JH * m2);
+        x2 += 2.0 * (d * d + u.J * u.J * m2);
         if (m.cls_on) cl += m.ca * m2 + m.cb * v0 + m.cc;
     }
     x1 = warp_sum(x1);
@@ -1057,20 +1059,21 @@ __device__ __forceinline__ void rs_proposal(const StageArgs& a, const StageVar& 
     w.lnu = log(u0);
 }
 
-// In-layer hopping of a window between sites a and b of a layer, at [a hs + b]
+// In-layer hopping of a window between sites i and j of a layer, at [i hs + j]
 // (an axis of extent 2 of a periodic cluster has two bonds), by one warp.
-template <typename T> __device__ __forceinline__ void rs_hopping(const Model& m, int site, T* hop, int hs, int lane) {
+template <typename T> __device__ __forceinline__ void rs_hopping(const StageArgs& a, int site, T* hop, int hs, int lane) {
+    const Model& m = a.m;
     const RsFrame f = rs_frame(m, site);
     const int e0 = f.e0, e1 = f.e1, ns = f.ns, per = m.cluster_periodic;
     for (int k = lane; k < hs * hs; k += 32) {
-        const int a = k / hs, b = k % hs;
+        const int i = k / hs, j = k % hs;
         double bonds = 0.0;
-        if (a < ns && b < ns) {
-            const int d0 = abs(a % e0 - b % e0), d1 = abs(a / e0 - b / e0);
+        if (i < ns && j < ns) {
+            const int d0 = abs(i % e0 - j % e0), d1 = abs(i / e0 - j / e0);
             if (d1 == 0 && d0 > 0) bonds = (d0 == 1) + (per && d0 == e0 - 1);
             if (d0 == 0 && d1 > 0) bonds = (d1 == 1) + (per && d1 == e1 - 1);
         }
-        hop[k] = T(m.t * bonds);
+        hop[k] = T(a.unit.t * bonds);
     }
 }
 
@@ -1175,6 +1178,7 @@ template <typename T> __device__ __forceinline__ void rs_load(RsOut<T>& r, const
 #pragma unroll
     for (int k = 0; k < 8; ++k) rs_get(r.P[k], &q->P[k]);
     rs_get(r.s, &q->s);
+    r.eta = q->eta;
 }
 
 // The last pivot of a node: lq = ln|det| and t0 = phase (against i^2) of the
@@ -1233,21 +1237,39 @@ __device__ __forceinline__ void rs_final(RsMode mode, const StageArgs& a, const 
 template <typename T>
 __device__ __forceinline__ void rs_decide(RsMode mode, const StageArgs& a, const StageVar& v, const RsVisit& h, const RsTerms& w,
                                           const RsOut<T>* out, int lane) {
-    const Model& m = a.m;
+    const RsUnit& u = a.unit;
     const double* so = v.S_in + 3 * (int64_t)h.site;
     const FermiNodes& f = RsFermi<T>::tab(h.cls >= 0 ? h.cls : 0);
     double Lo = 0.0, Th = 0.0, dL = 0.0, dT = 0.0;
+    float th = 0.f, dth = 0.f, eta = 0.f;   // FP32: phase, its change, rounding of the scale
     if (h.cls >= 0 && lane < f.M) {
         RsOut<T> r;
         rs_load(r, out + lane);
-        const T dd = T(-m.lam * (w.sn[0] - so[0])) * r.s, jx = T(m.JH * (w.sn[0] - so[0])) * r.s,
-                jy = T(m.JH * (w.sn[1] - so[1])) * r.s, jz = T(m.JH * (w.sn[2] - so[2])) * r.s;
+        const T dd = T(-u.lam * (w.sn[0] - so[0])) * r.s, jx = T(u.J * (w.sn[0] - so[0])) * r.s,
+                jy = T(u.J * (w.sn[1] - so[1])) * r.s, jz = T(u.J * (w.sn[2] - so[2])) * r.s;
         decltype(rs_log1p(r.s)) lq, t0, dl, dt;
         rs_last_pivot(r, dd, jx, jy, jz, lq, t0, dl, dt);
         Lo = f.a[lane] * (r.lnd + (double)lq);
         Th = f.b[lane] * (r.th + (double)t0);
         dL = f.a[lane] * (double)dl;
         dT = f.b[lane] * (double)dt;
+        if constexpr (sizeof(T) == 4) {
+            th = (float)r.th + (float)t0;
+            dth = (float)dt;
+            eta = r.eta;
+        }
+    }
+    if constexpr (sizeof(T) == 4) {
+        const int mid = fermi_middle(lane, f.M);
+        const float* w = c_slope.of[h.cls >= 0 ? h.cls : 0].w[lane < f.M ? lane : 0];
+        float d = 0.f, dd = 0.f;
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            d += w[i] * __shfl_sync(FULL_MASK, th, mid + i - 1);
+            dd += w[i] * __shfl_sync(FULL_MASK, dth, mid + i - 1);
+        }
+        Th += (double)(eta * d);
+        dT += (double)(eta * dd);
     }
     Lo = warp_sum(Lo);
     Th = warp_sum(Th);
@@ -1345,6 +1367,12 @@ static __device__ __noinline__ void rs_exact(const StageArgs& a, const StageVar&
     __syncthreads();
 }
 
+// Relative rounding error of s as a float.
+__device__ __forceinline__ float rs_rounding(double s) {
+    const float f = (float)s;
+    return __fdividef((float)((double)f - s), f);
+}
+
 // Visits [first, first + nv) of the work list (nv <= vb <= 32), by the CTA.
 // uniform: all windows have one shape (periodic lattices), so that a warp may
 // hold nodes of several visits.  kPairs: windows split by parity (uniform).
@@ -1370,7 +1398,7 @@ __device__ __forceinline__ void rs_visits(RsMode mode, const StageArgs& a, const
     }
     if (!kPairs)
         for (int k = nw - 1 - warp; k < (uniform ? 1 : nv); k += nw)
-            rs_hopping(a.m, v.sites[list ? list[first + k] : first + k], hop + k * Tl::NS * Tl::NS, Tl::NS, lane);
+            rs_hopping(a, v.sites[list ? list[first + k] : first + k], hop + k * Tl::NS * Tl::NS, Tl::NS, lane);
     if (kPairs && warp == nw - 1) rs_pairs(a.m, v.sites[list ? list[first] : first], pt, lane);
     if (threadIdx.x == 0) *s_task = 0;
     __syncthreads();
@@ -1381,10 +1409,10 @@ __device__ __forceinline__ void rs_visits(RsMode mode, const StageArgs& a, const
         rs_proposal(a, v, site, tm[lane]);
         const double* so = v.S_in + 3 * (int64_t)site;
         const double dx = tm[lane].sn[0] - so[0];
-        tm[lane].dv[0] = (float)(-a.m.lam * dx);
-        tm[lane].dv[1] = (float)(a.m.JH * dx);
-        tm[lane].dv[2] = (float)(a.m.JH * (tm[lane].sn[1] - so[1]));
-        tm[lane].dv[3] = (float)(a.m.JH * (tm[lane].sn[2] - so[2]));
+        tm[lane].dv[0] = (float)(-a.unit.lam * dx);
+        tm[lane].dv[1] = (float)(a.unit.J * dx);
+        tm[lane].dv[2] = (float)(a.unit.J * (tm[lane].sn[1] - so[1]));
+        tm[lane].dv[3] = (float)(a.unit.J * (tm[lane].sn[2] - so[2]));
     }
     __syncwarp();
     // Tasks: NPW nodes per warp, of one visit unless the windows are uniform.
@@ -1411,12 +1439,13 @@ __device__ __forceinline__ void rs_visits(RsMode mode, const StageArgs& a, const
             idle = j >= M;
             if (idle) j = M - 1;
         }
-        const double s = a.invT / c_fermi[hd[k].cls].y[j];
+        const double s = a.unit.T1 / c_fermi[hd[k].cls].y[j];
         RsOut<float> spare;
         RsOut<float>* const to = idle ? &spare : out + k * kFermiOut + j;
-        if constexpr (kPairs) RsNode<Tl>::run_pairs(pt, sites + k * max_sites, (float)s, (float)(a.m.t * s), buf, lane, to);
+        if (lane % Tl::LPN == 0) to->eta = rs_rounding(s);
+        if constexpr (kPairs) RsNode<Tl>::run_pairs(pt, sites + k * max_sites, (float)s, (float)(a.unit.t * s), buf, lane, to);
         else RsNode<Tl>::run(hd[k], sites + k * max_sites, hop + (uniform ? 0 : k * Tl::NS * Tl::NS), (float)s,
-                             (float)(a.m.t * s), buf, lane, to);
+                             (float)(a.unit.t * s), buf, lane, to);
     }
     __syncthreads();
     if constexpr (Tl::NS <= 4) {
@@ -1431,20 +1460,26 @@ __device__ __forceinline__ void rs_visits(RsMode mode, const StageArgs& a, const
             float lq, t0, dl, dt;
             rs_last_pivot(r, tm[k].dv[0] * r.s, tm[k].dv[1] * r.s, tm[k].dv[2] * r.s, tm[k].dv[3] * r.s, lq, t0, dl, dt);
             r.P[0] = lq; r.P[1] = t0; r.P[2] = dl; r.P[3] = dt;
+            r.P[4] = (float)r.th + t0;
         }
         __syncthreads();
         if (warp == 0 && lane < nv) {
             const FermiNodes& f = c_fermi[hd[lane].cls >= 0 ? hd[lane].cls : 0];
             double Lo = 0.0, Th = 0.0, dL = 0.0, dT = 0.0;
+            float th = 0.f, dth = 0.f;
             if (hd[lane].cls >= 0)
                 for (int j = 0; j < f.M; ++j) {
                     const RsOut<float>& r = out[lane * kFermiOut + j];
+                    const RsOut<float>* q = out + lane * kFermiOut + fermi_middle(j, f.M);
+                    const float* w = c_slope.of[hd[lane].cls].w[j];
+                    th += r.eta * (w[0] * q[-1].P[4] + w[1] * q[0].P[4] + w[2] * q[1].P[4]);
+                    dth += r.eta * (w[0] * q[-1].P[3] + w[1] * q[0].P[3] + w[2] * q[1].P[3]);
                     Lo += f.a[j] * (r.lnd + (double)r.P[0]);
                     Th += f.b[j] * (r.th + (double)r.P[1]);
                     dL += f.a[j] * (double)r.P[2];
                     dT += f.b[j] * (double)r.P[3];
                 }
-            rs_final(mode, a, v, hd[lane], tm[lane], f, Lo, Th, dL, dT);
+            rs_final(mode, a, v, hd[lane], tm[lane], f, Lo, Th + (double)th, dL, dT + (double)dth);
         }
     } else {
         for (int k = warp; k < nv; k += nw) rs_decide<float>(mode, a, v, hd[k], tm[k], out + k * kFermiOut, lane);
@@ -1515,7 +1550,7 @@ __device__ __forceinline__ void rs_visit_part(RsMode mode, const StageArgs& a, c
     if (warp == 0) rs_gather<T, 32, false>(a, v.S_in, c, site, h, tm, sites, lane);
     if (extra) {
         if constexpr (kPairs) rs_pairs(a.m, site, pt, lane);
-        else rs_hopping(a.m, site, hop, hs, lane);
+        else rs_hopping(a, site, hop, hs, lane);
     }
     __syncthreads();
     if (extra) {
@@ -1532,10 +1567,11 @@ __device__ __forceinline__ void rs_visit_part(RsMode mode, const StageArgs& a, c
             if (idle) u = mine - 1;
             if (E::kFullWarp && __all_sync(FULL_MASK, idle)) break;
             const int j = part + parts * u;
-            const double s = a.invT / f.y[j];
+            const double s = a.unit.T1 / f.y[j];
             RsOut<T> spare;
-            E::run(h, pt, sites, hop, hs, T(s), T(a.m.t * s), smem + lay.buf + (size_t)unit * E::bytes(max_sites), unit,
-                   idle ? &spare : out + j);
+            RsOut<T>* const to = idle ? &spare : out + j;
+            if (sizeof(T) == 4 && threadIdx.x % E::LANES == 0) to->eta = rs_rounding(s);
+            E::run(h, pt, sites, hop, hs, T(s), T(a.unit.t * s), smem + lay.buf + (size_t)unit * E::bytes(max_sites), unit, to);
         }
     }
     if constexpr (sizeof(T) == 8) {   // the re-solve

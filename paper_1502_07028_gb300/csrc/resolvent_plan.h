@@ -57,19 +57,23 @@ template <typename F> auto with_tile(const Model& m, F f) {
 struct RsStagePlan { int nw, vb; size_t bytes; };
 
 // Visits per CTA: enough that its warps share their nodes evenly (a warp takes
-// NPW nodes at a time).  Small windows: eight warps, 24 or 16 visits; fewer leave
-// turns empty or repeat the CTA's start too often.  Up to 8 sites per layer: two
-// (1099 us per 2500 visits of 8x8 clusters against 1219 with four).  One node per
-// warp and one CTA per SM: the count with the fewest idle warps (3.8 against
-// 5.4 ms for 8000 visits of 4x4x4 clusters, 11 nodes on 8 warps) of those that
-// `room` bytes hold: eight warps' blocks of 13 to 16 sites per layer take 204 KB,
-// each visit of a 16x16 window 5 KB more.
+// NPW nodes at a time).
+// - Small windows: eight warps and 16 visits, or, for chains, the visits that one
+//   turn of the warps takes (24 at 10 nodes); fewer leave turns empty or repeat the
+//   CTA's start too often.
+// - Up to 8 sites per layer: two (1099 us per 2500 visits of 8x8 clusters against
+//   1219 with four).
+// - One node per warp and one CTA per SM: the count with the fewest idle warps (3.8
+//   against 5.4 ms for 8000 visits of 4x4x4 clusters, 11 nodes on 8 warps), the
+//   largest where none idles (12 nodes: a 40^3 sweep takes 38.0 ms with four visits,
+//   39.7 with two), of those that `room` bytes hold: eight warps' blocks of 13 to 16 sites per layer
+//   take 204 KB, each visit of a 16x16 window 5 KB more.
 template <class Tl, bool kPairs>
 RsStagePlan rs_stage_plan(int M, int max_sites, bool uniform, int count, int sms, size_t room) {
     RsStagePlan p{std::min((M + Tl::NPW - 1) / Tl::NPW, Tl::MAXT / 32), 1, 0};
     if (Tl::NS <= 4) {
         p.nw = Tl::MAXT / 32;
-        p.vb = Tl::NS == 1 ? 24 : 16;
+        p.vb = Tl::NS == 1 ? std::min(24, 8 * Tl::NPW / M) : 16;
     } else if (Tl::NS <= 8) {
         p.vb = 2;
     } else if (Tl::NPW == 1 && uniform) {
@@ -77,7 +81,7 @@ RsStagePlan rs_stage_plan(int M, int max_sites, bool uniform, int count, int sms
         for (int v = 1; v <= 5 && (v == 1 || count >= 4 * v * sms); ++v) {
             if (v > 1 && rs_layout<Tl>(v, max_sites, p.nw, uniform, kPairs).total > room) break;
             const double share = (double)v * M / (((v * M + p.nw - 1) / p.nw) * p.nw);
-            if (share > best + 0.01) { best = share; p.vb = v; }
+            if (share >= best + (share < 1.0 ? 0.01 : 0.0)) { best = share; p.vb = v; }
         }
     }
     p.bytes = rs_layout<Tl>(p.vb, max_sites, p.nw, uniform, kPairs).total;
