@@ -1299,9 +1299,19 @@ ptca_status ptca_autotune(ptca_ctx* ctx, int32_t trial_sweeps, ptca_launch_confi
     cudaEventCreate(&e0);
     cudaEventCreate(&e1);
     std::vector<double> ms(cand.size(), -1.0);
+    std::vector<char> det(cand.size(), 0);
     int ibest = -1;
     for (size_t i = 0; i < cand.size(); ++i) {
         if (ptca_set_launch_config(ctx, &cand[i]) != PTCA_OK) continue;
+        // On determinants the width and the grid change nothing: one of a
+        // pipeline's candidates is timed for all.
+        det[i] = on_determinants(ctx);
+        size_t same = 0;
+        while (same < i && !(det[i] && det[same] && cand[same].pipeline == cand[i].pipeline && ms[same] >= 0)) ++same;
+        if (same < i) {
+            ms[i] = ms[same];
+            continue;
+        }
         cudaError_t e = restore();
         if (e == cudaSuccess) e = run_sweeps(ctx, 1, st);  // warm-up (and graph capture)
         if (e == cudaSuccess) e = restore();
