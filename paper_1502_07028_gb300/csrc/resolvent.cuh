@@ -1241,7 +1241,7 @@ __device__ __forceinline__ void rs_decide(RsMode mode, const StageArgs& a, const
     const double* so = v.S_in + 3 * (int64_t)h.site;
     const FermiNodes& f = RsFermi<T>::tab(h.cls >= 0 ? h.cls : 0);
     double Lo = 0.0, Th = 0.0, dL = 0.0, dT = 0.0;
-    float th = 0.f, dth = 0.f, eta = 0.f;   // FP32: phase, its change, rounding of the scale
+    float ln = 0.f, th = 0.f, dln = 0.f, dth = 0.f, eta = 0.f;   // FP32: logarithm, phase, changes, rounding of the scale
     if (h.cls >= 0 && lane < f.M) {
         RsOut<T> r;
         rs_load(r, out + lane);
@@ -1254,22 +1254,28 @@ __device__ __forceinline__ void rs_decide(RsMode mode, const StageArgs& a, const
         dL = f.a[lane] * (double)dl;
         dT = f.b[lane] * (double)dt;
         if constexpr (sizeof(T) == 4) {
+            ln = (float)r.lnd + (float)lq;
             th = (float)r.th + (float)t0;
+            dln = (float)dl;
             dth = (float)dt;
             eta = r.eta;
         }
     }
     if constexpr (sizeof(T) == 4) {
         const int mid = fermi_middle(lane, f.M);
-        const float* w = c_slope.of[h.cls >= 0 ? h.cls : 0].w[lane < f.M ? lane : 0];
-        float d = 0.f, dd = 0.f;
+        const FermiSlope& w = c_slope.of[h.cls >= 0 ? h.cls : 0][lane < f.M ? lane : 0];
+        float cl = 0.f, ct = 0.f, cdl = 0.f, cdt = 0.f;
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
-            d += w[i] * __shfl_sync(FULL_MASK, th, mid + i - 1);
-            dd += w[i] * __shfl_sync(FULL_MASK, dth, mid + i - 1);
+            cl += w.a[i] * __shfl_sync(FULL_MASK, ln, mid + i - 1);
+            ct += w.b[i] * __shfl_sync(FULL_MASK, th, mid + i - 1);
+            cdl += w.a[i] * __shfl_sync(FULL_MASK, dln, mid + i - 1);
+            cdt += w.b[i] * __shfl_sync(FULL_MASK, dth, mid + i - 1);
         }
-        Th += (double)(eta * d);
-        dT += (double)(eta * dd);
+        Lo += (double)(eta * cl);
+        Th += (double)(eta * ct);
+        dL += (double)(eta * cdl);
+        dT += (double)(eta * cdt);
     }
     Lo = warp_sum(Lo);
     Th = warp_sum(Th);
@@ -1460,26 +1466,43 @@ __device__ __forceinline__ void rs_visits(RsMode mode, const StageArgs& a, const
             float lq, t0, dl, dt;
             rs_last_pivot(r, tm[k].dv[0] * r.s, tm[k].dv[1] * r.s, tm[k].dv[2] * r.s, tm[k].dv[3] * r.s, lq, t0, dl, dt);
             r.P[0] = lq; r.P[1] = t0; r.P[2] = dl; r.P[3] = dt;
-            r.P[4] = (float)r.th + t0;
+        }
+        __syncthreads();
+        // corrections for the rounding of the scales (FermiSlope)
+        for (int q = threadIdx.x; q < nv * kFermiOut; q += blockDim.x) {
+            const int k = q / kFermiOut, j = q % kFermiOut, cls = hd[k].cls;
+            if (cls < 0 || j >= c_fermi[cls].M) continue;
+            const RsOut<float>* near = out + k * kFermiOut + fermi_middle(j, c_fermi[cls].M) - 1;
+            const FermiSlope& w = c_slope.of[cls][j];
+            float cl = 0.f, ct = 0.f, cdl = 0.f, cdt = 0.f;
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                cl += w.a[i] * ((float)near[i].lnd + near[i].P[0]);
+                ct += w.b[i] * ((float)near[i].th + near[i].P[1]);
+                cdl += w.a[i] * near[i].P[2];
+                cdt += w.b[i] * near[i].P[3];
+            }
+            RsOut<float>& r = out[q];
+            r.P[4] = r.eta * cl; r.P[5] = r.eta * ct; r.P[6] = r.eta * cdl; r.P[7] = r.eta * cdt;
         }
         __syncthreads();
         if (warp == 0 && lane < nv) {
             const FermiNodes& f = c_fermi[hd[lane].cls >= 0 ? hd[lane].cls : 0];
             double Lo = 0.0, Th = 0.0, dL = 0.0, dT = 0.0;
-            float th = 0.f, dth = 0.f;
+            float cl = 0.f, ct = 0.f, cdl = 0.f, cdt = 0.f;
             if (hd[lane].cls >= 0)
                 for (int j = 0; j < f.M; ++j) {
                     const RsOut<float>& r = out[lane * kFermiOut + j];
-                    const RsOut<float>* q = out + lane * kFermiOut + fermi_middle(j, f.M);
-                    const float* w = c_slope.of[hd[lane].cls].w[j];
-                    th += r.eta * (w[0] * q[-1].P[4] + w[1] * q[0].P[4] + w[2] * q[1].P[4]);
-                    dth += r.eta * (w[0] * q[-1].P[3] + w[1] * q[0].P[3] + w[2] * q[1].P[3]);
                     Lo += f.a[j] * (r.lnd + (double)r.P[0]);
                     Th += f.b[j] * (r.th + (double)r.P[1]);
                     dL += f.a[j] * (double)r.P[2];
                     dT += f.b[j] * (double)r.P[3];
+                    cl += r.P[4];
+                    ct += r.P[5];
+                    cdl += r.P[6];
+                    cdt += r.P[7];
                 }
-            rs_final(mode, a, v, hd[lane], tm[lane], f, Lo, Th + (double)th, dL, dT + (double)dth);
+            rs_final(mode, a, v, hd[lane], tm[lane], f, Lo + (double)cl, Th + (double)ct, dL + (double)cdl, dT + (double)cdt);
         }
     } else {
         for (int k = warp; k < nv; k += nw) rs_decide<float>(mode, a, v, hd[k], tm[k], out + k * kFermiOut, lane);
