@@ -648,17 +648,17 @@ cudaError_t ptca_screen_part(ptca_ctx* ctx, ptca::StageArgs& a, int part, int ro
 
 // Whether the context's sweeps take their free energies from determinants
 // (resolvent.cuh): the default reduction of a PTCA_MIXED context (rows up to the
-// shared-memory orders, shared above) with windows of up to 16 sites per
-// layer and T not below 1/4096 of the spectrum's half width.  The reductions
-// that a launch configuration names explicitly keep their own kernels.
+// shared-memory orders, shared above), also where a launch configuration names
+// it, with windows of up to 16 sites per layer and T not below 1/4096 of the
+// spectrum's half width.  The other reductions, and panels, keep their own kernels.
 static bool on_determinants(const ptca_ctx* ctx) {
     if (ctx->prec != 1 || ctx->panel > 1 || ctx->reduction != (ctx->large ? 2 : 0)) return false;
     return ptca::resolvent_supported(to_model(ctx->p));
 }
 
-// Stages of at most kFewVisits visits run the latency-bound form: a group of
-// threads per node instead of one warp (45 against 110 us for 16 visits of 8x8
-// clusters; 215 against 123 us for 100 of 10x10).
+// Stages of at most kFewVisits visits run the latency-bound form: more lanes per
+// node, and a visit's nodes dealt to several CTAs (45 against 110 us for 16 visits of
+// 8x8 clusters; 215 against 123 us for 100 of 10x10).
 static bool few_visits(const ptca_ctx* ctx) { return ctx->max_stage <= ptca::kFewVisits; }
 
 // A stage launch and a re-solve launch in the context's configuration
@@ -999,8 +999,8 @@ cudaError_t ptca_internal_settle(ptca_ctx* ctx, cudaStream_t st, bool have_strea
 }
 
 // Everything one persistent sweep launch needs, as stream work (capturable).
-// On determinants a stage takes tens of microseconds, spread over the whole GPU by
-// thread-block clusters: there the stages stay separate launches.
+// On determinants a stage takes tens of microseconds: there the stages stay separate
+// launches, each visit's nodes spread over CTAs that meet at a ticket alone.
 static cudaError_t enqueue_persistent(ptca_ctx* ctx, int32_t n_sweeps, cudaStream_t st) {
     if (on_determinants(ctx)) return sweep_stages(ctx, n_sweeps, st, nullptr, true);
     ptca::PersistArgs p;
