@@ -1373,10 +1373,12 @@ static __device__ __noinline__ void rs_exact(const StageArgs& a, const StageVar&
     __syncthreads();
 }
 
-// Relative rounding error of s as a float.
+// Relative rounding error of s > 0 as a float; none where that is zero or below the
+// normal floats (T above 1e36 |t|: levels and phases are then zero as well), where the
+// quotient would be 0 / 0.
 __device__ __forceinline__ float rs_rounding(double s) {
     const float f = (float)s;
-    return __fdividef((float)((double)f - s), f);
+    return f > 1e-37f ? __fdividef((float)((double)f - s), f) : 0.f;
 }
 
 // Visits [first, first + nv) of the work list (nv <= vb <= 32), by the CTA.
