@@ -657,8 +657,9 @@ static bool on_determinants(const ptca_ctx* ctx) {
 }
 
 // Stages of at most kFewVisits visits run the latency-bound form: more lanes per
-// node, and a visit's nodes dealt to several CTAs (45 against 110 us for 16 visits of
-// 8x8 clusters; 215 against 123 us for 100 of 10x10).
+// node, and a visit's nodes dealt to several CTAs (at 15 nodes: 45 against 110 us for 16
+// visits of 8x8 clusters; 215 against 123 us for 100 of 10x10; 47 us for the 16 at today's
+// 16 nodes).
 static bool few_visits(const ptca_ctx* ctx) { return ctx->max_stage <= ptca::kFewVisits; }
 
 // A stage launch and a re-solve launch in the context's configuration

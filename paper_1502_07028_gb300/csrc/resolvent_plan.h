@@ -61,8 +61,8 @@ struct RsStagePlan { int nw, vb; size_t bytes; };
 // - Small windows: eight warps and 16 visits, or, for chains, the visits that one
 //   turn of the warps takes (24 at 10 nodes); fewer leave turns empty or repeat the
 //   CTA's start too often.
-// - Up to 8 sites per layer: two (1099 us per 2500 visits of 8x8 clusters against
-//   1219 with four).
+// - Up to 8 sites per layer: two (1099 us per 2500 visits of 8x8 clusters at 13
+//   nodes against 1219 with four; 1160 us at today's 14).
 // - One node per warp and one CTA per SM: the count with the fewest idle warps (3.8
 //   against 5.4 ms for 8000 visits of 4x4x4 clusters, 11 nodes on 8 warps), the
 //   largest where none idles (12 nodes: a 40^3 sweep takes 38.0 ms with four visits,
