@@ -68,6 +68,12 @@ struct RsStagePlan { int nw, vb; size_t bytes; };
 //   largest where none idles (12 nodes: a 40^3 sweep takes 38.0 ms with four visits,
 //   39.7 with two), of those that `room` bytes hold: eight warps' blocks of 13 to 16 sites per layer
 //   take 204 KB, each visit of a 16x16 window 5 KB more.
+// - Two nodes per warp and one CTA per SM (9 to 12 sites per layer, seven warps): a
+//   visit of 15 nodes leaves one of its eight warp loads to a second turn, where it
+//   takes a quarter of a full turn; two visits together leave one of fifteen.  12x12
+//   clusters, 576 visits: 1576 -> 1267 us; 2500 visits: 6.54 -> 5.58 ms (14 nodes and
+//   one visit: 1261 us and 5.32 ms; two visits 1255 us and 5.53 ms).  Not at 16 nodes,
+//   where both leave one per visit (6.54 and 6.88 ms).
 template <class Tl, bool kPairs>
 RsStagePlan rs_stage_plan(int M, int max_sites, bool uniform, int count, int sms, size_t room) {
     RsStagePlan p{std::min((M + Tl::NPW - 1) / Tl::NPW, Tl::MAXT / 32), 1, 0};
@@ -83,6 +89,13 @@ RsStagePlan rs_stage_plan(int M, int max_sites, bool uniform, int count, int sms
             const double share = (double)v * M / (((v * M + p.nw - 1) / p.nw) * p.nw);
             if (share >= best + (share < 1.0 ? 0.01 : 0.0)) { best = share; p.vb = v; }
         }
+    } else if (uniform) {
+        // turns of the SM's CTAs one after another, four loads of a part-filled turn as a full one
+        auto turns = [&](int v) {
+            const int loads = (v * M + Tl::NPW - 1) / Tl::NPW, ctas = (count + v - 1) / v;
+            return (ctas + sms - 1) / sms * (loads / p.nw + std::min(1.0, 0.25 * (loads % p.nw)));
+        };
+        if (turns(2) < turns(1) && rs_layout<Tl>(2, max_sites, p.nw, uniform, kPairs).total <= room) p.vb = 2;
     }
     p.bytes = rs_layout<Tl>(p.vb, max_sites, p.nw, uniform, kPairs).total;
     return p;

@@ -46,3 +46,11 @@ def test_cubes_of_parity_split_windows(L, margin):
         assert eF <= 1e-9 * Fmax and edF <= 1e-9 * 14, (eF, edF, Fmax)
     else:
         assert eF <= 1e-6 * Fmax + 2e-7 * 2 * 18 and edF <= 2e-6 * 14, (eF, edF, Fmax)
+
+
+@pytest.mark.parametrize("Lx,Ly,L_c,T", [(57, 61, 9, 0.04), (60, 60, 11, 0.0375), (59, 59, 10, 0.013), (60, 60, 12, 0.007)])
+def test_two_visits_of_two_node_warps_in_a_cta(Lx, Ly, L_c, T):
+    # 899 or 900 visits a stage of 15, 17 or 19 nodes, on seven warps of two nodes
+    cfg = P.Config(Lx=Lx, Ly=Ly, L_c=L_c, J_H=8.0, mu=-6.5, T=T, seed=L_c, precision=P.MIXED, **BLOCK)
+    eF, edF, Fmax, _, _ = _stage0(cfg, None, 0.0, sample=2)
+    assert eF <= 1e-6 * Fmax + 2e-7 * 2 * 20.5 and edF <= 2e-6 * 14, (eF, edF, Fmax)
